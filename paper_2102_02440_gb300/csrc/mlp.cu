@@ -189,105 +189,231 @@ __global__ void k_mlp_infer(const float* __restrict__ P, int32_t nin, int32_t nh
 }
 
 // ---------------------------------------------------------------- training
-// Phase 1 (thread = sample): forward pass, d(loss)/dy = 2 (y - t) / n, activations and
-// hidden gradients in shared memory.  Phase 2 (thread = parameter): this CTA's gradient
-// contribution summed over its samples in a fixed order -> partial[cta][k].
+// One CTA per chunk of kTrainSamples samples (persistent beyond kTrainMaxCtas).  Phase 1
+// (thread = sample): forward pass in blocks of kHidBlock hidden units, d(loss)/dy and the
+// activations to shared memory.  Phase 2 (thread = hidden unit x every G-th input): the
+// chunk's gradient, summed over its samples in a fixed order -> partial[cta][k].
+// Bound: shared-memory wavefronts.  Both x and act are kept [feature][sample] with rows of
+// kTrainStride = 132 floats: phase 1's lanes (samples) touch consecutive words, and phase
+// 2's 16-byte loads of eight hidden units fall on eight different bank groups; the weights,
+// x and dy are read as 16-byte broadcasts.  The hidden gradient dy W2[h] [act > 0] is formed
+// from act instead of being stored.  Rows of 64 floats per sample made every access of both
+// phases a 32-way conflict: a step on 80,000 samples of 13 -> 64 -> 1 took 189 us (143 of them
+// here, 40 in k_mlp_adam) and takes 31 us.
+constexpr int kTrainStride = kTrainSamples + 4;  // floats: 16-byte aligned rows, 4 banks apart
+constexpr int kHidBlock = 16;
+constexpr int kColBlock = 8;                     // gradient columns per thread and pass over the samples
+constexpr int kTrainMaxCtas = 4096;
+
+struct TrainSmem {  // offsets in floats
+  int w1, b1, w2, xs, act, dys, total;
+};
+__host__ __device__ inline TrainSmem train_smem(int nin, int nh) {
+  const int nhp = (nh + kHidBlock - 1) / kHidBlock * kHidBlock;
+  TrainSmem L;
+  L.w1 = 0;                            // [nin][nhp], zero beyond nh
+  L.b1 = L.w1 + nin * nhp;             // [nhp]
+  L.w2 = L.b1 + nhp;                   // [nhp], then b2
+  L.xs = L.w2 + nhp + 4;               // [nin][kTrainStride]
+  L.act = L.xs + nin * kTrainStride;   // [nhp][kTrainStride]
+  L.dys = L.act + nhp * kTrainStride;  // dy[kTrainSamples], loss terms[kTrainSamples]
+  L.total = L.dys + 2 * kTrainSamples;
+  return L;
+}
+
 __global__ void __launch_bounds__(kTrainSamples) k_mlp_grad(const float* __restrict__ P, int32_t nin, int32_t nh,
                                                            int32_t skip, const float* __restrict__ x,
                                                            const float* __restrict__ t,
-                                                           int64_t n, float huber_delta, float* __restrict__ partial,
+                                                           int64_t n, float huber_delta, int64_t chunks,
+                                                           float* __restrict__ partial,
                                                            float* __restrict__ partial_loss) {
-  // dynamic shared memory: W[np] | xs[S][nin] | act[S][nh] | dz[S][nh] | dys[S] | err2[S]
-  extern __shared__ float shm[];
+  extern __shared__ __align__(16) float shm[];
+  const TrainSmem L = train_smem(nin, nh);
   const int np = nh * nin + 2 * nh + 1;
-  float* W = shm;
-  float* xsb = W + np;
-  float* actb = xsb + kTrainSamples * nin;
-  float* dzb = actb + kTrainSamples * nh;
-  float* dys = dzb + kTrainSamples * nh;
-  float* err2 = dys + kTrainSamples;
-  auto xs = [&](int s, int c) -> float& { return xsb[s * nin + c]; };
-  auto act = [&](int s, int h) -> float& { return actb[s * nh + h]; };
-  auto dz = [&](int s, int h) -> float& { return dzb[s * nh + h]; };
-  for (int k = threadIdx.x; k < np; k += blockDim.x) W[k] = bf16r(P[k]);
-  __syncthreads();
-  const float* W1 = W;
-  const float* b1 = W1 + nh * nin;
-  const float* W2 = b1 + nh;
-  const float b2 = W2[nh];
-  const int64_t s0 = int64_t(blockIdx.x) * kTrainSamples;
-  const int ns = int(min(int64_t(kTrainSamples), n - s0));
-  const int si = threadIdx.x;
-  if (si < ns) {
-    const int64_t s = s0 + si;
-    for (int c = 0; c < nin; c++) xs(si, c) = x[s * nin + c];
-    float acc = b2 + (skip >= 0 ? fmaxf(xs(si, skip), 0.f) : 0.f);
-    for (int h = 0; h < nh; h++) {
-      float z = b1[h];
-      for (int c = 0; c < nin; c++) z = fmaf(W1[h * nin + c], xs(si, c), z);
-      act(si, h) = z > 0.f ? z : 0.f;
-      if (z > 0.f) acc = fmaf(W2[h], z, acc);
-    }
-    const float e = acc - t[s];
-    float dy;
-    if (huber_delta > 0.f) {  // Huber: quadratic within delta, linear beyond
-      const float a = fabsf(e);
-      dy = (a <= huber_delta ? e : copysignf(huber_delta, e)) / float(n);
-      err2[si] = a <= huber_delta ? 0.5f * e * e : huber_delta * (a - 0.5f * huber_delta);
-    } else {
-      dy = 2.f * e / float(n);
-      err2[si] = e * e;
-    }
-    dys[si] = dy;
-    for (int h = 0; h < nh; h++) dz(si, h) = act(si, h) > 0.f ? dy * W2[h] : 0.f;
+  const int nhp = (nh + kHidBlock - 1) / kHidBlock * kHidBlock;
+  float *W1 = shm + L.w1, *B1 = shm + L.b1, *W2 = shm + L.w2, *xs = shm + L.xs, *act = shm + L.act,
+        *dys = shm + L.dys, *err = dys + kTrainSamples;
+  const int tid = threadIdx.x;
+  for (int k = tid; k < nin * nhp; k += kTrainSamples) {
+    const int c = k / nhp, h = k % nhp;
+    W1[k] = h < nh ? bf16r(P[h * nin + c]) : 0.f;
   }
-  __syncthreads();
-  float* out = partial + int64_t(blockIdx.x) * np;
-  for (int k = threadIdx.x; k < np; k += blockDim.x) {
-    float g = 0.f;
-    if (k < nh * nin) {
-      const int h = k / nin, c = k % nin;
-      for (int s = 0; s < ns; s++) g = fmaf(dz(s, h), xs(s, c), g);
-    } else if (k < nh * nin + nh) {
-      const int h = k - nh * nin;
-      for (int s = 0; s < ns; s++) g += dz(s, h);
-    } else if (k < nh * nin + 2 * nh) {
-      const int h = k - nh * nin - nh;
-      for (int s = 0; s < ns; s++) g = fmaf(dys[s], act(s, h), g);
-    } else {
-      for (int s = 0; s < ns; s++) g += dys[s];
-    }
-    out[k] = g;
+  for (int h = tid; h < nhp; h += kTrainSamples) {
+    B1[h] = h < nh ? bf16r(P[nh * nin + h]) : 0.f;
+    W2[h] = h < nh ? bf16r(P[nh * nin + nh + h]) : 0.f;
   }
-  if (threadIdx.x == 0) {
-    float l = 0.f;
-    for (int s = 0; s < ns; s++) l += err2[s];
-    partial_loss[blockIdx.x] = l;
+  const float b2 = bf16r(P[np - 1]);
+  // phase 2's share of this thread: hidden unit h, inputs g, g + G, ...
+  int hp2 = 1;
+  while (hp2 < nh) hp2 <<= 1;  // <= 64
+  const int G = kTrainSamples / hp2, h = tid & (hp2 - 1), g = tid / hp2;
+  for (int64_t chunk = blockIdx.x; chunk < chunks; chunk += gridDim.x) {
+    const int64_t s0 = chunk * kTrainSamples;
+    const int ns = int(min(int64_t(kTrainSamples), n - s0));
+    for (int i = tid; i < kTrainSamples * nin; i += kTrainSamples) {  // coalesced; samples beyond n are 0
+      const int si = i / nin, c = i - si * nin;
+      xs[c * kTrainStride + si] = si < ns ? __ldg(x + s0 * nin + i) : 0.f;
+    }
+    __syncthreads();
+    {
+      float acc = b2 + (skip >= 0 ? fmaxf(xs[skip * kTrainStride + tid], 0.f) : 0.f);
+      for (int h0 = 0; h0 < nhp; h0 += kHidBlock) {
+        float z[kHidBlock];
+#pragma unroll
+        for (int j = 0; j < kHidBlock; j += 4) {
+          const float4 b = *reinterpret_cast<const float4*>(B1 + h0 + j);
+          z[j] = b.x, z[j + 1] = b.y, z[j + 2] = b.z, z[j + 3] = b.w;
+        }
+        for (int c = 0; c < nin; c++) {
+          const float xv = xs[c * kTrainStride + tid];
+          const float4* wr = reinterpret_cast<const float4*>(W1 + c * nhp + h0);
+#pragma unroll
+          for (int j = 0; j < kHidBlock; j += 4) {
+            const float4 wv = wr[j / 4];
+            z[j] = fmaf(wv.x, xv, z[j]);
+            z[j + 1] = fmaf(wv.y, xv, z[j + 1]);
+            z[j + 2] = fmaf(wv.z, xv, z[j + 2]);
+            z[j + 3] = fmaf(wv.w, xv, z[j + 3]);
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < kHidBlock; j++) {
+          const bool on = z[j] > 0.f && tid < ns;
+          act[(h0 + j) * kTrainStride + tid] = on ? z[j] : 0.f;
+          if (on) acc = fmaf(W2[h0 + j], z[j], acc);
+        }
+      }
+      float dy = 0.f, l = 0.f;
+      if (tid < ns) {
+        const float e = acc - __ldg(t + s0 + tid);
+        if (huber_delta > 0.f) {  // Huber: quadratic within delta, linear beyond
+          const float a = fabsf(e);
+          dy = (a <= huber_delta ? e : copysignf(huber_delta, e)) / float(n);
+          l = a <= huber_delta ? 0.5f * e * e : huber_delta * (a - 0.5f * huber_delta);
+        } else {
+          dy = 2.f * e / float(n);
+          l = e * e;
+        }
+      }
+      dys[tid] = dy;
+      err[tid] = l;
+    }
+    __syncthreads();
+    float* out = partial + int64_t(blockIdx.x) * np;
+    const bool first = chunk == blockIdx.x;  // a later chunk of this CTA adds to its partial
+    auto put = [&](int k, float v) { out[k] = first ? v : out[k] + v; };
+    if (h < nh) {
+      const float4* ar = reinterpret_cast<const float4*>(act + h * kTrainStride);
+      const float4* dr = reinterpret_cast<const float4*>(dys);
+      const float w2 = W2[h];
+      for (int c0 = g; c0 < nin; c0 += G * kColBlock) {
+        float acc[kColBlock];
+#pragma unroll
+        for (int q = 0; q < kColBlock; q++) acc[q] = 0.f;
+#pragma unroll 2
+        for (int s4 = 0; s4 < kTrainSamples / 4; s4++) {
+          const float4 a = ar[s4], dy = dr[s4];
+          const float d0 = a.x > 0.f ? dy.x * w2 : 0.f, d1 = a.y > 0.f ? dy.y * w2 : 0.f,
+                      d2 = a.z > 0.f ? dy.z * w2 : 0.f, d3 = a.w > 0.f ? dy.w * w2 : 0.f;
+#pragma unroll
+          for (int q = 0; q < kColBlock; q++) {
+            if (c0 + q * G < nin) {  // uniform over the threads of a group
+              const float4 v = *reinterpret_cast<const float4*>(xs + (c0 + q * G) * kTrainStride + 4 * s4);
+              acc[q] = fmaf(d0, v.x, acc[q]);
+              acc[q] = fmaf(d1, v.y, acc[q]);
+              acc[q] = fmaf(d2, v.z, acc[q]);
+              acc[q] = fmaf(d3, v.w, acc[q]);
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kColBlock; q++)
+          if (c0 + q * G < nin) put(h * nin + c0 + q * G, acc[q]);
+      }
+      if (g == 0 || g == G - 1) {  // b1 and W2 (one thread of each hidden unit for either)
+        float gb = 0.f, gw = 0.f;
+        for (int s4 = 0; s4 < kTrainSamples / 4; s4++) {
+          const float4 a = ar[s4], dy = dr[s4];
+          gb += a.x > 0.f ? dy.x * w2 : 0.f;
+          gb += a.y > 0.f ? dy.y * w2 : 0.f;
+          gb += a.z > 0.f ? dy.z * w2 : 0.f;
+          gb += a.w > 0.f ? dy.w * w2 : 0.f;
+          gw = fmaf(dy.x, a.x, gw);
+          gw = fmaf(dy.y, a.y, gw);
+          gw = fmaf(dy.z, a.z, gw);
+          gw = fmaf(dy.w, a.w, gw);
+        }
+        if (g == 0) put(nh * nin + h, gb);
+        if (g == G - 1) put(nh * nin + nh + h, gw);
+      }
+    }
+    if (tid >= kTrainSamples - 32) {  // b2 and the loss: the last warp, a fixed tree
+      const int lane = tid & 31;
+      float sd = (dys[lane] + dys[lane + 32]) + (dys[lane + 64] + dys[lane + 96]);
+      float sl = (err[lane] + err[lane + 32]) + (err[lane + 64] + err[lane + 96]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sd += __shfl_xor_sync(0xffffffffu, sd, o);
+        sl += __shfl_xor_sync(0xffffffffu, sl, o);
+      }
+      if (lane == 0) {
+        put(np - 1, sd);
+        partial_loss[blockIdx.x] = first ? sl : partial_loss[blockIdx.x] + sl;
+      }
+    }
+    __syncthreads();  // xs, act and dys are rewritten by the next chunk
   }
 }
 
 // Sum of the CTA partials in a fixed order, then one Adam step (Kingma & Ba 2015) on the
-// fp32 master parameters.
-__global__ void k_mlp_adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v, int32_t np,
-                           const float* __restrict__ partial, const float* __restrict__ partial_loss, int32_t n_cta,
-                           int64_t n, float lr, int32_t step, float* __restrict__ loss, float* __restrict__ grad) {
+// fp32 master parameters.  A CTA takes 32 parameters: warp y sums partials y, y + 32, ...
+// (128-byte rows), then the 32 sums of a parameter meet in a fixed tree.  (One thread per
+// parameter walking all 625 partials of 80,000 samples, on four CTAs, took 40 us.)  Column
+// np is the loss, summed by the CTA after the last parameter block.
+__global__ void __launch_bounds__(1024) k_mlp_adam(float* __restrict__ P, float* __restrict__ m, float* __restrict__ v,
+                                                   int32_t np, const float* __restrict__ partial,
+                                                   const float* __restrict__ partial_loss, int32_t n_cta,
+                                                   int64_t n, float lr, int32_t step, float* __restrict__ loss,
+                                                   float* __restrict__ grad) {
+  __shared__ float part[32][33];
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const bool is_loss = int(blockIdx.x) == int(gridDim.x) - 1;
+  if (is_loss) {
+    float l = 0.f;
+    for (int c = int(threadIdx.x); c < n_cta; c += 1024) l += partial_loss[c];
+    part[lane][y] = l;
+  } else {
+    const int k = int(blockIdx.x) * 32 + lane;
+    float g = 0.f;
+    if (k < np)
+      for (int c = y; c < n_cta; c += 32) g += partial[int64_t(c) * np + k];
+    part[lane][y] = g;
+  }
+  __syncthreads();
+  float s = part[y][lane];  // warp y now holds parameter y of the block (loss: a 32nd of the terms)
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (is_loss) {
+    __syncthreads();
+    if (lane == 0) part[0][y] = s;
+    __syncthreads();
+    if (y != 0) return;
+    s = part[0][lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0 && loss) *loss = s / float(n);
+    return;
+  }
+  const int k = int(blockIdx.x) * 32 + y;
+  if (lane != 0 || k >= np) return;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = 1.f - powf(b1, float(step)), c2 = 1.f - powf(b2, float(step));
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < np; k += gridDim.x * blockDim.x) {
-    float g = 0.f;
-    for (int c = 0; c < n_cta; c++) g += partial[int64_t(c) * np + k];
-    if (grad) grad[k] = g;
-    const float mk = b1 * m[k] + (1.f - b1) * g;
-    const float vk = b2 * v[k] + (1.f - b2) * g * g;
-    m[k] = mk;
-    v[k] = vk;
-    P[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0 && loss) {
-    float l = 0.f;
-    for (int c = 0; c < n_cta; c++) l += partial_loss[c];
-    *loss = l / float(n);
-  }
+  if (grad) grad[k] = s;
+  const float mk = b1 * m[k] + (1.f - b1) * s;
+  const float vk = b2 * v[k] + (1.f - b2) * s * s;
+  m[k] = mk;
+  v[k] = vk;
+  P[k] -= lr * (mk / c1) / (sqrtf(vk / c2) + eps);
 }
 
 // Combined estimate: the plain median where it is a usable join size (>= 1 tuple), the
@@ -354,19 +480,20 @@ cudaError_t launch_mlp_train(float* P, float* m, float* v, int32_t nin, int32_t 
                              const float* t, int64_t n, float huber_delta, float lr, int32_t step, float* loss,
                              float* grad, float* partial,
                              float* partial_loss, cudaStream_t st) {
-  const int64_t ctas = mlp_train_ctas(n);
+  const int64_t chunks = mlp_train_ctas(n);
+  const int64_t ctas = chunks < kTrainMaxCtas ? chunks : kTrainMaxCtas;
   const int32_t np = nh * nin + 2 * nh + 1;
   if (ctas > 0) {
-    const size_t smem = sizeof(float) * size_t(np + kTrainSamples * (nin + 2 * nh + 2));
+    const size_t smem = sizeof(float) * size_t(train_smem(nin, nh).total);
     cudaError_t e0 = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e0 != cudaSuccess) return e0;
-    k_mlp_grad<<<unsigned(ctas), kTrainSamples, smem, st>>>(P, nin, nh, skip, x, t, n, huber_delta, partial,
+    k_mlp_grad<<<unsigned(ctas), kTrainSamples, smem, st>>>(P, nin, nh, skip, x, t, n, huber_delta, chunks, partial,
                                                             partial_loss);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
-  k_mlp_adam<<<unsigned((np + 255) / 256), 256, 0, st>>>(P, m, v, np, partial, partial_loss, int32_t(ctas), n, lr,
-                                                         step, loss, grad);
+  k_mlp_adam<<<unsigned((np + 31) / 32 + 1), 1024, 0, st>>>(P, m, v, np, partial, partial_loss, int32_t(ctas), n, lr,
+                                                            step, loss, grad);
   return cudaGetLastError();
 }
 
