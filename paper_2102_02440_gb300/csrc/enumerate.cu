@@ -10,13 +10,37 @@
 // (beyond the exact range) counts as +inf, a negative one as 0.  Pruning and the update of
 // the best plan are strict, so of equal-cost plans the first found is kept.
 //
-// One warp per graph, its first lane searching: the search is sequential (each source's
-// search starts from the best cost found so far), and graphs in separate warps do not
-// serialise each other's divergent paths.  The stack, one frame per prefix length, lives in
-// the workspace; the estimates come from the device array the estimate wrote (no host round
-// trip), found through the graph's open-addressing table of sub-plan masks.  f(v) and the
-// costs are computed with explicitly rounded double operations (no fused multiply-add), so
-// every comparison sees the same values as a plain IEEE evaluation.
+// One CTA per graph.  The search is sequential by definition: every completed plan may lower
+// the best cost, which decides what is pruned from then on, and the counters count what the
+// sequential search visits.  But between two completed plans the best cost does not change,
+// and the subtrees still to be searched are independent.  So the first warp searches, and
+// when it has extended kEnumSeqNodes prefixes without completing a plan, the CTA runs a
+// round: the unvisited prefixes, in search order, are split (the shallowest first) into up to
+// kEnumItems pieces, the warps search the pieces side by side under the current best cost,
+// and the results are taken in search order up to and including the first piece that
+// completed a plan (all of it: its warp lowered the best cost for itself).  What came after
+// that piece is discarded and searched again under the new best cost.  The counters, the
+// costs and the plan are those of the sequential search; a round that would exceed the
+// search budget is discarded and the sequential search goes on alone.
+//
+// Everything a prefix extension touches is kept close, for its latency is what a search
+// costs:
+//  - the search frames (one per prefix length and warp) live in shared memory;
+//  - the graph's open-addressing table of (sub-plan mask, estimate) is staged in shared
+//    memory when it has at most kEnumStageSlots slots (64 KB), else read through the
+//    read-only cache (mask slot, then the estimate the slot points to);
+//  - a prefix's candidates are looked up side by side, lane v taking table v (and v + 32),
+//    and sorted by (estimate, id) by counting each one's predecessors;
+//  - estimates and costs are never negative, so they are ordered as their bit patterns, in
+//    integers (double comparisons run at 1/64 of their rate here); the one double addition
+//    per candidate, its cost, is made for all candidates of a prefix side by side;
+//  - candidates are in ascending estimate order and cost + estimate is monotone under
+//    rounding, so the first pruned candidate prunes the rest of its frame at once.
+// Ten chains and cycles of 4 to 17 tables (993 sub-plans, 100,000 extensions): 46.2 ms with one
+// lane per graph and its frames in global memory, 33.7 ms with the above on one warp, 4.6 ms
+// with the rounds.
+// f(v) and the costs are computed with explicitly rounded double operations (no fused
+// multiply-add), so every comparison sees the same values as a plain IEEE evaluation.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -44,12 +68,9 @@ struct EnumSlot {
   uint64_t mask;
   int64_t sub;
 };
-__host__ __device__ inline uint64_t enum_hash(uint64_t m) {
-  m ^= m >> 31;
-  m *= 0x7fb5d329728ea185ull;
-  m ^= m >> 27;
-  m *= 0x81dadef4bc2dd44dull;
-  return m ^ (m >> 33);
+// (the high bits of the product are hashed: shift by 64 - log2 of the table's slots)
+__host__ __device__ inline uint64_t enum_hash(uint64_t m, int log2_size) {
+  return ((m ^ (m >> 29)) * 0x9E3779B97F4A7C15ull) >> (64 - log2_size);
 }
 
 struct EnumPlanHdr {
@@ -57,20 +78,76 @@ struct EnumPlanHdr {
   int32_t version, n_graphs;
   int64_t n_sub, n_slots;
   int64_t off_graphs, off_slots, total_bytes, ws_bytes;
+  int32_t n_max, stage_slots;  // most tables of a graph; slots of the largest staged table
 };
+constexpr int32_t kEnumPlanVersion = 3;
 constexpr uint64_t kEnumPlanMagic = 0x434d50454e554d31ull;  // "CMPENUM1"
 
-// One search frame per prefix length: the prefix, its cost, its candidates sorted by
-// (estimate, id) with their estimates, the next candidate, the neighbours of the prefix.
-struct EnumFrames {
-  uint64_t mask[kEnumMaxN];
-  uint64_t nb[kEnumMaxN];
-  double cost[kEnumMaxN];
-  int32_t n_cand[kEnumMaxN], next[kEnumMaxN], path[kEnumMaxN];
-  uint8_t cand[kEnumMaxN][kEnumMaxN];
-  double e[kEnumMaxN][kEnumMaxN];
+constexpr int kEnumMaxWarps = 16;
+constexpr int kEnumStageSlots = 4096;    // 64 KB
+constexpr int kEnumItems = 256;          // pieces of a round
+constexpr int kEnumTasksWanted = 96;     // pieces to search that a round stops splitting at
+constexpr int64_t kEnumSeqNodes = 192;   // prefixes extended alone before a round
+
+// Shared memory of one warp's search over n tables: per prefix length its candidates sorted
+// by (estimate, id) with the costs of the prefixes they extend to, the prefix, its
+// neighbours, its cost, the next candidate; the best plan.
+struct EnumFrame {
+  int e, cost, mask, nb, n_cand, next, path, best, cand, bytes;
 };
-constexpr size_t kEnumFrameBytes = (sizeof(EnumFrames) + 255) & ~size_t(255);
+__host__ __device__ inline EnumFrame enum_frame(int n) {
+  EnumFrame L;
+  int o = 0;
+  L.e = o;      o += 8 * n * n;
+  L.cost = o;   o += 8 * n;
+  L.mask = o;   o += 8 * n;
+  L.nb = o;     o += 8 * n;
+  L.n_cand = o; o += 4 * n;
+  L.next = o;   o += 4 * n;
+  L.path = o;   o += 4 * n;
+  L.best = o;   o += 4 * n;
+  L.cand = o;   o += n * n;
+  L.bytes = (o + 15) & ~15;
+  return L;
+}
+// One piece of a round: nothing (kNone), an unsearched prefix (kTask, itself one extension),
+// `count` pruned extensions (kPruned) or a complete plan (kPlan).  pre: extensions visited
+// right before it (prefixes split into pieces); missing: one of them lacked an estimate.
+enum { kNone = 0, kTask = 1, kPruned = 2, kPlan = 3 };
+struct EnumPiece {
+  uint64_t mask, cost;
+  int32_t pre, count;
+  uint8_t kind, len, missing, pad[5];  // len: tables of the prefix
+};
+struct EnumResult {  // of a searched piece: extensions (itself included), pruned ones, plans, best cost
+  int64_t nodes, pruned;
+  uint64_t cost;
+  int32_t plans;
+  uint8_t warp, missing, over, improved;
+};
+// The block's shared memory: warp frames, two lists of pieces with their paths (n bytes each),
+// results, the source order, the staged table.
+struct EnumSmem {
+  int frame, piece[2], path[2], result, src, table;
+};
+__host__ __device__ inline EnumSmem enum_smem(int n, int warps) {
+  EnumSmem L;
+  int o = 0;
+  L.frame = o;  o += enum_frame(n).bytes * warps;
+  for (int k = 0; k < 2; k++) {
+    L.piece[k] = o;
+    o += int(sizeof(EnumPiece)) * kEnumItems;
+    L.path[k] = o;
+    o += (n * kEnumItems + 15) & ~15;
+  }
+  L.result = o; o += int(sizeof(EnumResult)) * kEnumItems;
+  L.src = o;    o += 4 * n;
+  L.table = (o + 15) & ~15;
+  return L;
+}
+// workspace of a plan: the search needs none beyond shared memory; the entry point still
+// takes a buffer of this size
+constexpr size_t kEnumWsBytes = 16;
 
 struct EnumArgs {
   const EnumGraph* graphs;
@@ -79,152 +156,624 @@ struct EnumArgs {
   int32_t n_graphs;
   double alpha, beta;
   int64_t max_plans, max_nodes;
-  unsigned char* ws;
+  int32_t n_max, stage_slots, warps;  // most tables of a graph; slots of the shared-memory table; warps per CTA
   int32_t* order;
   double* cost;
   int64_t* stats;
   int32_t* status;
 };
 
-__device__ double lookup(const EnumArgs& A, const EnumGraph& g, uint64_t m, bool* missing) {
-  const uint64_t size = uint64_t(1) << g.h_log2;
-  uint64_t i = enum_hash(m) & (size - 1);
-  int64_t sub = -1;
-  for (uint64_t probe = 0; probe < size; probe++) {  // the table has empty slots: ends early
-    const EnumSlot sl = A.slots[g.h_begin + int64_t(i)];
-    if (sl.mask == m) {
-      sub = sl.sub;
-      break;
-    }
-    if (sl.mask == 0) break;
-    i = (i + 1) & (size - 1);
-  }
-  if (sub < 0) {
-    *missing = true;
-    return INFINITY;
-  }
-  const double v = A.est[sub];
-  if (v != v) return INFINITY;  // NaN: beyond the exact range
-  return v < 0.0 ? 0.0 : v;
+// The bits of an estimate as the search takes it: NaN (beyond the exact range) as +inf, a
+// negative one (or -0) as 0.  Bits of non-negative doubles order as the values.
+constexpr uint64_t kInfBits = 0x7ff0000000000000ull;
+__device__ __forceinline__ uint64_t est_bits(double v) {
+  const uint64_t b = uint64_t(__double_as_longlong(v));
+  if ((b & ~(1ull << 63)) > kInfBits) return kInfBits;  // NaN
+  return (b >> 63) ? 0ull : b;
+}
+__device__ __forceinline__ double bits_double(uint64_t b) { return __longlong_as_double((long long)b); }
+
+// A slot's fields through the read-only cache.
+__device__ __forceinline__ uint64_t load_mask(const EnumSlot* s) {
+  return __ldg(reinterpret_cast<const unsigned long long*>(&s->mask));
+}
+__device__ __forceinline__ int64_t load_sub(const EnumSlot* s) {
+  return __ldg(reinterpret_cast<const long long*>(&s->sub));
 }
 
-// Candidates of frame d: neighbours of the prefix not in it, sorted by (estimate, id).
-__device__ void expand(const EnumArgs& A, const EnumGraph& g, EnumFrames& F, int d, bool* missing) {
-  const uint64_t m = F.mask[d];
-  uint64_t c = F.nb[d] & ~m;
-  int k = 0;
-  while (c) {
-    const int v = __ffsll(static_cast<long long>(c)) - 1;
-    c &= c - 1;
-    const double e = lookup(A, g, m | (1ull << v), missing);
-    int j = k;  // ids ascend, so inserting after equal estimates keeps id order
-    while (j > 0 && F.e[d][j - 1] > e) {
-      F.e[d][j] = F.e[d][j - 1];
-      F.cand[d][j] = F.cand[d][j - 1];
-      j--;
+// The estimate of sub-plan m in the staged table (tmask, tval) or the plan's slots.
+__device__ __forceinline__ uint64_t lookup(const EnumArgs& A, const EnumGraph& g, const uint64_t* tmask,
+                                           const uint64_t* tval, bool staged, uint64_t m, bool* missing) {
+  const uint64_t size = uint64_t(1) << g.h_log2;
+  uint64_t i = enum_hash(m, g.h_log2);
+  for (uint64_t probe = 0; probe < size; probe++) {  // the table has empty slots: ends early
+    if (staged) {
+      const uint64_t k = tmask[i];
+      if (k == m) return tval[i];
+      if (k == 0) break;
+    } else {
+      const EnumSlot* sl = A.slots + g.h_begin + int64_t(i);
+      const uint64_t k = load_mask(sl);
+      const int64_t sub = load_sub(sl);
+      if (k == m) return est_bits(__ldg(A.est + sub));
+      if (k == 0) break;
     }
-    F.e[d][j] = e;
-    F.cand[d][j] = uint8_t(v);
-    k++;
+    i = (i + 1) & (size - 1);
   }
-  F.n_cand[d] = k;
-  F.next[d] = 0;
+  *missing = true;
+  return kInfBits;
 }
+
+// A warp's search: its frames in shared memory, the current frame in registers (warp-uniform).
+struct EnumWarp {
+  const EnumArgs& A;
+  const EnumGraph& g;
+  const uint64_t *tmask, *tval;
+  bool staged;
+  int n, lane;
+  uint64_t full;
+  uint64_t *fe, *fcost, *fmask, *fnb;
+  int32_t *fn, *fnext, *path, *best;
+  uint8_t* fcand;
+  int d, nx, nc;
+  uint64_t m, nb, cost;
+  bool missing;
+
+  __device__ EnumWarp(const EnumArgs& A_, const EnumGraph& g_, unsigned char* base, const uint64_t* tm,
+                      const uint64_t* tv, bool st)
+      : A(A_), g(g_), tmask(tm), tval(tv), staged(st), n(g_.n), lane(threadIdx.x & 31) {
+    const EnumFrame L = enum_frame(A_.n_max);
+    full = n == 64 ? ~0ull : ((1ull << n) - 1);
+    fe = reinterpret_cast<uint64_t*>(base + L.e);
+    fcost = reinterpret_cast<uint64_t*>(base + L.cost);
+    fmask = reinterpret_cast<uint64_t*>(base + L.mask);
+    fnb = reinterpret_cast<uint64_t*>(base + L.nb);
+    fn = reinterpret_cast<int32_t*>(base + L.n_cand);
+    fnext = reinterpret_cast<int32_t*>(base + L.next);
+    path = reinterpret_cast<int32_t*>(base + L.path);
+    best = reinterpret_cast<int32_t*>(base + L.best);
+    fcand = base + L.cand;
+    missing = false;
+  }
+  // Neighbours of a set of tables.
+  __device__ __forceinline__ uint64_t neighbours(uint64_t mask) const {
+    uint64_t r = 0;
+    for (; mask; mask &= mask - 1) r |= g.adj[__ffsll(static_cast<long long>(mask)) - 1];
+    return r;
+  }
+  // Candidates of frame fd for the prefix pm with neighbours pnb and cost pc, sorted by
+  // (estimate, id), with the costs of the extended prefixes.  Returns their number.
+  __device__ int expand(int fd, uint64_t pm, uint64_t pnb, uint64_t pc) {
+    const uint64_t c = pnb & ~pm;
+    const int v0 = lane, v1 = lane + 32;
+    const bool h0 = (c >> v0) & 1, h1 = (c >> v1) & 1;
+    uint64_t e0 = kInfBits, e1 = kInfBits;
+    bool miss = false;
+    if (h0) e0 = lookup(A, g, tmask, tval, staged, pm | (1ull << v0), &miss);
+    if (h1) e1 = lookup(A, g, tmask, tval, staged, pm | (1ull << v1), &miss);
+    if (__any_sync(0xffffffffu, miss)) missing = true;
+    int r0 = 0, r1 = 0;
+    if (c & (c - 1)) {
+      for (uint64_t rest = c; rest; rest &= rest - 1) {
+        const int j = __ffsll(static_cast<long long>(rest)) - 1;
+        const uint64_t ej = __shfl_sync(0xffffffffu, (unsigned long long)(j < 32 ? e0 : e1), j & 31);
+        r0 += ej < e0 || (ej == e0 && j < v0);
+        r1 += ej < e1 || (ej == e1 && j < v1);
+      }
+    }
+    const double base = bits_double(pc);
+    if (h0) {
+      fe[fd * n + r0] = uint64_t(__double_as_longlong(__dadd_rn(base, bits_double(e0))));
+      fcand[fd * n + r0] = uint8_t(v0);
+    }
+    if (h1) {
+      fe[fd * n + r1] = uint64_t(__double_as_longlong(__dadd_rn(base, bits_double(e1))));
+      fcand[fd * n + r1] = uint8_t(v1);
+    }
+    __syncwarp();
+    return __popcll(c);
+  }
+  // The current frame to shared memory (read by the warp's later returns to it, and by rounds).
+  __device__ __forceinline__ void save() {
+    __syncwarp();  // every lane has read what is rewritten now
+    if (lane == 0) {
+      fmask[d] = m;
+      fnb[d] = nb;
+      fcost[d] = cost;
+      fnext[d] = nx;
+      fn[d] = nc;
+    }
+    __syncwarp();
+  }
+  __device__ __forceinline__ void load(int fd) {
+    d = fd;
+    m = fmask[d];
+    nb = fnb[d];
+    cost = fcost[d];
+    nx = fnext[d];
+    nc = fn[d];
+  }
+  enum { kDone, kLimit, kPause, kFull, kAbort };
+  // Depth-first search of everything left at depths >= d0 (kDone), until `limit` extensions
+  // have been made (kLimit: another one was due), `pause` of them without completing a plan
+  // (kPause), or `plans` has reached max_plans (kFull); `stop`: a piece with an index below
+  // `self` completed a plan (kAbort).
+  __device__ int run(int d0, int64_t limit, int64_t pause, int64_t max_plans, int64_t& nodes, int64_t& pruned,
+                     int64_t& plans, uint64_t& min_cost, bool& improved, const volatile int* stop, int self) {
+    int64_t quiet = 0;
+    while (true) {
+      if (nx == nc) {  // back to the previous prefix
+        if (d == d0) return kDone;
+        load(d - 1);
+        continue;
+      }
+      if (nodes == limit) return kLimit;
+      if (quiet >= pause) return kPause;
+      if (stop && (quiet & 15) == 0 && __shfl_sync(0xffffffffu, *stop, 0) < self) return kAbort;
+      const uint64_t cc = fe[d * n + nx];
+      if (cc > min_cost) {  // early pruning, of this candidate and the dearer ones after it
+        const int64_t take = min(int64_t(nc - nx), limit - nodes);
+        nodes += take;
+        pruned += take;
+        nx += int(take);
+        quiet++;
+        continue;
+      }
+      const int v = fcand[d * n + nx];
+      nodes++;
+      nx++;
+      quiet++;
+      const uint64_t cm = m | (1ull << v);
+      if (cm == full) {  // complete plan
+        plans++;
+        quiet = 0;
+        if (cc < min_cost) {
+          min_cost = cc;
+          improved = true;
+          __syncwarp();
+          for (int t = lane; t <= d; t += 32) best[t] = path[t];
+          if (lane == 0) best[d + 1] = v;
+          __syncwarp();
+        }
+        if (max_plans > 0 && plans >= max_plans) return kFull;  // (-1: never)
+        continue;
+      }
+      save();
+      if (lane == 0) path[d + 1] = v;
+      d++;
+      m = cm;
+      nb |= g.adj[v];
+      cost = cc;
+      nx = 0;
+      nc = expand(d, m, nb, cost);
+    }
+  }
+};
+
+// A round's shared state.
+struct EnumRound {
+  int cmd, n_items, next, first, cur;  // cur: the list in use
+  uint64_t min_cost;
+  int64_t limit, plans;
+};
+enum { kCmdExit = 0, kCmdRound = 1 };
 
 }  // namespace
 
-__global__ void k_enumerate(const __grid_constant__ EnumArgs A) {
-  const int gi = int(blockIdx.x);
-  if (gi >= A.n_graphs || threadIdx.x != 0) return;
-  const EnumGraph& g = A.graphs[gi];
-  EnumFrames& F = *reinterpret_cast<EnumFrames*>(A.ws + size_t(gi) * kEnumFrameBytes);
-  const int n = g.n;
-  const uint64_t full = n == 64 ? ~0ull : ((1ull << n) - 1);
-  // source order: f(v) increasing, ties by id
-  int64_t mc = 0;
-  int32_t md = 0;
-  for (int v = 0; v < n; v++) {
-    mc = max(mc, g.card[v]);
-    md = max(md, g.deg[v]);
-  }
-  int src[kEnumMaxN];
-  double fv[kEnumMaxN];
-  for (int v = 0; v < n; v++) {
-    const double a = mc > 0 ? __ddiv_rn(__ll2double_rn(g.card[v]), __ll2double_rn(mc)) : 0.0;
-    const double b = md > 0 ? __ddiv_rn(double(g.deg[v]), double(md)) : 0.0;
-    const double f = __dadd_rn(__dmul_rn(A.alpha, a), __dmul_rn(A.beta, b));
-    int j = v;
-    while (j > 0 && fv[j - 1] > f) {
-      fv[j] = fv[j - 1];
-      src[j] = src[j - 1];
-      j--;
+__global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_constant__ EnumArgs A) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ EnumRound R;
+  __shared__ int scan[kEnumMaxWarps * 32 + 1];
+  const EnumGraph& g = A.graphs[blockIdx.x];
+  const int n = g.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = A.warps;
+  const EnumSmem L = enum_smem(A.n_max, W);
+  uint64_t* tmask = reinterpret_cast<uint64_t*>(smem + L.table);
+  uint64_t* tval = tmask + A.stage_slots;
+  int32_t* src = reinterpret_cast<int32_t*>(smem + L.src);
+  EnumPiece* piece[2] = {reinterpret_cast<EnumPiece*>(smem + L.piece[0]), reinterpret_cast<EnumPiece*>(smem + L.piece[1])};
+  uint8_t* ppath[2] = {smem + L.path[0], smem + L.path[1]};  // [kEnumItems][n]
+  EnumResult* result = reinterpret_cast<EnumResult*>(smem + L.result);
+  const int64_t size = int64_t(1) << g.h_log2;
+  const bool staged = size <= A.stage_slots;
+  if (staged)
+    for (int64_t i = threadIdx.x; i < size; i += blockDim.x) {
+      const EnumSlot* sl = A.slots + g.h_begin + i;
+      const uint64_t k = load_mask(sl);
+      tmask[i] = k;
+      tval[i] = k ? est_bits(__ldg(A.est + load_sub(sl))) : 0;
     }
-    fv[j] = f;
-    src[j] = v;
-  }
-  double min_cost = INFINITY;
-  int best[kEnumMaxN];
-  bool have = false, missing = false, out_of_budget = false;
-  int64_t plans = 0, nodes = 0, pruned = 0;
-  for (int si = 0; si < n && !out_of_budget; si++) {
-    const int s = src[si];
-    int64_t p = 0;
-    F.mask[0] = 1ull << s;
-    F.nb[0] = g.adj[s];
-    F.cost[0] = 0.0;
-    F.path[0] = s;
-    if (F.mask[0] == full) {  // one table: the plan is complete and costs nothing
-      plans++;
-      if (0.0 < min_cost) {
-        min_cost = 0.0;
-        best[0] = s;
-        have = true;
-      }
-      continue;
+  if (warp == 0) {  // source order: f(v) increasing, ties by id; lane v takes tables v and v + 32
+    const int v0 = lane, v1 = lane + 32;
+    const int64_t card0 = v0 < n ? g.card[v0] : 0, card1 = v1 < n ? g.card[v1] : 0;
+    int64_t mc = max(int64_t(0), max(card0, card1));
+    int32_t md = max(v0 < n ? g.deg[v0] : 0, v1 < n ? g.deg[v1] : 0);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      mc = max(mc, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mc, o));
+      md = max(md, __shfl_xor_sync(0xffffffffu, md, o));
     }
-    expand(A, g, F, 0, &missing);
-    int d = 0;
-    while (d >= 0) {
-      if (F.next[d] == F.n_cand[d]) {
-        d--;
-        continue;
+    auto f_of = [&](int v, int64_t card) {
+      if (v >= n) return double(INFINITY);
+      const double a = mc > 0 ? __ddiv_rn(__ll2double_rn(card), __ll2double_rn(mc)) : 0.0;
+      const double b = md > 0 ? __ddiv_rn(double(g.deg[v]), double(md)) : 0.0;
+      return __dadd_rn(__dmul_rn(A.alpha, a), __dmul_rn(A.beta, b));
+    };
+    const double f0 = f_of(v0, card0), f1 = f_of(v1, card1);
+    int r0 = 0, r1 = 0;
+    for (int j = 0; j < n; j++) {
+      const double fj = __shfl_sync(0xffffffffu, j < 32 ? f0 : f1, j & 31);
+      r0 += fj < f0 || (fj == f0 && j < v0);
+      r1 += fj < f1 || (fj == f1 && j < v1);
+    }
+    if (v0 < n) src[r0] = v0;
+    if (v1 < n) src[r1] = v1;
+  }
+  __syncthreads();
+  EnumWarp S(A, g, smem + L.frame + size_t(enum_frame(A.n_max).bytes) * warp, tmask, tval, staged);
+
+  // ---- the sequential search's state (warp 0; uniform over its lanes)
+  uint64_t min_cost = kInfBits;
+  bool have = false, missing = false, out_of_budget = false, alone = W < 2;
+  int64_t plans = 0, nodes = 0, pruned = 0, p = 0;  // p: plans completed from this source
+  int si = -1;
+  bool open = false;  // a source's search is under way, at S's current frame
+
+  // Warp 0: the unvisited prefixes of the open search as the first list of pieces, in search
+  // order (the deepest frame's remaining candidates first); false when they are too many.
+  auto collect = [&]() {
+    int at = 0;
+    for (int fd = S.d; fd >= 0; fd--) {
+      const int k0 = S.fnext[fd], k1 = S.fn[fd];
+      int live = 0;  // candidates not yet pruned: a prefix of the frame's order
+      for (int k = k0; k < k1; k++) live += S.fe[fd * n + k] <= min_cost;
+      const int rest = k1 - k0 - live;
+      if (at + live + (rest > 0) > kEnumItems) return false;
+      for (int k = k0 + lane; k < k0 + live; k += 32) {
+        EnumPiece q;
+        const int v = S.fcand[fd * n + k];
+        q.mask = S.fmask[fd] | (1ull << v);
+        q.cost = S.fe[fd * n + k];
+        q.pre = q.count = 0;
+        q.kind = q.mask == S.full ? kPlan : kTask;
+        q.len = uint8_t(fd + 2);
+        q.missing = 0;
+        uint8_t* pp = ppath[0] + size_t(at + k - k0) * n;
+        for (int t = 0; t <= fd; t++) pp[t] = uint8_t(S.path[t]);
+        pp[fd + 1] = uint8_t(v);
+        piece[0][at + k - k0] = q;
       }
-      const int k = F.next[d]++;
-      const int v = F.cand[d][k];
-      if (nodes == A.max_nodes) {  // budget spent: stop after exactly max_nodes extensions
-        out_of_budget = true;
-        break;
-      }
-      nodes++;
-      const uint64_t cm = F.mask[d] | (1ull << v);
-      const double cc = __dadd_rn(F.cost[d], F.e[d][k]);
-      F.path[d + 1] = v;
-      if (cc > min_cost) {  // early pruning
-        pruned++;
-        continue;
-      }
-      if (cm == full) {  // complete plan
-        plans++;
-        if (cc < min_cost) {
-          min_cost = cc;
-          for (int t = 0; t <= d + 1; t++) best[t] = F.path[t];
-          have = true;
+      at += live;
+      if (rest > 0) {
+        if (lane == 0) {
+          EnumPiece q = {};
+          q.kind = kPruned;
+          q.count = rest;
+          piece[0][at] = q;
         }
-        if (A.max_plans > 0 && ++p == A.max_plans) break;  // this source's search ends (-1: never)
-        continue;
+        at++;
       }
-      d++;
-      F.mask[d] = cm;
-      F.nb[d] = F.nb[d - 1] | g.adj[v];
-      F.cost[d] = cc;
-      expand(A, g, F, d, &missing);
     }
+    __syncwarp();
+    if (lane == 0) {
+      R.n_items = at;
+      R.cur = 0;
+    }
+    return true;
+  };
+
+  for (;;) {
+    if (warp == 0) {
+      int cmd = kCmdExit;
+      while (!out_of_budget) {
+        if (!open) {  // the next source
+          if (++si >= n) break;
+          p = 0;
+          S.d = 0;
+          S.m = 1ull << src[si];
+          S.nb = g.adj[src[si]];
+          S.cost = 0;  // 0.0
+          S.nx = 0;
+          __syncwarp();
+          if (lane == 0) S.path[0] = src[si];
+          if (S.m == S.full) {  // one table: the plan is complete and costs nothing
+            plans++;
+            if (min_cost != 0) {
+              min_cost = 0;
+              if (lane == 0) S.best[0] = src[si];
+              have = true;
+            }
+            continue;
+          }
+          S.nc = S.expand(0, S.m, S.nb, S.cost);
+          open = true;
+        }
+        bool improved = false;
+        const int64_t p0 = p;
+        // (a search without a limit on its plans completes them all the time: alone)
+        const int64_t pause = alone || A.max_plans < 0 ? INT64_MAX : kEnumSeqNodes;
+        const int why =
+            S.run(0, A.max_nodes, pause, A.max_plans, nodes, pruned, p, min_cost, improved, nullptr, 0);
+        plans += p - p0;
+        have |= improved;
+        if (why == EnumWarp::kLimit) out_of_budget = true;  // budget spent: exactly max_nodes extensions
+        if (why == EnumWarp::kDone || why == EnumWarp::kFull) open = false;
+        if (why == EnumWarp::kPause) {
+          S.save();
+          if (!collect()) {
+            alone = true;
+            continue;
+          }
+          cmd = kCmdRound;
+          if (lane == 0) {
+            R.min_cost = min_cost;
+            R.limit = A.max_nodes - nodes;
+            R.plans = p;
+            R.next = 0;
+          }
+          break;
+        }
+      }
+      if (lane == 0) R.cmd = cmd;
+      missing |= S.missing;
+      S.missing = false;
+    }
+    __syncthreads();
+    if (R.cmd == kCmdExit) break;
+
+    // ---- a round.  Split the shallowest unsearched prefixes while the list has room.
+    for (int step = 0; step < 64; step++) {
+      const int ni = R.n_items, cur = R.cur, i = threadIdx.x;
+      int len = 1 << 20;
+      bool task = false;
+      if (i < ni && i < kEnumItems && piece[cur][i].kind == kTask) {
+        task = true;
+        len = piece[cur][i].len;
+      }
+      const int n_task = __syncthreads_count(task);
+      // shallowest length (prefixes of n - 2 tables and more are searched whole)
+      scan[threadIdx.x] = len;
+      __syncthreads();
+      for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+        if (i < o) scan[i] = min(scan[i], scan[i + o]);
+        __syncthreads();
+      }
+      const int shallow = scan[0];
+      __syncthreads();
+      if (n_task == 0 || n_task >= kEnumTasksWanted || shallow > n - 3) break;  // block-uniform
+      // pieces each one becomes, in order, as long as the whole list fits
+      const bool want = task && len == shallow;
+      int more = 0;
+      if (want) more = __popcll(S.neighbours(piece[cur][i].mask) & ~piece[cur][i].mask);  // its children + pruned rest
+      int incl = more;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      if (lane == 31) scan[warp] = incl;
+      __syncthreads();
+      for (int k = 0; k < warp; k++) incl += scan[k];
+      const bool fits = ni + incl <= kEnumItems;
+      const int dst = i + (fits ? incl - more : 0);
+      // (once one does not fit, none after it does: incl is monotone; they move by the last fitting sum)
+      __syncthreads();
+      if (i == 0) scan[0] = 0;
+      __syncthreads();
+      if (fits) atomicMax(&scan[0], incl);
+      __syncthreads();
+      const int grown = scan[0];
+      const int to = fits ? dst : i + grown;
+      const int any = __syncthreads_or(want && fits && more > 0);
+      if (!any) break;
+      if (i < ni && !(want && fits)) {  // moves
+        piece[cur ^ 1][to] = piece[cur][i];
+        for (int t = 0; t < n; t++) ppath[cur ^ 1][size_t(to) * n + t] = ppath[cur][size_t(i) * n + t];
+      }
+      // each split prefix: a warp expands it and writes its children
+      __shared__ int todo[kEnumItems], todo_at[kEnumItems], n_todo;
+      if (i == 0) n_todo = 0;
+      __syncthreads();
+      if (i < ni && want && fits) {
+        const int k = atomicAdd(&n_todo, 1);
+        todo[k] = i;
+        todo_at[k] = to;
+      }
+      __syncthreads();
+      for (int k = warp < W ? warp : n_todo; k < n_todo; k += W) {
+        const EnumPiece q = piece[cur][todo[k]];
+        const uint8_t* pp = ppath[cur] + size_t(todo[k]) * n;
+        const uint64_t pnb = S.neighbours(q.mask);
+        const int slots = 1 + __popcll(pnb & ~q.mask);  // the room reserved for it
+        // (warp 0's frames hold the open search: candidates go to the row of the last prefix
+        // length, n - 1, whose frame has none of its own)
+        S.missing = false;
+        const int nc = S.expand(n - 1, q.mask, pnb, q.cost);
+        int live = 0;
+        for (int c = lane; c < nc; c += 32) live += S.fe[(n - 1) * n + c] <= R.min_cost;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
+        for (int c = lane; c < slots; c += 32) {
+          EnumPiece r = {};
+          const size_t o = size_t(todo_at[k] + c);
+          if (c < live) {
+            const int v = S.fcand[(n - 1) * n + c];
+            r.mask = q.mask | (1ull << v);
+            r.cost = S.fe[(n - 1) * n + c];
+            r.kind = r.mask == S.full ? kPlan : kTask;
+            r.len = uint8_t(q.len + 1);
+            for (int t = 0; t < q.len; t++) ppath[cur ^ 1][o * n + t] = pp[t];
+            ppath[cur ^ 1][o * n + q.len] = uint8_t(v);
+          } else if (c == live) {  // its pruned candidates (or nothing): the prefix itself counts here at the latest
+            r.kind = kPruned;
+            r.count = nc - live;
+          }
+          if (c == 0) {  // the prefix's own extension comes right before its first piece
+            r.pre = q.pre + 1;
+            r.missing = q.missing | uint8_t(S.missing);
+          }
+          piece[cur ^ 1][o] = r;
+        }
+        __syncwarp();
+      }
+      __syncthreads();
+      if (i == 0) {
+        R.n_items = ni + grown;
+        R.cur = cur ^ 1;
+      }
+      __syncthreads();
+    }
+    // the first complete plan among the pieces ends the round's useful part
+    {
+      const int i = threadIdx.x;
+      __syncthreads();
+      if (i == 0) R.first = INT32_MAX;
+      __syncthreads();
+      if (i < R.n_items && i < kEnumItems && piece[R.cur][i].kind == kPlan) atomicMin(&R.first, i);
+      __syncthreads();
+    }
+    const EnumPiece* list = piece[R.cur];
+    const uint8_t* lpath = ppath[R.cur];
+    const int n_items = R.n_items;
+    // Search the pieces in order.  Warp 0 keeps the open search's frames: it takes no piece.
+    if (warp > 0 && warp < W) {
+      for (;;) {
+        int k = 0;
+        if (lane == 0) {
+          k = atomicAdd(&R.next, 1);
+          if (k >= n_items || k > *const_cast<volatile int*>(&R.first)) k = -1;
+        }
+        k = __shfl_sync(0xffffffffu, k, 0);
+        if (k < 0) break;
+        const EnumPiece q = list[k];
+        if (q.kind != kTask) continue;
+        S.d = q.len - 1;
+        S.m = q.mask;
+        S.nb = S.neighbours(q.mask);
+        S.cost = q.cost;
+        S.nx = 0;
+        S.missing = false;
+        __syncwarp();
+        for (int t = lane; t < q.len; t += 32) S.path[t] = lpath[size_t(k) * n + t];
+        __syncwarp();
+        S.nc = S.expand(S.d, S.m, S.nb, S.cost);
+        int64_t wn = 1, wp = 0, wplans = R.plans;
+        uint64_t wcost = R.min_cost;
+        bool improved = false;
+        // (limit + 1: reaching it means more than the budget is left for)
+        const int why = S.run(S.d, R.limit + 1, INT64_MAX, A.max_plans, wn, wp, wplans, wcost, improved, &R.first, k);
+        if (lane == 0) {
+          EnumResult& r = result[k];
+          r.nodes = wn;
+          r.pruned = wp;
+          r.cost = wcost;
+          r.plans = int32_t(wplans - R.plans);
+          r.warp = uint8_t(warp);
+          r.missing = S.missing;
+          r.over = why == EnumWarp::kLimit;
+          r.improved = improved;
+          __threadfence_block();
+          if (wplans > R.plans) atomicMin(&R.first, k);
+        }
+        __syncwarp();
+        if (wplans > R.plans) break;  // its best plan stays in this warp's frames
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {  // take the results in search order, up to the first piece with a plan
+      const int first = R.first;  // INT32_MAX: none
+      int64_t rn = 0, rp = 0;
+      bool over = false, miss = false;
+      for (int k = lane; k < n_items && k <= first; k += 32) {
+        const EnumPiece q = list[k];
+        rn += q.pre;
+        miss |= q.missing != 0;
+        if (q.kind == kTask) {
+          const EnumResult r = result[k];
+          rn += r.nodes;
+          rp += r.pruned;
+          miss |= r.missing != 0;
+          over |= r.over != 0;
+        } else if (q.kind == kPruned) {
+          rn += q.count;
+          rp += q.count;
+        } else if (q.kind == kPlan) {
+          rn += 1;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        rn += __shfl_xor_sync(0xffffffffu, (long long)rn, o);
+        rp += __shfl_xor_sync(0xffffffffu, (long long)rp, o);
+      }
+      over = __any_sync(0xffffffffu, over);
+      miss = __any_sync(0xffffffffu, miss);
+      if (over || rn > A.max_nodes - nodes) {  // the budget ends inside: the sequential search finds where
+        alone = true;
+        S.load(S.d);
+      } else {
+        nodes += rn;
+        pruned += rp;
+        missing |= miss;
+        if (first == INT32_MAX) {
+          open = false;  // nothing left from this source
+        } else {
+          const EnumPiece q = list[first];
+          const uint8_t* pp = lpath + size_t(first) * n;
+          int64_t got = 1;
+          if (q.kind == kPlan) {
+            if (q.cost < min_cost) {
+              min_cost = q.cost;
+              have = true;
+              __syncwarp();
+              for (int t = lane; t < n; t += 32) S.best[t] = pp[t];
+            }
+          } else {
+            const EnumResult r = result[first];
+            got = r.plans;
+            if (r.improved) {
+              min_cost = r.cost;
+              have = true;
+              const int32_t* wb = reinterpret_cast<const int32_t*>(
+                  smem + L.frame + size_t(enum_frame(A.n_max).bytes) * r.warp + enum_frame(A.n_max).best);
+              __syncwarp();
+              for (int t = lane; t < n; t += 32) S.best[t] = wb[t];
+            }
+          }
+          plans += got;
+          p += got;
+          if (A.max_plans > 0 && p >= A.max_plans) {
+            open = false;
+          } else {  // go on after that piece: its path's frames, each past the table the path takes
+            __syncwarp();
+            for (int t = lane; t < q.len; t += 32) S.path[t] = pp[t];
+            __syncwarp();
+            uint64_t m = 1ull << S.path[0], nb = g.adj[S.path[0]], cost = 0;
+            for (int fd = 0; fd + 1 < q.len; fd++) {
+              const int nc = S.expand(fd, m, nb, cost), v = S.path[fd + 1];
+              int at = 0;
+              while (at < nc && S.fcand[fd * n + at] != v) at++;  // a candidate by construction
+              S.d = fd, S.m = m, S.nb = nb, S.cost = cost, S.nx = at + 1, S.nc = nc;
+              const uint64_t next = at < nc ? S.fe[fd * n + at] : cost;
+              S.save();
+              m |= 1ull << v;
+              nb |= g.adj[v];
+              cost = next;
+            }
+          }
+        }
+      }
+      S.missing = false;  // (what counts is in `missing`)
+    }
+    __syncthreads();
   }
-  for (int t = 0; t < kEnumMaxN; t++) A.order[int64_t(gi) * kEnumMaxN + t] = (have && t < n) ? best[t] : -1;
-  A.cost[gi] = have ? min_cost : INFINITY;
-  A.stats[int64_t(gi) * 3 + 0] = plans;
-  A.stats[int64_t(gi) * 3 + 1] = nodes;
-  A.stats[int64_t(gi) * 3 + 2] = pruned;
+  if (warp != 0) return;
+  for (int t = lane; t < kEnumMaxN; t += 32)
+    A.order[int64_t(blockIdx.x) * kEnumMaxN + t] = (have && t < n) ? S.best[t] : -1;
+  if (lane != 0) return;
+  A.cost[blockIdx.x] = bits_double(have ? min_cost : kInfBits);
+  A.stats[int64_t(blockIdx.x) * 3 + 0] = plans;
+  A.stats[int64_t(blockIdx.x) * 3 + 1] = nodes;
+  A.stats[int64_t(blockIdx.x) * 3 + 2] = pruned;
   if (missing) set_status(A.status, CMP_EUNSUPPORTED);
   if (out_of_budget) set_status(A.status, CMP_ETIMEOUT);
 }
@@ -279,7 +828,7 @@ cmp_status enum_plan(const cmp_graph* graphs, int32_t n_graphs, int32_t n_sub, c
     EnumSlot* tab = P->slots.data() + g.h_begin;
     const uint64_t size = uint64_t(1) << lg;
     for (const auto& x : list) {
-      uint64_t i = enum_hash(x.first) & (size - 1);
+      uint64_t i = enum_hash(x.first, lg);
       while (tab[i].mask != 0) i = (i + 1) & (size - 1);
       tab[i] = EnumSlot{x.first, x.second};
     }
@@ -287,7 +836,7 @@ cmp_status enum_plan(const cmp_graph* graphs, int32_t n_graphs, int32_t n_sub, c
   EnumPlanHdr& H = P->hdr;
   std::memset(&H, 0, sizeof(H));
   H.magic = kEnumPlanMagic;
-  H.version = 2;
+  H.version = kEnumPlanVersion;
   H.n_graphs = n_graphs;
   H.n_sub = n_sub;
   H.n_slots = int64_t(P->slots.size());
@@ -297,7 +846,13 @@ cmp_status enum_plan(const cmp_graph* graphs, int32_t n_graphs, int32_t n_sub, c
   H.off_slots = int64_t(off);
   off += align16(sizeof(EnumSlot) * P->slots.size());
   H.total_bytes = int64_t(off);
-  H.ws_bytes = int64_t(kEnumFrameBytes * size_t(n_graphs));
+  H.ws_bytes = int64_t(kEnumWsBytes);
+  H.n_max = 1;
+  H.stage_slots = 0;
+  for (const EnumGraph& g : P->graphs) {
+    H.n_max = std::max(H.n_max, g.n);
+    if ((int64_t(1) << g.h_log2) <= kEnumStageSlots) H.stage_slots = std::max(H.stage_slots, 1 << g.h_log2);
+  }
   return CMP_OK;
 }
 
@@ -340,7 +895,7 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
   if (!plan_host || !plan_dev) return CMP_EINVAL;
   EnumPlanHdr H;
   std::memcpy(&H, plan_host, sizeof(H));
-  if (H.magic != kEnumPlanMagic || H.version != 2) return CMP_EINVAL;
+  if (H.magic != kEnumPlanMagic || H.version != kEnumPlanVersion) return CMP_EINVAL;
   if (!order_dev || !cost_dev || !stats_dev || (H.n_sub > 0 && !est_dev)) return CMP_EINVAL;
   if (!ws_dev || ws_bytes < size_t(H.ws_bytes)) return CMP_EWORKSPACE;
   double alpha = 0.5, beta = 0.5;
@@ -361,12 +916,22 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
   a.beta = beta;
   a.max_plans = max_plans;
   a.max_nodes = max_nodes;
-  a.ws = static_cast<unsigned char*>(ws_dev);
+  a.n_max = H.n_max;
+  a.stage_slots = H.stage_slots;
   a.order = order_dev;
   a.cost = cost_dev;
   a.stats = stats_dev;
   a.status = status_dev;
-  k_enumerate<<<unsigned(H.n_graphs), 32, 0, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+  // as many warps as their frames leave room for beside the lists and the staged table
+  int warps = kEnumMaxWarps;
+  auto smem_of = [&](int k) { return size_t(enum_smem(H.n_max, k).table) + 16 * size_t(H.stage_slots); };
+  while (warps > 8 && smem_of(warps) > size_t(200) * 1024) warps >>= 1;  // 256 threads at least: one per piece
+  a.warps = warps;
+  while (a.warps > 1 && smem_of(a.warps) > size_t(200) * 1024) a.warps--;  // those beyond search nothing
+  const size_t smem = smem_of(a.warps);
+  if (cudaFuncSetAttribute(k_enumerate, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
+    return CMP_ECUDA;
+  k_enumerate<<<unsigned(H.n_graphs), 32 * warps, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
   return cudaGetLastError() == cudaSuccess ? CMP_OK : CMP_ECUDA;
 }
 
