@@ -37,6 +37,7 @@ struct PlanOut {
   std::vector<TriSub> tris;
   std::vector<EstItem> tri_items;  // appended after the generic items
   int32_t tri_max_leaves = 0;
+  std::vector<CycSub> cycs;
   std::vector<StarFam> stars;
   std::vector<StarUnit> star_suf_units, star_lat_units;
   int64_t star_suf_words = 0, star_t_entries = 0, n_star_sub = 0;
@@ -152,6 +153,53 @@ bool plan_triangle(const cmp_graph& g, const std::vector<int>& es, const std::ve
       it.c1 = std::min(w, (ch + 1) * kTriCols);
       P->tri_items.push_back(it);
     }
+  return true;
+}
+
+// A simple cycle of four or more tables (estimate_cycle.cu): every table touches two edges.
+// Its sketches are listed in cycle order from the lowest table.  w: widths that fit; chunks:
+// a row's partial sums must hold its CycRow.
+bool plan_cycle(const cmp_graph& g, const std::vector<int>& es, uint64_t mask, int32_t w, int32_t n_chunks,
+                int32_t sub_index, PlanOut* P, EstSub* sb) {
+  const int n = __builtin_popcountll(mask);
+  if (n < 4 || int(es.size()) != n || w > kCycMaxW || n_chunks < kCycRowItems) return false;
+  auto touches = [&](int e, int t) { return g.edge_u[e] == t || g.edge_v[e] == t; };
+  std::vector<int> deg(g.n_tables, 0);
+  for (int e : es) deg[g.edge_u[e]]++, deg[g.edge_v[e]]++;
+  for (int t = 0; t < g.n_tables; t++)
+    if (((mask >> t) & 1) && deg[t] != 2) return false;
+  CycSub c;
+  std::memset(&c, 0, sizeof(c));
+  c.in_begin = int32_t(P->ins.size());
+  c.n = n;
+  c.sub = sub_index;
+  int t = 0, before = -1;
+  while (!((mask >> t) & 1)) t++;
+  for (int e : es)  // the cycle is entered by the first edge of its lowest table
+    if (before < 0 && touches(e, t)) before = e;
+  for (int k = 0; k < n; k++) {
+    int after = -1;
+    for (int e : es)
+      if (e != before && touches(e, t)) after = e;
+    for (int e : {before, after}) {
+      const int me = g.edge_u[e] == t ? 0 : 1;
+      EstIn x;
+      std::memset(&x, 0, sizeof(x));
+      x.s = g.sketch[2 * e + me];
+      x.abs = g.abs_sorted[2 * e + me];
+      x.perm = g.perm[2 * e + me];
+      x.rk = g.ranks[2 * e + me];
+      x.tslot = g.slot[2 * e + me];
+      x.kind = kInCond;
+      x.slot = e;
+      x.suf = -1;
+      P->ins.push_back(x);
+    }
+    t = g.edge_u[after] == t ? g.edge_v[after] : g.edge_u[after];
+    before = after;
+  }
+  sb->cyc = int32_t(P->cycs.size());
+  P->cycs.push_back(c);
   return true;
 }
 
@@ -437,6 +485,7 @@ cmp_status plan_sub(const cmp_graph& g, int32_t gi, uint64_t mask, int32_t d, in
   std::memset(&sb, 0, sizeof(sb));
   sb.job = -1;
   sb.star = -1;
+  sb.cyc = -1;
   sb.scale = 1.0;  // sampled tables: prod over the sub-plan's tables, ascending, of 1 / rate
   if (g.sample_rate)
     for (int t = 0; t < nt; t++) {
@@ -480,6 +529,7 @@ cmp_status plan_sub(const cmp_graph& g, int32_t gi, uint64_t mask, int32_t d, in
   // the root's sorted positions, split into kRootSplit chunks (one CTA each)
   sb.split = cond.empty() && sb.n_ops == 1 && w >= kRootSplitMinW && P->ops[sb.op_begin].k >= 2 ? 1 : 0;
   if (sb.split) sb.n_chunks = kRootSplit;
+  if (cond.size() == 1 && !(flags & CMP_EST_GENERIC_ONLY)) plan_cycle(g, es, mask, w, sb.n_chunks, sub_index, P, &sb);
   P->subs.push_back(sb);
   for (int i = 0; i < d; i++)
     for (int ch = 0; ch < sb.n_chunks; ch++) {
@@ -521,6 +571,7 @@ cmp_status plan_jobs(const cmp_graph* graphs, int32_t d, int32_t n_sub, CacheCtx
       EstSub sb;
       std::memset(&sb, 0, sizeof(sb));
       sb.job = n.cid;
+      sb.cyc = -1;
       sb.scale = 1.0;
       sb.tri = -1;
       sb.n_chunks = 1;
@@ -729,6 +780,9 @@ cmp_status plan_all(const cmp_graph* graphs, int32_t n_graphs, int32_t d, int32_
   off += align16(sizeof(StarUnit) * size_t(H->n_star_units));
   H->star_suf_words = P->star_suf_words;
   H->star_t_entries = P->star_t_entries;
+  H->n_cyc = int64_t(P->cycs.size());
+  H->off_cyc = int64_t(off);
+  off += align16(sizeof(CycSub) * P->cycs.size());
   H->off_star_q = int64_t(off);
   H->n_star_q = int64_t(P->star_q.size());
   off += align16(sizeof(int32_t) * P->star_q.size());
@@ -883,6 +937,7 @@ cmp_status cmp_estimate_plan_encode(const cmp_graph* graphs, int32_t n_graphs, i
   if (!P.star_lat_units.empty())
     std::memcpy(b + H.off_star_units + sizeof(StarUnit) * P.star_suf_units.size(), P.star_lat_units.data(),
                 sizeof(StarUnit) * P.star_lat_units.size());
+  if (!P.cycs.empty()) std::memcpy(b + H.off_cyc, P.cycs.data(), sizeof(CycSub) * P.cycs.size());
   if (!P.star_q.empty()) std::memcpy(b + H.off_star_q, P.star_q.data(), sizeof(int32_t) * P.star_q.size());
   if (!F.subs.empty()) {  // the exact tier's own generic plan
     std::memcpy(b + H.wide_off_subs, F.subs.data(), sizeof(EstSub) * F.subs.size());

@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(MAXT, MINB) k_estimate_items(const __grid_cons
     if (retry && A.partial_ovf[it] != 2) continue;  // block-uniform
     const EstItem item = A.items[it];
     const EstSub sb = A.subs[item.sub];
+    if (sb.cyc >= 0 && A.partial_ovf[it] == kCycDone) continue;  // k_cycle has the row (block-uniform)
     const int64_t ro = int64_t(item.row) * w;  // row offset inside every [d][w] array
     i128* const gout = sb.job >= 0 ? A.cache + (int64_t(sb.job) * A.d + item.row) * w : nullptr;
     const int in0 = A.ops[sb.op_begin].in_begin;
@@ -820,6 +821,12 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_estimate_finalize(const __
         ovf |= A.star_tf[idx] != 0;
         ovf |= add_ovf(s, A.star_t[idx], &s);
       }
+    } else if (const CycRow* cr = cyc_taken(A, q, i)) {  // a simple cycle's row: its limbs
+      uint32_t v[kCycMaxLimbs];
+      cyc_value(*cr, v);
+      s = i128((u128((uint64_t(v[3]) << 32) | v[2]) << 64) | ((uint64_t(v[1]) << 32) | v[0]));
+      const uint32_t ext = (v[3] >> 31) ? ~0u : 0u;
+      for (int l = 4; l < kCycMaxLimbs; l++) ovf |= v[l] != ext;
     } else {
       const int64_t it0 = int64_t(sb.item_begin) + int64_t(i) * sb.n_chunks;
       for (int ch = 0; ch < sb.n_chunks; ch++) {
@@ -847,7 +854,8 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_estimate_finalize(const __
     if (ovf) {
       const uint32_t k = atomicAdd(A.wide_queue, 1u);
       const bool lat = wide_star_row(A, q);
-      const uint32_t nch = uint32_t(wide_row_units(A, q));
+      const bool cyc = cyc_taken(A, q, i) != nullptr;
+      const uint32_t nch = uint32_t(wide_row_units(A, q, i));
       const uint32_t cap = uint32_t(A.wide_unit_cap);
       // no reservation once the units are used up (the counter cannot wrap)
       const bool room = k < uint32_t(A.wide_qcap) && *reinterpret_cast<volatile uint32_t*>(A.wide_queue + 2) < cap;
@@ -855,7 +863,7 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_estimate_finalize(const __
       if (u0 < cap && nch <= cap - u0) {
         A.wide_queue[4 + k] = uint32_t(q * d + i);
         A.wide_row_start[k] = int32_t(u0);
-        for (uint32_t c = 0; c < nch; c++) A.wide_units[u0 + c] = (uint64_t(k) << 32) | (lat ? kUnitLattice : c);
+        for (uint32_t c = 0; c < nch; c++) A.wide_units[u0 + c] = (uint64_t(k) << 32) | (lat ? kUnitLattice : (cyc ? kUnitCycle : c));
         if (lat) {  // its lattice sums start from 0 (residues) and 0.0 (bound)
           for (int j = 0; j <= kWideMods; j++) A.wide_part[int64_t(u0) * (kWideMods + 1) + j] = 0;
           atomicAdd(A.wide_star_cnt + int64_t(sb.star) * d + i, 1u);
@@ -897,6 +905,10 @@ __global__ void __launch_bounds__(kFinalizeThreads) k_estimate_finalize(const __
 
 cudaError_t launch_estimate(const EstArgs& a, const EstPlanHdr& H, double* est, int64_t* row_est, cudaStream_t st,
                             int64_t* wide_rows) {
+  {  // simple cycles first: the generic items of the rows it takes return at once
+    const cudaError_t e = launch_estimate_cycle(a, st);
+    if (e != cudaSuccess) return e;
+  }
   // cached subtree messages, one launch per level, in int128 storage
   // three register budgets: 1024 threads (one CTA per SM), 512 (wider ILP), 256 (four CTAs
   // per SM: more items in flight when each is bound by its barriers, e.g. conditioned cycles)

@@ -52,6 +52,9 @@ struct EstSub {
   uint32_t sbits;     // star: its leaf edges, bit u = edge u of the family (ascending edge id)
   int32_t split;      // 1: a tree whose only operation is the root; its chunks split the root's
                       // sorted positions (item [c0, c1)), each recomputing the leaf suffix sums
+  int32_t cyc;        // >= 0: a simple cycle (its CycSub); its items are the fallback of rows that
+                      // k_cycle does not take
+  int32_t pad;
 };
 constexpr int32_t kRootSplitMinW = 16384;  // widths from which such roots are split
 constexpr int32_t kRootSplit = 8;          // chunks of sorted positions per row
@@ -112,6 +115,25 @@ constexpr int32_t kTriMaxW = 16384;   // queries and rows are sorted in shared m
 constexpr int32_t kTriMaxLeaves = 16; // leaves per triangle node
 constexpr int32_t kTriCols = 256;     // columns per sweep item (one per thread)
 
+// Simple cycles (estimate_cycle.cu): n >= 4 tables, each joined to its two neighbours.  Table
+// position t has two EstIn from in_begin + 2 t: its sketch on the edge before it and on the
+// edge after it, in cycle order (EstIn.slot = the edge id).
+struct CycSub {
+  int32_t in_begin, n, sub, pad;
+};
+// A row's state, in the partial sums of its first items (at least kCycRowItems of them): the
+// limb sums of its value modulo 2^(32 limbs), two's complement, carries unresolved; where and
+// in which direction the cycle is cut.  The row's items carry kCycDone in partial_ovf.
+constexpr int kCycMaxLimbs = 10;
+struct CycRow {
+  unsigned long long acc[kCycMaxLimbs];
+  int32_t limbs, cols, start, back;
+};
+constexpr int kCycRowItems = 8;  // 8 partial sums of 16 bytes hold a CycRow
+static_assert(sizeof(CycRow) <= 16 * kCycRowItems, "CycRow lives in the partial sums");
+constexpr int32_t kCycDone = 4;
+constexpr int32_t kCycMaxW = 4096;  // two product vectors of two limbs and the sketches fit in shared memory
+
 // Per triangle row (sub-plan, sketch row) scratch, in bytes, and its regions.
 struct TriLayout {
   int64_t hdr, vec, tmp, sg, pre, rkx, rpre, cky, ccol, qs, qr, qpre, gr, gqb, bytes;
@@ -167,6 +189,7 @@ struct EstPlanHdr {
   int32_t wide_max_slots, wide_max_in, wide_max_suf, wide_grid;
   int64_t wide_scratch_per_cta;
   int32_t wide_unit_cap, pad2;  // (row, conditioning chunk) units the tier can take per call
+  int64_t n_cyc, off_cyc;       // simple cycles
 };
 constexpr int32_t kWideQueueMax = 1 << 19;
 constexpr int32_t kWideCtasPerSm = 8;  // the tier's generic kernel: 128-thread CTAs, 8 per SM
@@ -175,7 +198,7 @@ constexpr int32_t kWideUnitMax = 1 << 20;
 // extend it to this size when it is smaller)
 constexpr int64_t kWideScratchBudget = int64_t(256) << 20;
 constexpr uint64_t kEstPlanMagic = 0x434d504553544d54ull;  // "CMPESTMT"
-constexpr int32_t kEstPlanVersion = 8;
+constexpr int32_t kEstPlanVersion = 9;
 
 // Exact tier beyond int128: a row is evaluated modulo kWideMods primes p_j = 2^62 - c_j
 // (exact ring arithmetic: the contraction is sums of products of the counters, and the
@@ -212,6 +235,8 @@ struct EstArgs {
   unsigned char* tri_scratch;  // tri_slots rows of tri_row_bytes
   int64_t tri_row_bytes, tri_slots;
   int32_t tri_max_leaves, tri_nch;
+  const CycSub* cyc;
+  int64_t n_cyc;
   i128* cache;          // [n_jobs][d][w] cached subtree messages, bucket order
   int32_t* cache_ovf;   // [n_jobs][d] 1: the message left int128
   int64_t n_job_items;
@@ -250,6 +275,34 @@ struct EstArgs {
 // conditioning chunk, or kUnitLattice: a star row's single unit, which its family's lattice
 // fills (the residues summed over its leaves a of T_a(S \ {a}), the largest of their bounds).
 constexpr uint32_t kUnitLattice = 0x80000000u;
+// ... or kUnitCycle: a simple cycle's row, whose value k_cycle left in the row's CycRow.
+constexpr uint32_t kUnitCycle = 0x40000000u;
+
+// The state of a cycle's row (it0 = its first item), and whether k_cycle has taken the row.
+__device__ __forceinline__ CycRow* cyc_row(const EstArgs& A, int64_t it0) {
+  return reinterpret_cast<CycRow*>(A.partial + it0);
+}
+__device__ __forceinline__ const CycRow* cyc_taken(const EstArgs& A, int64_t q, int row) {
+  const EstSub& sb = A.subs[q];
+  if (sb.cyc < 0) return nullptr;
+  const int64_t it0 = sb.item_begin + int64_t(row) * sb.n_chunks;
+  return A.partial_ovf[it0] == kCycDone ? cyc_row(A, it0) : nullptr;
+}
+// Its value as sign-extended 32-bit limbs (carries resolved).
+__device__ __forceinline__ void cyc_value(const CycRow& r, uint32_t (&v)[kCycMaxLimbs]) {
+  unsigned long long carry = 0;
+  uint32_t top = 0;
+#pragma unroll
+  for (int l = 0; l < kCycMaxLimbs; l++) {
+    if (l < r.limbs) {
+      const unsigned long long lo = (r.acc[l] & 0xFFFFFFFFull) + (carry & 0xFFFFFFFFull);
+      v[l] = top = uint32_t(lo);
+      carry = (r.acc[l] >> 32) + (carry >> 32) + (lo >> 32);
+    } else {
+      v[l] = (top >> 31) ? ~0u : 0u;
+    }
+  }
+}
 
 // A star sub-plan whose leaf set maps to it in its family's table: its queued rows are
 // evaluated on the family's lattice in modular arithmetic when enough rows of the (family,
@@ -258,8 +311,11 @@ __device__ __forceinline__ bool wide_star_row(const EstArgs& A, int64_t q) {
   const int32_t f = A.subs[q].star;
   return f >= 0 && A.star_q[A.star[f].q_off + A.subs[q].sbits] == int32_t(q);
 }
-// Units of a queued row of sub-plan q: one per conditioning chunk of its generic plan.
-__device__ __forceinline__ int wide_row_units(const EstArgs& A, int64_t q) { return max(1, A.wsubs[q].n_chunks); }
+// Units of a queued row of sub-plan q: one per conditioning chunk of its generic plan, one for
+// a cycle's row that k_cycle has taken.
+__device__ __forceinline__ int wide_row_units(const EstArgs& A, int64_t q, int row) {
+  return cyc_taken(A, q, row) ? 1 : max(1, A.wsubs[q].n_chunks);
+}
 
 // Round-to-nearest-even of (neg ? -1 : 1) * (top * 2^128 + mag) to binary64, from the
 // definition: the top 53 significant bits, then half-ulp and sticky bits.
@@ -434,6 +490,8 @@ inline EstArgs est_args(const EstPlanHdr& H, const unsigned char* pd, unsigned c
   a.tri_slots = tri_slots;
   a.tri_max_leaves = H.tri_max_leaves;
   a.tri_nch = H.tri_nch;
+  a.cyc = reinterpret_cast<const CycSub*>(pd + H.off_cyc);
+  a.n_cyc = H.n_cyc;
   return a;
 }
 
@@ -442,6 +500,7 @@ cudaError_t launch_estimate(const EstArgs& a, const EstPlanHdr& H, double* est, 
 cudaError_t launch_estimate_wide(const EstArgs& a, double* est, int64_t* wide_rows, cudaStream_t st);
 cudaError_t launch_estimate_tri(const EstArgs& a, cudaStream_t st);
 cudaError_t launch_estimate_star(const EstArgs& a, cudaStream_t st);
+cudaError_t launch_estimate_cycle(const EstArgs& a, cudaStream_t st);
 cudaError_t launch_cross_ranks(const uint32_t* abs, const int32_t* perm, int32_t k, int32_t d, int32_t w,
                                const int32_t* edge_id, int32_t* ranks, cudaStream_t st);
 cudaError_t launch_cross_ranks_multi(const uint32_t* abs, const int32_t* perm, int32_t n_tables, const int32_t* k,

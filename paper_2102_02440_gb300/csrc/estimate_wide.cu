@@ -331,7 +331,7 @@ __device__ __forceinline__ int wide_mods_for(double B) {
 // star row on its lattice, |S| times the largest bound of its terms T_a(S \ {a}).
 __device__ __forceinline__ double wide_row_bound(const EstArgs& A, uint32_t e) {
   const uint32_t qr = A.wide_queue[4 + e];
-  const int nch = wide_row_units(A, qr / uint32_t(A.d));
+  const int nch = wide_row_units(A, qr / uint32_t(A.d), int(qr % uint32_t(A.d)));
   const uint64_t* part = A.wide_part + int64_t(A.wide_row_start[e]) * (kWideMods + 1);
   if (uint32_t(A.wide_units[A.wide_row_start[e]]) & kUnitLattice)
     return __dmul_ru(__longlong_as_double((long long)part[kWideMods]),
@@ -339,6 +339,33 @@ __device__ __forceinline__ double wide_row_bound(const EstArgs& A, uint32_t e) {
   double B = 0.0;
   for (int c = 0; c < nch; c++) B = __dadd_ru(B, __longlong_as_double((long long)part[int64_t(c) * (kWideMods + 1) + kWideMods]));
   return B;
+}
+
+// A cycle row's value modulo prime j, or (j = kWideMods) its magnitude rounded upwards.
+__device__ __forceinline__ uint64_t cyc_unit(const CycRow& cr, int j) {
+  uint32_t v[kCycMaxLimbs];
+  cyc_value(cr, v);
+  const bool neg = (v[kCycMaxLimbs - 1] >> 31) != 0;
+  if (neg) {  // magnitude
+    uint64_t c = 1;
+#pragma unroll
+    for (int l = 0; l < kCycMaxLimbs; l++) {
+      c += uint64_t(~v[l]);
+      v[l] = uint32_t(c);
+      c >>= 32;
+    }
+  }
+  if (j == kWideMods) {
+    double B = 0.0;
+#pragma unroll
+    for (int l = kCycMaxLimbs - 1; l >= 0; l--) B = __dadd_ru(__dmul_ru(B, 0x1p32), double(v[l]));
+    return uint64_t(__double_as_longlong(B));
+  }
+  const ModArith ar{wide_p(j), wide_c(j)};
+  uint64_t r = 0;
+#pragma unroll
+  for (int l = kCycMaxLimbs - 1; l >= 0; l--) r = ar.add(ar.mul(r, uint64_t(1) << 32), v[l]);
+  return neg && r ? ar.p - r : r;
 }
 
 // Persistent over the units of the queued rows: pass 0 computes every unit's bound, pass 1
@@ -369,7 +396,9 @@ __global__ void __launch_bounds__(kWideThreads, kWideCtasPerSm) k_estimate_wide(
     const int row = int(qr % uint32_t(A.d));
     const EstSub sb = A.wsubs[q];
     uint64_t result = 0;
-    if (sb.single) {  // never queued (an exact count); kept for completeness
+    if (uint32_t(ent) & kUnitCycle) {  // the value is known: its residue, or its magnitude as the bound
+      if (threadIdx.x == 0) result = cyc_unit(*cyc_taken(A, q, row), j);
+    } else if (sb.single) {  // never queued (an exact count); kept for completeness
       const int64_t n = *sb.sv;
       result = j < kWideMods ? ModArith{wide_p(j), wide_c(j)}.from(n)
                              : uint64_t(__double_as_longlong(fabs(double(n))));
@@ -723,7 +752,7 @@ __global__ void __launch_bounds__(kWideFinThreads) k_estimate_wide_finalize(cons
         const int K = wide_mods_for(wide_row_bound(A, uint32_t(slot)));
         if (K == 0) atomicOr(&bad, 1);
         // the row's residues: its units' residues summed modulo each prime
-        const int nch = wide_row_units(A, q);
+        const int nch = wide_row_units(A, q, tid);
         const uint64_t* part = A.wide_part + int64_t(A.wide_row_start[slot]) * (kWideMods + 1);
         uint64_t r[kWideMods];
         for (int j = 0; j < K; j++) {
