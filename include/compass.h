@@ -129,7 +129,8 @@ typedef struct {
   int32_t tile_rows;      /* rows per tile (multiple of 128, <= 16384)                              */
   int32_t dedupe;         /* -1 auto, 0 off, 1 aggregate equal keys of a tile before hashing        */
   int32_t ctas_per_sm;    /* CTAs per SM the grid is sized for                                      */
-  int32_t aggregate;      /* batched build only: -1 auto (tables of >= 2^18 rows), 0 off, 1 every
+  int32_t aggregate;      /* batched build only: -1 auto (tables of >= 2^18 rows, and of >= 2^13 rows
+                             when the count array has at most 16 slots per row), 0 off, 1 every
                              table: aggregate each key column's survivors per distinct key before
                              hashing (needs dedupe; same counters)                                  */
   int32_t unique;         /* batched build only: 0 or 1 on, -1 off: key columns declared
@@ -184,8 +185,8 @@ cmp_status cmp_sketch_build(const cmp_table* table, int32_t d, int32_t w, const 
  * that is not declared unique are first counted per distinct key, then each distinct key
  * is hashed once per (sketch, row) with its count as the multiplier.  The count array
  * covers the column's declared domain (CMP_COL_DOMAIN, at most 2^27 values), else the
- * power of two at or above min(rows, 2^27), indexed by the key modulo its size; the
- * counting pass also finds the surviving keys' range.  The update is linear and the
+ * power of two at or above min(rows, 2^27) (for fewer rows up to eight times that, at most
+ * 2^20), indexed by the key modulo its size; the counting pass also finds the surviving keys' range.  The update is linear and the
  * counters wrap exactly, so the result is bit-identical to one update per tuple; a column
  * whose surviving keys span more values than its array (or leave its declared domain)
  * falls back to the per-row path in the same build.  Key columns declared unique

@@ -249,6 +249,15 @@ cmp_status cmp_sketch_build(const cmp_table* table, int32_t d, int32_t w, const 
 // most this many slots (a column whose key range is wider keeps the per-row path).
 constexpr int64_t kAggMinRows = int64_t(1) << 18;
 constexpr int64_t kAggMaxCap = int64_t(1) << 27;
+// Smaller tables (from kAggSmallRows rows) are aggregated too when the count array has at most
+// kAggSmallFill slots per row: clearing and scanning 16 slots costs less than hashing one row
+// for a single sketch row does.
+constexpr int64_t kAggSmallRows = int64_t(1) << 13;
+constexpr int64_t kAggSmallFill = 16;
+// Without a declared domain the keys' range is unknown: at least kAggMinCap slots (4 MB, or
+// kAggSmallFill per row for smaller tables), so that keys sparser than the rows still fit.
+constexpr int64_t kAggMinCap = int64_t(1) << 20;
+constexpr int64_t kCountChunksPerCta = 12;
 
 // Unique-key kernel: shared-memory budget of a slab's counters (room is left on the SM for
 // a CTA of the counting pass), rows per tile.
@@ -280,10 +289,11 @@ struct BuildPlanParts {
   std::vector<CountItem> cnt_items;
   int64_t cnt_total_chunks = 0;
   int32_t cnt_grid = 0;
+  int64_t cnt_filtered = 0;  // first chunk of the tables with predicates or a sample
   int64_t cnt_split = 0;  // > 0: two launches, the tables with presence columns first
   int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the second counting launch
   int32_t cnt_grid_b = 0;
-  int64_t hash_total_chunks = 0;
+  int64_t hash_total_chunks = 0, hash_chunk = kHashChunkMax;
   int32_t hash_max_pairs = 1, hash_grid = 0;
   std::vector<std::vector<int32_t>> col_agg;  // [table][col] AggCol index or -1
   size_t bytes = 0, ws_bytes = 0;
@@ -325,11 +335,11 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   P->surv_by.assign(n_tables, kSurvRow);
   P->col_agg.assign(n_tables, std::vector<int32_t>(CMP_MAX_COLS, -1));
   P->aggs.clear();
-  size_t ws = al256(16 * size_t(n_tables) * CMP_MAX_SKETCHES + 32);  // stats + chunk counters (upper bound)
+  size_t ws = al256(16 * size_t(n_tables) * CMP_MAX_SKETCHES + 40);  // stats + chunk counters (upper bound)
   for (int32_t t = 0; t < n_tables; t++) {
     const cmp_table& tb = tables[t];
     const bool agg_on = tb.n_sketches > 0 && tb.n_rows > 0 && s.dedupe &&
-                        (agg_mode == 1 || (agg_mode == -1 && tb.n_rows >= kAggMinRows));
+                        (agg_mode == 1 || (agg_mode == -1 && tb.n_rows >= kAggSmallRows));
     const bool unfiltered = tb.n_preds == 0 && !(tb.sample_rate > 0.0 && tb.sample_rate < 1.0);
     for (int k = 0; k < tb.n_sketches; k++) {
       const int c = tb.key_col[k];
@@ -366,9 +376,11 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
         a.mask = ~0ull;
       } else {  // a power of two, slot = key mod cap
         a.cap = int64_t(next_pow2_64(uint64_t(std::min<int64_t>(tb.n_rows, kAggMaxCap))));
+        a.cap = std::max(a.cap, std::min(kAggMinCap, a.cap * (kAggSmallFill / 2)));
         a.base = 0;
         a.mask = uint64_t(a.cap) - 1;
       }
+      if (agg_mode == -1 && tb.n_rows < kAggMinRows && a.cap > kAggSmallFill * tb.n_rows) continue;  // per row
       P->col_agg[t][c] = int32_t(P->aggs.size());
       P->aggs.push_back(a);
     }
@@ -504,13 +516,19 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
       raw.push_back(r);
     }
   }
-  // hashing pass of the aggregated columns: chunks of kHashChunk count-array slots
+  // hashing pass of the aggregated columns: chunks of hash_chunk count-array slots
   P->hash_total_chunks = 0;
   P->hash_max_pairs = 1;
+  {
+    int64_t slots = 0;
+    for (const AggCol& ac : P->aggs) slots += ac.kind == kAggPresence ? 0 : ac.cap;
+    const int64_t want = slots / (int64_t(sm_count()) * 2 * kHashChunksPerCta) / 512 * 512;
+    P->hash_chunk = std::max(kHashChunkMin, std::min(kHashChunkMax, want));
+  }
   for (AggCol& ac : P->aggs) {
     ac.hash_chunk0 = P->hash_total_chunks;
     if (ac.kind == kAggPresence) continue;  // hashed by the dense kernel
-    P->hash_total_chunks += (ac.cap + kHashChunk - 1) / kHashChunk;
+    P->hash_total_chunks += (ac.cap + P->hash_chunk - 1) / P->hash_chunk;
     int32_t np = 0;
     for (int32_t k = 0; k < tables[ac.table].n_sketches; k++) np += tables[ac.table].key_col[k] == ac.col ? d : 0;
     P->hash_max_pairs = std::max(P->hash_max_pairs, np);
@@ -608,7 +626,8 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   // long), at most 64 tiles; a persistent grid of about one resident wave takes the chunks
   // in order
   // (tables with a presence column first, so that a split pass completes every bitmap in its
-  // first launch)
+  // first launch; then the other tables without a selection, then those with one: each kind is
+  // counted by its own kernel)
   P->cnt_items.clear();
   P->cnt_total_chunks = 0;
   auto has_presence = [&](int32_t t) {
@@ -617,24 +636,6 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
     return false;
   };
   int64_t presence_chunks = 0;
-  for (int pass = 0; pass < 2; pass++)
-  for (int32_t t = 0; t < n_tables; t++) {
-    int ncol = 0;
-    for (int32_t c = 0; c < CMP_MAX_COLS; c++) ncol += P->col_agg[t][c] >= 0;
-    if (!ncol || has_presence(t) != (pass == 0)) continue;
-    CountItem ci;
-    ci.table = t;
-    ci.pad = 0;
-    const int64_t unit = 4 * int64_t(R);
-    const int64_t want = tables[t].n_rows / (int64_t(sm_count()) * 2 * 16);
-    ci.chunk_rows = unit * std::max<int64_t>(1, std::min<int64_t>(16, want / unit));
-    ci.chunk_begin = P->cnt_total_chunks;
-    ci.n_chunks = (tables[t].n_rows + ci.chunk_rows - 1) / ci.chunk_rows;
-    P->cnt_total_chunks += ci.n_chunks;
-    if (pass == 0) presence_chunks += ci.n_chunks;
-    P->cnt_items.push_back(ci);
-  }
-  P->cnt_grid = 0;  // set below, once the unique-key items are known
   // hot-key caches of the counting pass: the most aggregated columns of any table (at most
   // 4 cached), a power-of-two number of slots per column in about 64 KB
   {
@@ -650,6 +651,43 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
     while (P->cache_cols && h > 256 && size_t(h) * 8 * size_t(P->cache_cols) > (size_t(64) << 10)) h >>= 1;
     P->cache_slots = P->cache_cols ? h : 256;
   }
+  // A CTA that moves to another table writes its cache out and clears it, and with many tables
+  // it moves after every chunk: chunks are long enough that about kCountChunksPerCta of them
+  // make up a CTA's share of each kind, and a cache has at most one slot per 16 rows of a
+  // chunk.  (Chunks of 16,384 rows with caches of 8192 slots sent 103 M of 160 M keys of 96
+  // tables to L2.)
+  auto count_kind = [&](int32_t t) {  // 0 presence columns, 1 no selection, 2 a selection, -1 not counted
+    int ncol = 0;
+    for (int32_t c = 0; c < CMP_MAX_COLS; c++) ncol += P->col_agg[t][c] >= 0;
+    if (!ncol) return -1;
+    const bool filtered = tables[t].n_preds > 0 || sample_keep_of(tables[t].sample_rate) != 0;
+    return has_presence(t) ? 0 : (filtered ? 2 : 1);
+  };
+  int64_t kind_rows[3] = {0, 0, 0};
+  for (int32_t t = 0; t < n_tables; t++)
+    if (count_kind(t) >= 0) kind_rows[count_kind(t)] += tables[t].n_rows;
+  const int64_t cnt_ctas = int64_t(sm_count()) * (P->uitems.empty() ? 2 : 1);
+  for (int pass = 0; pass < 3; pass++) {
+  if (pass == 2) P->cnt_filtered = P->cnt_total_chunks;
+  for (int32_t t = 0; t < n_tables; t++) {
+    if (count_kind(t) != pass) continue;
+    CountItem ci;
+    ci.table = t;
+    const int64_t unit = 4 * int64_t(R);
+    const int64_t want = std::max(tables[t].n_rows / (int64_t(sm_count()) * 2 * 16),
+                                  kind_rows[pass] / (cnt_ctas * kCountChunksPerCta));
+    ci.chunk_rows = unit * std::max<int64_t>(1, std::min<int64_t>(16, want / unit));
+    ci.cache_slots = P->cache_slots;
+    while (ci.cache_slots > 256 && 16 * int64_t(ci.cache_slots) > std::min(ci.chunk_rows, tables[t].n_rows))
+      ci.cache_slots >>= 1;
+    ci.chunk_begin = P->cnt_total_chunks;
+    ci.n_chunks = (tables[t].n_rows + ci.chunk_rows - 1) / ci.chunk_rows;
+    P->cnt_total_chunks += ci.n_chunks;
+    if (pass == 0) presence_chunks += ci.n_chunks;
+    P->cnt_items.push_back(ci);
+  }
+  }
+  P->cnt_grid = 0;  // set below, once the unique-key items are known
   // counting pass: 512-thread CTAs, two per SM; one per SM when the unique-key kernel runs
   // beside it
   P->cnt_grid = int32_t(std::min<int64_t>(P->cnt_total_chunks, int64_t(sm_count()) * (P->uitems.empty() ? 2 : 1)));
@@ -780,12 +818,14 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.cnt_total_chunks = P.cnt_total_chunks;
   h.cnt_grid = P.cnt_grid;
   h.cnt_split = P.cnt_split;
+  h.cnt_filtered = P.cnt_filtered;
   h.cnt_grid_b = P.cnt_grid_b;
   h.d_cut = P.d_cut;
   h.cnt_threads = 512;
   h.cnt_cache_slots = P.cache_slots;
   h.cnt_cache_cols = P.cache_cols;
   h.hash_total_chunks = P.hash_total_chunks;
+  h.hash_chunk = P.hash_chunk;
   h.hash_max_pairs = P.hash_max_pairs;
   h.hash_grid = P.hash_grid;
   h.ws_bytes = int64_t(P.ws_bytes);
@@ -861,12 +901,13 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     a.n_cnt_items = int32_t(h.n_cnt_items);
     a.cnt_total_chunks = h.cnt_total_chunks;
     a.hash_total_chunks = h.hash_total_chunks;
+    a.hash_chunk = h.hash_chunk;
     a.hash_max_pairs = h.hash_max_pairs;
     a.cnt_cache_slots = h.cnt_cache_slots;
     a.cnt_cache_cols = h.cnt_cache_cols;
     // the (max, min) key ranges start from zero (decoding as an empty column), so do the
     // chunk counters of the counting and hashing passes after them
-    if (cudaMemsetAsync(ws_dev, 0, 16 * size_t(h.n_agg) + 24, cs) != cudaSuccess) return CMP_ECUDA;
+    if (cudaMemsetAsync(ws_dev, 0, 16 * size_t(h.n_agg) + 40, cs) != cudaSuccess) return CMP_ECUDA;
     if (launch_agg_zero(a, cs) != cudaSuccess) return CMP_ECUDA;
   }
   const int32_t hash_grid = h.n_agg > 0 ? h.hash_grid : 0;
@@ -875,9 +916,10 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     // the tables with presence columns, then the others with the dense kernel beside them
     // (its programmatic dependent: one CTA of each per SM, a memory-bound scan beside an
     // integer-bound walk; every bitmap is complete before the second launch starts)
-    if (launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid, 0, 0, h.cnt_split, cs) != cudaSuccess ||
+    if (launch_count_rows(a, h.cnt_grid, 0, 0, h.cnt_split, cs) != cudaSuccess ||
         launch_presence_check(a, cs) != cudaSuccess ||
-        launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid_b, 2, h.cnt_split, h.cnt_total_chunks, cs) !=
+        launch_count_rows(a, h.cnt_grid_b, 2, h.cnt_split, h.cnt_filtered, cs) != cudaSuccess ||
+        launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid_b, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
             cudaSuccess)
       return CMP_ECUDA;
     // the dense kernel: its share beside the counting launch, then the rest with 512 threads
@@ -894,7 +936,9 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     return launch_agg_hash(a, hash_grid, cs) == cudaSuccess ? CMP_OK : CMP_ECUDA;
   }
   if (h.n_agg > 0 &&
-      launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid, 0, 0, h.cnt_total_chunks, cs) != cudaSuccess)
+      (launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
+           cudaSuccess ||
+       launch_count_rows(a, h.cnt_grid, 0, 0, h.cnt_filtered, cs) != cudaSuccess))
     return CMP_ECUDA;
   // the unique-key kernel right after the counting pass, as its programmatic dependent:
   // one CTA of each per SM, the two overlap (memory-bound scan, integer-bound hashing)
@@ -920,10 +964,12 @@ extern "C" cmp_status cmp_build_plan_stats(const void* plan_host, cmp_build_plan
   info->n_unique_items = h.n_uitems;
   info->row_grid = h.shape.grid;
   info->ws_bytes = h.ws_bytes;
-  // zeroing; clearing (+ counting when it has chunks) and hashing of the counted keys; the
-  // unique-key kernel; the row kernel
-  // unique-key kernel; the row kernel; the presence check and the dense kernel
-  info->launches = 1 + (h.n_agg > 0 ? 1 + (h.cnt_grid > 0 ? 1 : 0) + (h.cnt_split > 0 ? 1 : 0) + (h.hash_grid > 0 ? 1 : 0) : 0) +
+  // zeroing; clearing, counting (tables without and with a selection, presence columns apart in
+  // a split pass; each when it has chunks) and hashing of the counted keys; the unique-key
+  // kernel; the row kernel; the presence check and the dense kernel
+  const int32_t count_launches = (h.cnt_split > 0 ? 1 : 0) + (h.cnt_filtered > h.cnt_split ? 1 : 0) +
+                                 (h.cnt_total_chunks > h.cnt_filtered ? 1 : 0);
+  info->launches = 1 + (h.n_agg > 0 ? 1 + count_launches + (h.hash_grid > 0 ? 1 : 0) : 0) +
                    (h.n_uitems > 0 && h.u_grid > 0 ? 1 : 0) + (h.shape.grid > 0 ? 1 : 0) +
                    (h.n_ditems > 0 && h.d_grid > 0 ? 2 : 0) +  // the presence check and the dense kernel
                    (h.n_ditems > 0 && h.d_grid > 0 && h.cnt_split > 0 && h.d_cut < 1024 ? 1 : 0);  // its second part

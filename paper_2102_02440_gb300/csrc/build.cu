@@ -356,8 +356,8 @@ __host__ __device__ inline size_t agg_count_surv_entries(int32_t tile_rows, int3
   return tile_rows > 16 * threads ? size_t(tile_rows) : size_t(16) * threads;
 }
 
-// Counting pass of key aggregation.  Persistent CTAs take chunks of whole tiles of a
-// table's rows (CountItem.chunk_rows) in order from an atomic counter.  For every surviving
+// Counting pass of key aggregation over tables with predicates or a row sample (the others:
+// k_count_rows, build_count.cu).  Persistent CTAs take chunks of whole tiles of a table's rows (CountItem.chunk_rows) in order from an atomic counter.  For every surviving
 // row and every aggregated key column of the table, the key's slot (key - base) & mask gets
 // one count (a presence column: its bit is set; a bit found set already makes the column
 // inactive): in the CTA's two-way set-associative shared-memory cache when a way of its set
@@ -382,11 +382,11 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
   __shared__ uint32_t akeys;  // the current table's aggregated key columns (bit c: column c)
   __shared__ long long next_chunk;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
-  const int R = A.tile_rows, H = A.cnt_cache_slots, n_cache = A.cnt_cache_cols;
-  const int hshift = 32 - (31 - __clz(H));  // H is a power of two >= 256
+  const int R = A.tile_rows, n_cache = A.cnt_cache_cols;
+  int H = 0, hshift = 0;  // the current table's cache slots per column, a power of two >= 256 (block-uniform)
   uint32_t* ckey = reinterpret_cast<uint32_t*>(smem);  // [n_cache][H] cached slot index
-  uint32_t* ccnt = ckey + size_t(H) * n_cache;          // [n_cache][H] its count so far
-  unsigned char* sp = smem + align16(sizeof(uint32_t) * 2 * size_t(H) * n_cache);
+  uint32_t* ccnt = ckey;                                // [n_cache][H] its count so far
+  unsigned char* sp = smem + align16(sizeof(uint32_t) * 2 * size_t(A.cnt_cache_slots) * n_cache);
   uint16_t* surv = reinterpret_cast<uint16_t*>(sp);
   sp += align16(sizeof(uint16_t) * agg_count_surv_entries(R, T));
   int32_t* sint = reinterpret_cast<int32_t*>(sp);
@@ -496,6 +496,9 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
     const DevTable* tb = A.tables + ci.table;
     if (it != item) {  // a new table: flush the caches, then set them up for its columns
       if (item >= 0) flush();
+      H = ci.cache_slots;
+      hshift = 32 - (31 - __clz(H));
+      ccnt = ckey + size_t(H) * n_cache;
       if (tid == 0) {
         int n = 0;
         uint32_t keys = 0;
@@ -532,56 +535,7 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
     const int64_t n_rows = tb->n_rows;
     const int64_t r_begin = (c - ci.chunk_begin) * ci.chunk_rows, r_end = min(n_rows, r_begin + ci.chunk_rows);
     const bool vec = tb->vec_ok != 0;
-    if (!tb->filtered) {
-      if (tid == 0 && r_end > r_begin)
-        atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), (unsigned long long)(r_end - r_begin));
-      // every row survives: eight consecutive rows per thread and step, two 16-byte loads
-      // for int32 keys
-      for (int a = 0; a < nac; a++) {
-        const void* kbase = tb->col[acol[a]];
-        const int32_t kdt = tb->dtype[acol[a]];
-        int64_t mn = INT64_MAX, mx = INT64_MIN;
-        bool ok = true;
-        for (int64_t r = r_begin + 8 * int64_t(tid); r < r_end; r += 8 * int64_t(T)) {
-          if (lane == 0) {  // this warp's 256 rows of the next step (this column, else the next one's first)
-            const int64_t rw = r + 8 * int64_t(T);
-            if (rw < r_end) {
-              prefetch_rows(tb, 1u << acol[a], rw, min(r_end, rw + 256), 0, 1);
-            } else if (a + 1 < nac) {
-              const int64_t rn = r_begin + (rw - r_begin) % (8 * int64_t(T));
-              prefetch_rows(tb, 1u << acol[a + 1], rn, min(r_end, rn + 256), 0, 1);
-            }
-          }
-          int64_t v[8];
-          int nv = int(min(int64_t(8), r_end - r));
-          if (vec && nv == 8) {
-            if (kdt == CMP_I32) {
-              const int4* p = reinterpret_cast<const int4*>(reinterpret_cast<const int32_t*>(kbase) + r);
-              const int4 u = __ldg(p), q = __ldg(p + 1);
-              v[0] = u.x, v[1] = u.y, v[2] = u.z, v[3] = u.w, v[4] = q.x, v[5] = q.y, v[6] = q.z, v[7] = q.w;
-            } else {
-              const longlong2* p = reinterpret_cast<const longlong2*>(reinterpret_cast<const long long*>(kbase) + r);
-#pragma unroll
-              for (int h = 0; h < 4; h++) {
-                const longlong2 u = __ldg(p + h);
-                v[2 * h] = u.x, v[2 * h + 1] = u.y;
-              }
-            }
-          } else {
-            for (int q = 0; q < 8; q++) v[q] = q < nv ? load1(kbase, kdt, r + q) : 0;
-          }
-#pragma unroll
-          for (int q = 0; q < 8; q++)
-            if (q < nv) {
-              mn = min(mn, v[q]);
-              mx = max(mx, v[q]);
-              ok &= count_key(a, v[q]);
-            }
-        }
-        if (!ok) mn = INT64_MIN, mx = INT64_MAX;  // outside the declared domain: out of range
-        fold_range(a, mn, mx);
-      }
-    } else if (vec && !tb->sample_keep && tb->n_preds >= 1 && tb->n_preds <= 2 && nac <= 2 &&
+    if (vec && !tb->sample_keep && tb->n_preds >= 1 && tb->n_preds <= 2 && nac <= 2 &&
                tb->dtype[tb->pred[0].col] == CMP_I32 && tb->dtype[tb->pred[tb->n_preds - 1].col] == CMP_I32 &&
                akind[0] == kAggCount && akind[nac - 1] == kAggCount) {
       // Warp-autonomous scan in three stages (no block barrier inside the chunk).  Warp w
@@ -854,14 +808,14 @@ __global__ void __launch_bounds__(kHashThreads) k_agg_hash(const __grid_constant
       cur = ai;
       __syncthreads();
     }
-    const int64_t s0 = (c - ac.hash_chunk0) * kHashChunk, range = s_range;
+    const int64_t s0 = (c - ac.hash_chunk0) * A.hash_chunk, range = s_range;
     if (active && s0 < range) {
       const int32_t* cnts = reinterpret_cast<const int32_t*>(A.ws + ac.off);
       const int64_t kmin = s_kmin;
       // key kmin + j sits in slot (kmin - base + j) & mask
       const uint64_t off0 = uint64_t(kmin) - uint64_t(ac.base), mask = ac.mask;
       const int np = n_pairs;
-      const int64_t per = kHashChunk / nw;  // a multiple of 32
+      const int64_t per = A.hash_chunk / nw;  // a multiple of 32
       const int64_t ws0 = min(range, s0 + warp * per), ws1 = min(range, ws0 + per);
       // the first n entries of the warp's buffer, lane l taking l, l + 32, ...: kHashPer
       // independent hash chains per lane sharing every parameter load

@@ -264,10 +264,13 @@ struct AggCol {
   int64_t off;   // byte offset of the count array (presence: the bitmap) in the workspace
   int64_t base;  // key of slot 0 (declared domain) or 0
   uint64_t mask; // ~0 (declared domain) or cap - 1 (power of two)
-  int64_t hash_chunk0;  // first chunk of this column in the hashing pass (kHashChunk slots each)
+  int64_t hash_chunk0;  // first chunk of this column in the hashing pass (hash_chunk slots each)
   int32_t kind, pad;    // kAggCount / kAggPresence
 };
-constexpr int64_t kHashChunk = 16384;
+// Slots per chunk of the hashing pass: a multiple of 512 (32 per warp), as large as leaves about
+// kHashChunksPerCta chunks per resident CTA, so that the last chunks end together.
+constexpr int64_t kHashChunkMin = 1024, kHashChunkMax = 16384;
+constexpr int64_t kHashChunksPerCta = 16;
 // Presence bitmaps are walked in runs of kDenseRun keys (8 words); a bitmap holds whole runs.
 constexpr int64_t kDenseRun = 256;
 __host__ __device__ inline int64_t presence_words(int64_t cap) { return (cap + kDenseRun - 1) / kDenseRun * (kDenseRun / 32); }
@@ -329,7 +332,7 @@ struct BuildItem {
 // chunk_begin + n_chunks) of the pass's global chunk sequence (chunk_rows each), handed out
 // to the persistent CTAs in order by an atomic counter.
 struct CountItem {
-  int32_t table, pad;
+  int32_t table, cache_slots;  // cache_slots: hot-key cache slots per column (a power of two)
   int64_t chunk_begin, n_chunks;
   int64_t chunk_rows;  // a multiple of 4 tiles
 };
@@ -367,7 +370,7 @@ struct BuildArgs {
   int64_t cnt_chunk_begin, cnt_chunk_end;     // its chunks
   int32_t cnt_cache_slots, cnt_cache_cols;  // counting pass: hot-key cache slots per column, columns cached
   int64_t cnt_total_chunks;
-  int64_t hash_total_chunks;  // hashing pass of the aggregated columns
+  int64_t hash_total_chunks, hash_chunk;  // hashing pass of the aggregated columns: chunks, slots of one
   int32_t hash_max_pairs;     // most (sketch, row) pairs on one aggregated column
   // unique-key kernel
   const UniqSlab* uslab;
@@ -400,7 +403,7 @@ struct BuildPlanHdr {
   int32_t cnt_grid, cnt_threads;
   int64_t ws_bytes;
   int32_t cnt_cache_slots, cnt_cache_cols;
-  int64_t hash_total_chunks;
+  int64_t hash_total_chunks, hash_chunk;
   int32_t hash_max_pairs, hash_grid;
   int64_t n_uslab, off_uslab, n_uitems, off_uitems, off_u_cta;  // unique-key kernel
   int32_t u_grid, u_pack16, u_words, u_tile_rows;
@@ -412,8 +415,10 @@ struct BuildPlanHdr {
   // split pass: the dense kernel walks the first d_cut / 1024 of each item's runs beside the
   // second counting launch, the rest after it with 512 threads (d_cut = 1024: all beside)
   int32_t cnt_grid_b, d_cut;
+  // chunks from here on are of tables with predicates or a sample (k_agg_count; before: k_count_rows)
+  int64_t cnt_filtered;
 };
-constexpr int32_t kBuildPlanVersion = 10;
+constexpr int32_t kBuildPlanVersion = 11;
 struct ZeroSpan {
   void* ptr;
   int64_t bytes;
@@ -450,6 +455,8 @@ cudaError_t launch_agg_zero(const BuildArgs& a, cudaStream_t st);
 cudaError_t launch_presence_check(const BuildArgs& a, cudaStream_t st);
 cudaError_t launch_agg_count(const BuildArgs& a, int32_t tile_rows, int32_t cnt_threads, int32_t cnt_grid,
                              int32_t work_slot, int64_t chunk_begin, int64_t chunk_end, cudaStream_t st);
+cudaError_t launch_count_rows(const BuildArgs& a, int32_t grid, int32_t work_slot, int64_t chunk_begin,
+                              int64_t chunk_end, cudaStream_t st);
 size_t uniq_smem_bytes(int32_t words, int32_t tile_rows);
 cudaError_t launch_uniq(const BuildArgs& a, int32_t grid, int32_t threads, int32_t tile_rows, cudaStream_t st);
 cudaError_t launch_zero_spans(const ZeroSpan* spans_dev, int32_t n, cudaStream_t st);
