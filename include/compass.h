@@ -186,9 +186,9 @@ cmp_status cmp_sketch_build(const cmp_table* table, int32_t d, int32_t w, const 
  * is hashed once per (sketch, row) with its count as the multiplier.  The count array
  * covers the column's declared domain (CMP_COL_DOMAIN, at most 2^27 values), else the
  * power of two at or above min(rows, 2^27) (for fewer rows up to eight times that, at most
- * 2^20), indexed by the key modulo its size; the counting pass also finds the surviving keys' range.  The update is linear and the
- * counters wrap exactly, so the result is bit-identical to one update per tuple; a column
- * whose surviving keys span more values than its array (or leave its declared domain)
+ * 2^20), indexed by the key modulo its size; the counting pass also finds the surviving
+ * keys' range.  The update is linear and the counters wrap exactly, so the result is
+ * bit-identical to one update per tuple; a column whose surviving keys span more values than its array (or leave its declared domain)
  * falls back to the per-row path in the same build.  Key columns declared unique
  * (CMP_COL_UNIQUE, cfg->unique) are hashed once per surviving row by a kernel that keeps
  * one or more (sketch, row) pairs' counters in shared memory: int32, or two 16-bit halves

@@ -517,12 +517,10 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
     }
   }
   // hashing pass of the aggregated columns: chunks of hash_chunk count-array slots
-  P->hash_total_chunks = 0;
-  P->hash_max_pairs = 1;
   {
     int64_t slots = 0;
     for (const AggCol& ac : P->aggs) slots += ac.kind == kAggPresence ? 0 : ac.cap;
-    const int64_t want = slots / (int64_t(sm_count()) * 2 * kHashChunksPerCta) / 512 * 512;
+    const int64_t want = slots / (int64_t(sm_count()) * 2) / 512 * 512;  // two CTAs per SM
     P->hash_chunk = std::max(kHashChunkMin, std::min(kHashChunkMax, want));
   }
   for (AggCol& ac : P->aggs) {
@@ -654,7 +652,7 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   // A CTA that moves to another table writes its cache out and clears it, and with many tables
   // it moves after every chunk: chunks are long enough that about kCountChunksPerCta of them
   // make up a CTA's share of each kind, and a cache has at most one slot per 16 rows of a
-  // chunk.  (Chunks of 16,384 rows with caches of 8192 slots sent 103 M of 160 M keys of 96
+  // chunk.  (Chunks of 16,384 rows with caches of 8192 slots sent 103 M of 162.5 M keys of 58
   // tables to L2.)
   auto count_kind = [&](int32_t t) {  // 0 presence columns, 1 no selection, 2 a selection, -1 not counted
     int ncol = 0;
@@ -819,13 +817,13 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.cnt_grid = P.cnt_grid;
   h.cnt_split = P.cnt_split;
   h.cnt_filtered = P.cnt_filtered;
+  h.hash_chunk = P.hash_chunk;
   h.cnt_grid_b = P.cnt_grid_b;
   h.d_cut = P.d_cut;
   h.cnt_threads = 512;
   h.cnt_cache_slots = P.cache_slots;
   h.cnt_cache_cols = P.cache_cols;
   h.hash_total_chunks = P.hash_total_chunks;
-  h.hash_chunk = P.hash_chunk;
   h.hash_max_pairs = P.hash_max_pairs;
   h.hash_grid = P.hash_grid;
   h.ws_bytes = int64_t(P.ws_bytes);

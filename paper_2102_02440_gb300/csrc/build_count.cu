@@ -6,13 +6,15 @@
 //
 // Bound by the shared-memory and L2 reductions of the keys (about one 32-key group per 50
 // cycles and SM), so the kernel keeps everything else out of their way: a column's
-// parameters and eight keys per thread in registers (113 instructions per key when the
-// descriptors were read from shared memory for each key, about 45 now), no selection code in
+// parameters and eight keys per thread in registers (131 instructions per
+// key when the descriptors were read from shared memory for each key, 49 now, caches and
+// flushes included), no selection code in
 // the kernel (its registers spilled, and with the whole SM's L1 given to shared memory a
 // spill is an L2 access), and the next chunk's rows bulk-prefetched into L2 while this chunk
 // is counted, since a chunk is only four steps long.
-// 81 M int32 keys of two fact tables (domains of 0.13 to 4 M): 592 us before, 259 us now; 160 M
-// keys of 96 tables without declared domains: 1158 us before, 859 us now.
+// 81 M int32 keys of two fact tables (domains of 0.13 to 4 M): 592 us before, 259 us now, the
+// unique-key kernel beside it both times; 165 M keys of 96 tables without declared domains (164
+// instructions per key before, 89 now): 1158 us before, for the 58 largest, 859 us now.
 #include <cuda_runtime.h>
 
 #include <algorithm>
