@@ -293,8 +293,9 @@ struct BuildPlanParts {
   int64_t cnt_split = 0;  // > 0: two launches, the tables with presence columns first
   int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the second counting launch
   int32_t cnt_grid_b = 0;
-  int64_t hash_total_chunks = 0, hash_chunk = kHashChunkMax;
-  int32_t hash_max_pairs = 1, hash_grid = 0;
+  int64_t hash_items = 0;
+  int32_t hash_private = 0;
+  int32_t hash_grid = 0;
   std::vector<std::vector<int32_t>> col_agg;  // [table][col] AggCol index or -1
   size_t bytes = 0, ws_bytes = 0;
   int32_t cache_slots = 256, cache_cols = 0;  // counting pass
@@ -516,22 +517,37 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
       raw.push_back(r);
     }
   }
-  // hashing pass of the aggregated columns: chunks of hash_chunk count-array slots
+  // Hashing pass of the aggregated columns.  A column's pairs are hashed in slabs whose
+  // counters fit a CTA's shared memory (wider rows: up to kHashMaxPairs, counters in global
+  // memory); a slab's slots are dealt to items in proportion to slots x pairs.  The kernel
+  // deals them to fewer when the keys' range turns out smaller than the count array.
   {
-    int64_t slots = 0;
-    for (const AggCol& ac : P->aggs) slots += ac.kind == kAggPresence ? 0 : ac.cap;
-    const int64_t want = slots / (int64_t(sm_count()) * 2) / 512 * 512;  // two CTAs per SM
-    P->hash_chunk = std::max(kHashChunkMin, std::min(kHashChunkMax, want));
+    auto pairs_of = [&](const AggCol& ac) {
+      int32_t np = 0;
+      for (int32_t k = 0; k < tables[ac.table].n_sketches; k++) np += tables[ac.table].key_col[k] == ac.col ? d : 0;
+      return np;
+    };
+    const int32_t fit = int32_t(kHashBudget / (4 * int64_t(w)));  // pairs whose counters fit
+    const int64_t items = fit > 0 ? kHashItems : kHashDirectItems;
+    double total = 0;
+    for (const AggCol& ac : P->aggs)
+      if (ac.kind != kAggPresence) total += double(ac.cap) * pairs_of(ac);
+    const int64_t ctas = int64_t(sm_count()) * 2;
+    const double per_item = std::max(1.0, total / double(ctas * items));
+    for (AggCol& ac : P->aggs) {
+      ac.hash_item0 = P->hash_items;
+      if (ac.kind == kAggPresence) continue;  // hashed by the dense kernel
+      const int32_t np = pairs_of(ac), most = std::min(kHashMaxPairs, fit > 0 ? fit : kHashMaxPairs);
+      ac.hash_slabs = (np + most - 1) / most;
+      ac.hash_pairs = (np + ac.hash_slabs - 1) / ac.hash_slabs;
+      const double want = double(ac.cap) * ac.hash_pairs / per_item;
+      const double steps = double((ac.cap + 3) / (kHashStep * kHashThreads / 32) + 1);  // one step at least
+      ac.hash_groups = int32_t(std::max(1.0, std::min({std::ceil(want), double(ctas * items), steps})));
+      P->hash_items += int64_t(ac.hash_slabs) * ac.hash_groups;
+      if (fit > 0) P->hash_private = std::max(P->hash_private, ac.hash_pairs * w);
+    }
+    P->hash_grid = int32_t(std::min<int64_t>(P->hash_items, ctas));
   }
-  for (AggCol& ac : P->aggs) {
-    ac.hash_chunk0 = P->hash_total_chunks;
-    if (ac.kind == kAggPresence) continue;  // hashed by the dense kernel
-    P->hash_total_chunks += (ac.cap + P->hash_chunk - 1) / P->hash_chunk;
-    int32_t np = 0;
-    for (int32_t k = 0; k < tables[ac.table].n_sketches; k++) np += tables[ac.table].key_col[k] == ac.col ? d : 0;
-    P->hash_max_pairs = std::max(P->hash_max_pairs, np);
-  }
-  P->hash_grid = int32_t(std::min<int64_t>(P->hash_total_chunks, int64_t(sm_count()) * 2));  // resident: 2 per SM
   // dense kernel: slabs of each presence column's pairs (as for the unique-key kernel);
   // each slab's domain split into items of whole runs, about equal work (keys x pairs) per
   // CTA, one CTA per SM; consecutive items of a CTA share a slab where they can
@@ -817,14 +833,13 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.cnt_grid = P.cnt_grid;
   h.cnt_split = P.cnt_split;
   h.cnt_filtered = P.cnt_filtered;
-  h.hash_chunk = P.hash_chunk;
+  h.hash_private = P.hash_private;
   h.cnt_grid_b = P.cnt_grid_b;
   h.d_cut = P.d_cut;
   h.cnt_threads = 512;
   h.cnt_cache_slots = P.cache_slots;
   h.cnt_cache_cols = P.cache_cols;
-  h.hash_total_chunks = P.hash_total_chunks;
-  h.hash_max_pairs = P.hash_max_pairs;
+  h.hash_items = P.hash_items;
   h.hash_grid = P.hash_grid;
   h.ws_bytes = int64_t(P.ws_bytes);
   h.total_bytes = int64_t(P.bytes);
@@ -898,9 +913,8 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     a.cnt_items = reinterpret_cast<const CountItem*>(dev + h.off_cnt_items);
     a.n_cnt_items = int32_t(h.n_cnt_items);
     a.cnt_total_chunks = h.cnt_total_chunks;
-    a.hash_total_chunks = h.hash_total_chunks;
-    a.hash_chunk = h.hash_chunk;
-    a.hash_max_pairs = h.hash_max_pairs;
+    a.hash_items = h.hash_items;
+    a.hash_private = h.hash_private;
     a.cnt_cache_slots = h.cnt_cache_slots;
     a.cnt_cache_cols = h.cnt_cache_cols;
     // the (max, min) key ranges start from zero (decoding as an empty column), so do the

@@ -148,16 +148,28 @@ __global__ void __launch_bounds__(1024) k_sketch_build(const __grid_constant__ B
   // Hash the first n_entries (field element, count) entries of mkey / mcnt for the pairs
   // of key column kc, or (no map) the keys of the tile's first n_entries survivors.  Two
   // entries per thread share every parameter load: two independent hash chains.
-  auto hash_pairs = [&](auto smallx, const KeyPow& k0, const KeyPow& k1, int32_t m0, int32_t m1, int pl_begin,
-                        int pl_end) {
-    constexpr bool SMALLX = decltype(smallx)::value;
+  auto hash_pairs = [&](auto form, uint64_t x0, uint64_t x1, int32_t m0, int32_t m1, int pl_begin, int pl_end) {
+    constexpr int F = decltype(form)::value;
+    constexpr bool SMALLX = F != kAnyKey;
+    KeyPow k0, k1;
+    if (!SMALLX) k0 = key_powers(x0), k1 = key_powers(x1);
     for (int j = pl_begin; j < pl_end; j++) {
       const int pp = plist[j];
       const PairParam q = prm[pp];
-      const uint32_t h0 = cw_bucket<POW2, SMALLX>(q, k0, uint32_t(w));
-      const uint32_t h1 = cw_bucket<POW2, SMALLX>(q, k1, uint32_t(w));
-      const int32_t v0 = cw_sign<SMALLX>(q, k0) * m0;
-      const int32_t v1 = cw_sign<SMALLX>(q, k1) * m1;
+      uint32_t h0, h1;
+      int32_t v0, v1;
+      if (SMALLX) {
+        h0 = sx_bucket<POW2, F>(q, uint32_t(x0), uint32_t(w));
+        h1 = sx_bucket<POW2, F>(q, uint32_t(x1), uint32_t(w));
+        v0 = sx_odd<F>(q, uint32_t(x0)) ? -m0 : m0;
+        v1 = sx_odd<F>(q, uint32_t(x1)) ? -m1 : m1;
+      } else {
+        const PairLimb l = pair_limbs(q);
+        h0 = cw_bucket<POW2>(q, l, k0, uint32_t(w));
+        h1 = cw_bucket<POW2>(q, l, k1, uint32_t(w));
+        v0 = cw_sign(q, l, k0) * m0;
+        v1 = cw_sign(q, l, k1) * m1;
+      }
       int32_t* row = (GLOBAL ? gcnt : cnt) + size_t(pp) * w;  // L2 counters, or the CTA's shared ones
       if (GLOBAL) {
         red_add(row + h0, v0);
@@ -183,13 +195,8 @@ __global__ void __launch_bounds__(1024) k_sketch_build(const __grid_constant__ B
         m0 = 1;
         if (e1 < n_entries) x1 = key_field(load1(kbase, kdt, r0 + (filtered ? surv[e1] : e1))), m1 = 1;
       }
-      const KeyPow k0 = key_powers(x0);
-      const KeyPow k1 = key_powers(x1);
-      // keys below 2^31 (every non-negative int32 key) have a zero high limb
-      if (__all_sync(__activemask(), (k0.x.hi | k1.x.hi) == 0))
-        hash_pairs(std::true_type{}, k0, k1, m0, m1, pl_begin, pl_end);
-      else
-        hash_pairs(std::false_type{}, k0, k1, m0, m1, pl_begin, pl_end);
+      // keys below 2^31 (every non-negative int32 key) take the small-key steps
+      with_form(key_form(x0 | x1), [&](auto form) { hash_pairs(form, x0, x1, m0, m1, pl_begin, pl_end); });
     }
   };
 
@@ -736,154 +743,254 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
 }
 
 // Hashing of the aggregated key columns: every nonzero (key, count) entry of a count array
-// is hashed once per (sketch, row) pair on that column, and count * xi is added to the
-// global counters.  Persistent CTAs take chunks of count-array slots in order from an
-// atomic counter; a CTA loads the pairs' parameters when its column changes.  Each warp
-// compacts the nonzero entries of its part of a chunk, 32 slots at a time, into a 96-entry
-// buffer and hashes 64 of them, two per lane, whenever it holds 64.
-constexpr int kHashThreads = 512;
+// is hashed once per (sketch, row) pair on that column, and count * xi is added to the pair's
+// counters.  Persistent CTAs take items (a slab of the column's pairs, a range of its slots) in
+// order from an atomic counter.  The slab's counters are kept in shared memory while a CTA's
+// items are of one slab and added to the global ones when it moves on (one by one, the
+// reductions take L2 about a cycle per slice), unless the entries are too few for that to pay
+// or the rows too wide.  Each warp reads 128 slots (four per lane) at a time, the next ones requested before
+// these are used, compacts the nonzero ones into its buffer and hashes 128 of them, four
+// independent chains per lane sharing every parameter read, whenever it holds 128; what is
+// left over stays in the buffer for the next item of the slab, so sparse counts still fill
+// their batches.  Bound by the integer ALU of the
+// hash arithmetic where the counters are private, by L2's reductions where not.
+// 64 M evaluations of dense counts (w 4096): 438 us with global reductions, 240 us now; 48 joins
+// of w 4096: 593 us for their 58 largest tables before, 429 us for all 96 now; a 100 M key
+// domain at w 65536 (global reductions): 766 us before, 490 us now.
 
-constexpr int kHashPer = 2;                    // entries per lane and batch: independent hash chains
-constexpr int kHashBatch = 32 * kHashPer;        // entries hashed at a time by a warp
-constexpr int kHashBuf = kHashBatch + 32;        // entries buffered per warp (31 carried over)
+constexpr int kHashBatch = 128;                  // entries hashed at a time by a warp
+constexpr int kHashBuf = kHashBatch + 128;       // entries buffered per warp (127 carried over)
+constexpr size_t kHashBufBytes = size_t(kHashThreads / 32) * kHashBuf * sizeof(uint2);
 
-size_t agg_hash_smem_bytes(int32_t max_pairs) {
-  return align16(sizeof(PairParam) * size_t(max_pairs)) + align16(sizeof(int32_t*) * size_t(max_pairs)) +
-         (kHashThreads / 32) * kHashBuf * (sizeof(unsigned long long) + sizeof(int32_t));
+// The first n <= 32 E entries (offset j, count) of a warp's buffer, lane l taking l, l + 32, ...:
+// E independent chains per lane.  Keys are kmin + j, all of form F.  cs: the slab's counters in
+// shared memory (a shared address; PRIV), else rows grow[p] in global memory.  Lanes past n add 0.
+template <bool POW2, bool PRIV, int F, int E>
+__device__ __forceinline__ void hash_batch(const PairParam* prm, int32_t* const* grow, uint32_t cs, int np, uint32_t w,
+                                           int64_t kmin, const uint2* buf, int n) {
+  constexpr bool SMALL = F != kAnyKey;
+  const int lane = threadIdx.x & 31;
+  int32_t m[E];
+  uint32_t x[E];
+  KeyPow k[SMALL ? 1 : E];
+#pragma unroll
+  for (int e = 0; e < E; e++) {
+    const int j = lane + 32 * e;
+    const uint2 v = j < n ? buf[j] : make_uint2(0, 0);
+    const uint32_t off = v.x;
+    m[e] = int32_t(v.y);
+    if (SMALL) x[e] = uint32_t(kmin) + off;
+    else k[SMALL ? 0 : e] = key_powers(key_field(kmin + int64_t(off)));
+  }
+  for (int p = 0; p < np; p++, cs += 4 * w) {
+    const PairParam q = prm[p];
+    int32_t* row = PRIV ? nullptr : grow[p];
+#pragma unroll
+    for (int e = 0; e < E; e++) {
+      const uint32_t h = SMALL ? sx_bucket<POW2, F>(q, x[e], w) : cw_bucket<POW2>(q, pair_limbs(q), k[SMALL ? 0 : e], w);
+      const uint32_t odd = SMALL ? sx_odd<F>(q, x[e]) : uint32_t(cw_sign_residue(q, pair_limbs(q), k[SMALL ? 0 : e])) & 1u;
+      const uint32_t v = odd * (0u - 2u * uint32_t(m[e])) + uint32_t(m[e]);  // one multiply-add
+      if (PRIV) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(cs + 4 * h), "r"(v) : "memory");
+      else if (m[e]) red_add(row + h, int32_t(v));
+    }
+  }
 }
 
 template <bool POW2>
-__global__ void __launch_bounds__(kHashThreads) k_agg_hash(const __grid_constant__ BuildArgs A) {
+__global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_constant__ BuildArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   // the presence-bitmap kernel, launched next as a programmatic dependent, reads nothing
   // this pass writes: let it start now
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  __shared__ long long next_chunk;
-  __shared__ int32_t n_pairs, active;
-  __shared__ long long s_kmin, s_range;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int mp = A.hash_max_pairs;
-  PairParam* prm = reinterpret_cast<PairParam*>(smem);
-  int32_t** prow = reinterpret_cast<int32_t**>(smem + align16(sizeof(PairParam) * size_t(mp)));
-  unsigned long long* bkey = reinterpret_cast<unsigned long long*>(reinterpret_cast<unsigned char*>(prow) +
-                                                                   align16(sizeof(int32_t*) * size_t(mp))) +
-                             kHashBuf * warp;
-  int32_t* bcnt = reinterpret_cast<int32_t*>(reinterpret_cast<unsigned long long*>(
-                      reinterpret_cast<unsigned char*>(prow) + align16(sizeof(int32_t*) * size_t(mp))) +
-                                             kHashBuf * nw) +
-                  kHashBuf * warp;
+  __shared__ PairParam prm[kHashMaxPairs];
+  __shared__ int32_t* grow[kHashMaxPairs];
+  __shared__ long long s_item, s_kmin, s_range;
+  __shared__ unsigned long long s_work;
+  __shared__ int32_t n_pairs;
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = T >> 5;
+  uint2* buf = reinterpret_cast<uint2*>(smem) + kHashBuf * warp;  // (offset, count)
+  int32_t* cs = reinterpret_cast<int32_t*>(smem + kHashBufBytes);  // [n_pairs][w]
+  const uint32_t cs32 = uint32_t(__cvta_generic_to_shared(cs));
   unsigned long long* work = reinterpret_cast<unsigned long long*>(A.ws) + 2 * int64_t(A.n_agg) + 1;
   const uint32_t w = uint32_t(A.w);
-  int cur = -1;  // block-uniform
-  for (;;) {
-    if (tid == 0) next_chunk = (long long)atomicAdd(work, 1ull);
+  for (int j = tid; j < A.hash_private; j += T) cs[j] = 0;
+  // block-uniform: the current column, its pairs, its items per slab, their slots; the current slab
+  int cur_ai = -1, cur_slab = -1, groups = 1, np_col = 0;
+  int64_t kmin = 0, range = 0, len = 0;
+  bool priv = false, open = false;  // the slab's counters are in shared memory; a slab is loaded
+  int nb = 0;                       // entries buffered: warp-uniform
+  auto batch = [&](int n) {         // one full batch, or the last entries of a slab
+    const int64_t k0 = s_kmin;
+    const int np = n_pairs;
+    const int64_t kend = k0 >= 0 && k0 < (1ll << 31) ? k0 + s_range : INT64_MAX;
+    auto run = [&](auto pv) {
+      constexpr bool PRIV = decltype(pv)::value;
+      if (kend <= (1ll << 29)) {
+        if (n > 64) hash_batch<POW2, PRIV, kSmall29, 4>(prm, grow, cs32, np, w, k0, buf, n);
+        else hash_batch<POW2, PRIV, kSmall29, 2>(prm, grow, cs32, np, w, k0, buf, n);
+      } else {  // (the powers of two keys fit the registers)
+        for (int i = 0; i < n; i += 64) {
+          if (kend <= (1ll << 31))
+            hash_batch<POW2, PRIV, kSmall31, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
+          else
+            hash_batch<POW2, PRIV, kAnyKey, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
+        }
+      }
+    };
+    if (priv) run(std::true_type{});
+    else run(std::false_type{});
+  };
+  auto finish = [&]() {  // the current slab (block-wide): its last entries, its counters
+    if (nb > 0) batch(nb);
+    nb = 0;
     __syncthreads();
-    const int64_t c = next_chunk;
-    if (c >= A.hash_total_chunks) break;
-    int ai = 0;
-    while (ai + 1 < A.n_agg && A.agg[ai + 1].hash_chunk0 <= c) ai++;
-    const AggCol ac = A.agg[ai];
-    const DevTable* tb = A.tables + ac.table;
-    if (ai != cur) {  // a new column: its pairs' parameters and counter rows
-      if (tid == 0) {
-        int64_t kmin = 0, range = 0;
-        active = agg_active(ac, ai, A.ws, &kmin, &range) ? 1 : 0;
-        s_kmin = kmin;
-        s_range = range;
-        int n = 0;
-        for (int s = 0; s < tb->n_sketches; s++)
-          if (tb->key_col[s] == ac.col) n += A.d;
-        n_pairs = n;
-      }
-      __syncthreads();
-      const int np = n_pairs;
-      for (int p = tid; p < np; p += blockDim.x) {
-        int s = 0, k = p / A.d;  // the k-th sketch on this column
-        for (;; s++)
-          if (tb->key_col[s] == ac.col && k-- == 0) break;
-        const int i = p % A.d;
-        prm[p] = make_pair_param(A.hash[size_t(tb->edge_id[s]) * A.d + i]);
-        prow[p] = tb->counters + (size_t(s) * A.d + i) * w;
-      }
-      cur = ai;
-      __syncthreads();
-    }
-    const int64_t s0 = (c - ac.hash_chunk0) * A.hash_chunk, range = s_range;
-    if (active && s0 < range) {
-      const int32_t* cnts = reinterpret_cast<const int32_t*>(A.ws + ac.off);
-      const int64_t kmin = s_kmin;
-      // key kmin + j sits in slot (kmin - base + j) & mask
-      const uint64_t off0 = uint64_t(kmin) - uint64_t(ac.base), mask = ac.mask;
-      const int np = n_pairs;
-      const int64_t per = A.hash_chunk / nw;  // a multiple of 32
-      const int64_t ws0 = min(range, s0 + warp * per), ws1 = min(range, ws0 + per);
-      // the first n entries of the warp's buffer, lane l taking l, l + 32, ...: kHashPer
-      // independent hash chains per lane sharing every parameter load
-      auto hash_batch = [&](int n) {
-        KeyPow k[kHashPer];
-        int32_t m[kHashPer];
-        uint32_t hi_or = 0;
-#pragma unroll
-        for (int e = 0; e < kHashPer; e++) {
-          const int j = lane + 32 * e;
-          m[e] = j < n ? bcnt[j] : 0;
-          k[e] = key_powers(j < n ? bkey[j] : 0);
-          hi_or |= k[e].x.hi;
-        }
-        auto run = [&](auto smallx) {
-          constexpr bool SX = decltype(smallx)::value;
-          for (int p = 0; p < np; p++) {
-            const PairParam q = prm[p];
-            int32_t* row = prow[p];
-#pragma unroll
-            for (int e = 0; e < kHashPer; e++) {
-              const uint32_t h = cw_bucket<POW2, SX>(q, k[e], w);
-              const int32_t v = cw_sign<SX>(q, k[e]) * m[e];
-              if (m[e]) red_add(row + h, v);
-            }
+    if (priv) {
+      if (w % 4 == 0) {
+        int4* c4 = reinterpret_cast<int4*>(cs);
+        const uint32_t w4 = w / 4;
+        for (int p = 0; p < n_pairs; p++)
+          for (uint32_t j = tid; j < w4; j += T) {
+            const int4 v = c4[p * w4 + j];
+            int32_t* g = grow[p] + 4 * j;
+            if (v.x) red_add(g, v.x);
+            if (v.y) red_add(g + 1, v.y);
+            if (v.z) red_add(g + 2, v.z);
+            if (v.w) red_add(g + 3, v.w);
+            c4[p * w4 + j] = make_int4(0, 0, 0, 0);
           }
-        };
-        if (__all_sync(0xffffffffu, hi_or == 0)) run(std::true_type{});
-        else run(std::false_type{});
-      };
-      int nb = 0;  // warp-uniform
-      for (int64_t sb = ws0; sb < ws1; sb += 32) {
-        const int64_t j = sb + lane;
-        const int32_t cnt = j < ws1 ? __ldg(cnts + ((off0 + uint64_t(j)) & mask)) : 0;
-        const unsigned nz = __ballot_sync(0xffffffffu, cnt != 0);
-        if (cnt != 0) {
-          const int pos = nb + __popc(nz & ((1u << lane) - 1u));
-          bkey[pos] = key_field(kmin + j);
-          bcnt[pos] = cnt;
+      } else {
+        for (int p = 0; p < n_pairs; p++)
+          for (uint32_t j = tid; j < w; j += T) {
+            const int32_t v = cs[p * w + j];
+            if (v) red_add(grow[p] + j, v);
+            cs[p * w + j] = 0;
+          }
+      }
+    }
+    __syncthreads();
+  };
+  // the work there is, slots in the key ranges x pairs, sets the length of an item
+  if (tid == 0) {
+    s_item = (long long)atomicAdd(work, 1ull);
+    s_work = 0;
+  }
+  __syncthreads();
+  for (int ai = tid; ai < A.n_agg; ai += T) {
+    int64_t k0, r;
+    if (A.agg[ai].kind == kAggCount && agg_active(A.agg[ai], ai, A.ws, &k0, &r))
+      atomicAdd(&s_work, (unsigned long long)r * (unsigned long long)(A.agg[ai].hash_slabs * A.agg[ai].hash_pairs));
+  }
+  __syncthreads();
+  const int64_t item_work = int64_t(s_work / (unsigned long long)(gridDim.x * kHashItems)) + 1;
+  const unsigned lt = (1u << lane) - 1u;
+  const int64_t step = kHashStep * nw;  // slots the CTA reads at a time
+  for (;;) {
+    __syncthreads();
+    const int64_t c = s_item;
+    if (c >= A.hash_items) break;
+    long long c_next = 0;
+    if (tid == 0) c_next = (long long)atomicAdd(work, 1ull);  // one item ahead
+    int ai = max(cur_ai, 0);                                  // items come in order
+    while (ai + 1 < A.n_agg && A.agg[ai + 1].hash_item0 <= c) ai++;
+    const AggCol& ac = A.agg[ai];
+    const DevTable* tb = A.tables + ac.table;
+    if (ai != cur_ai) {  // a new column: private counters or not, its items
+      if (open) finish();
+      open = false;
+      cur_ai = ai;
+      cur_slab = -1;
+      if (!agg_active(ac, ai, A.ws, &kmin, &range)) range = 0;
+      np_col = 0;
+      for (int s = 0; s < tb->n_sketches; s++)
+        if (tb->key_col[s] == ac.col) np_col += A.d;
+      // Writing a slab's counters out costs about two updates for each, so private ones want
+      // twice as many entries as buckets in an item (at most as many as survivors).
+      groups = int(max(int64_t(1), min(int64_t(ac.hash_groups), range * ac.hash_pairs / item_work)));
+      priv = A.hash_private > 0 && min(range, int64_t(*tb->survivors)) / groups >= 2 * int64_t(w);
+      if (!priv) {  // all pairs at once (as far as they fit), shorter items
+        const bool one = np_col <= kHashMaxPairs;
+        const int64_t most = one ? int64_t(ac.hash_groups) * ac.hash_slabs : ac.hash_groups;
+        groups = int(max(int64_t(1), min(most, range * min(np_col, kHashMaxPairs) * (kHashDirectItems / kHashItems) / item_work)));
+      }
+      len = ((range + 3 + groups - 1) / groups + step - 1) / step * step;
+    }
+    const bool one_slab = !priv && np_col <= kHashMaxPairs;
+    const int local = int(c - ac.hash_item0);
+    const int slab = one_slab ? 0 : local / ac.hash_groups, group = one_slab ? local : local % ac.hash_groups;
+    if (slab != cur_slab) {
+      if (open) finish();
+      open = false;
+      cur_slab = slab;
+    }
+    // key kmin + j sits in slot (kmin - base + j) & mask; a load takes four slots from a multiple
+    // of four (count arrays are whole int4 words, a masked one at least 8 slots): from j = -shift
+    const uint64_t off0 = uint64_t(kmin) - uint64_t(ac.base), mask = ac.mask;
+    const int64_t shift = int64_t(off0 & 3), begin = group * len - shift, end = min(range, begin + len);
+    if (group < groups && begin < end) {
+      if (!open) {
+        const int p0 = slab * ac.hash_pairs, np = one_slab ? np_col : min(np_col - p0, ac.hash_pairs);
+        if (tid < np) {
+          int s = 0, k = (p0 + tid) / A.d;  // the k-th sketch on this column
+          for (;; s++)
+            if (tb->key_col[s] == ac.col && k-- == 0) break;
+          const int i = (p0 + tid) % A.d;
+          prm[tid] = make_pair_param(A.hash[size_t(tb->edge_id[s]) * A.d + i]);
+          grow[tid] = tb->counters + (size_t(s) * A.d + i) * w;
         }
-        nb += __popc(nz);
+        if (tid == 0) {
+          n_pairs = np;
+          s_kmin = kmin;
+          s_range = range;
+        }
+        open = true;
+        __syncthreads();
+      }
+      const int32_t* cnts = reinterpret_cast<const int32_t*>(A.ws + ac.off);
+      const int64_t j0 = begin + kHashStep * warp + 4 * lane;
+      auto load = [&](int64_t j) {
+        return j < end ? __ldg(reinterpret_cast<const int4*>(cnts + ((off0 + uint64_t(j)) & mask))) : make_int4(0, 0, 0, 0);
+      };
+      int4 next = load(j0);
+      for (int64_t j = j0; j - 4 * lane < end; j += step) {  // warp-uniform
+        const int4 cur4 = next;
+        next = load(j + step);
+        int32_t cv[4] = {cur4.x, cur4.y, cur4.z, cur4.w};
+        const int64_t jw = j - 4 * lane;
+        if (jw < 0 || jw + kHashStep > range) {  // (warp-uniform: the ends of the key range)
+#pragma unroll
+          for (int q = 0; q < 4; q++)
+            if (j + q < 0 || j + q >= range) cv[q] = 0;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+          const unsigned nz = __ballot_sync(0xffffffffu, cv[q] != 0);
+          if (cv[q] != 0) buf[nb + __popc(nz & lt)] = make_uint2(uint32_t(j) + q, uint32_t(cv[q]));
+          nb += __popc(nz);
+        }
         __syncwarp();
         if (nb >= kHashBatch) {
-          hash_batch(kHashBatch);
+          batch(kHashBatch);
           __syncwarp();
-          if (lane < nb - kHashBatch) {  // keep the overflow at the front
-            bkey[lane] = bkey[kHashBatch + lane];
-            bcnt[lane] = bcnt[kHashBatch + lane];
-          }
+          for (int i = lane; i < nb - kHashBatch; i += 32) buf[i] = buf[kHashBatch + i];  // the overflow to the front
           nb -= kHashBatch;
           __syncwarp();
         }
       }
-      if (nb > 0) hash_batch(nb);
     }
-    __syncthreads();  // next_chunk and the parameters are rewritten next
+    __syncthreads();  // every thread has read s_item
+    if (tid == 0) s_item = c_next;
   }
+  if (open) finish();
 }
 
 cudaError_t launch_agg_hash(const BuildArgs& a, int32_t grid, cudaStream_t st) {
   if (a.n_agg <= 0 || grid <= 0) return cudaSuccess;
-  const size_t smem = agg_hash_smem_bytes(a.hash_max_pairs);
   const bool pow2 = (a.w & (a.w - 1)) == 0;
-  cudaError_t e = pow2 ? cudaFuncSetAttribute(k_agg_hash<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))
-                       : cudaFuncSetAttribute(k_agg_hash<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  const size_t smem = kHashBufBytes + sizeof(int32_t) * size_t(a.hash_private);
+  auto k = pow2 ? k_agg_hash<true> : k_agg_hash<false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
-  if (pow2) k_agg_hash<true><<<unsigned(grid), kHashThreads, smem, st>>>(a);
-  else k_agg_hash<false><<<unsigned(grid), kHashThreads, smem, st>>>(a);
+  k<<<unsigned(grid), kHashThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 

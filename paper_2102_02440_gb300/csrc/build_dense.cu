@@ -52,12 +52,13 @@ struct Diff {
 
 // The state at field element x0 (< p) for the pair's parameters; D3 is returned apart.
 __device__ __forceinline__ Diff diff_at(const PairParam& q, uint64_t x0, uint64_t* D3) {
+  const PairLimb l = pair_limbs(q);
   uint64_t v[4];
 #pragma unroll
   for (int j = 0; j < 4; j++) {
     uint64_t x = x0 + uint64_t(j);
     x = x >= kP61 ? x - kP61 : x;
-    v[j] = cw_sign_residue<false>(q, key_powers(x));
+    v[j] = cw_sign_residue(q, l, key_powers(x));
   }
   const uint64_t d01 = sub_mod(v[1], v[0]), d12 = sub_mod(v[2], v[1]), d23 = sub_mod(v[3], v[2]);
   const uint64_t e0 = sub_mod(d12, d01), e1 = sub_mod(d23, d12);
@@ -66,7 +67,7 @@ __device__ __forceinline__ Diff diff_at(const PairParam& q, uint64_t x0, uint64_
   s.P = v[0];
   s.D1 = d01;
   s.D2 = e0;
-  s.B = cw_bucket_residue<false>(q, key_powers(x0));
+  s.B = cw_bucket_residue(q, l, key_powers(x0));
   return s;
 }
 
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(THREADS, 512 / THREADS) k_dense_hash(const __g
       }
       for (int p = 0; p < n_pairs; p++) {
         const PairParam q = prm[p];
-        const uint64_t a_step = q.a_lo | (uint64_t(q.a_hi) << 31);
+        const uint64_t a_step = q.a;
         int32_t* g = grow[p];
         uint32_t* c = PACK16 ? cs : cs + size_t(p) * w;
         Diff st[kRuns];

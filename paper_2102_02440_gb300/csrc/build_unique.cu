@@ -38,6 +38,7 @@ template <bool PACK16, bool POW2>
 __global__ void __launch_bounds__(kUniqThreads, 2) k_uniq_hash(const __grid_constant__ BuildArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ PairParam prm[kUniqMaxPairs];
+  __shared__ PairLimb lim;  // packed: of the slab's one pair, split once and not per key
   __shared__ int32_t* grow[kUniqMaxPairs];
   const int tid = threadIdx.x, T = blockDim.x;
   const uint32_t w = uint32_t(A.w);
@@ -82,6 +83,7 @@ __global__ void __launch_bounds__(kUniqThreads, 2) k_uniq_hash(const __grid_cons
         const int pair = sl.pair[tid];
         const int s = pair / A.d, i = pair % A.d;
         prm[tid] = make_pair_param(A.hash[size_t(tb->edge_id[s]) * A.d + i]);
+        if (PACK16) lim = pair_limbs(prm[tid]);
         grow[tid] = tb->counters + size_t(pair) * w;
       }
       cur = it.slab;
@@ -95,40 +97,49 @@ __global__ void __launch_bounds__(kUniqThreads, 2) k_uniq_hash(const __grid_cons
     int64_t my_surv = 0;
     // KPT keys per thread and step: independent hash chains sharing the parameters; their
     // counter updates are issued before any of their results is examined
-    // (packed slabs hold one pair: the Horner form, no shared powers; int32 slabs share the
-    // key's powers x^2, x^3 among their pairs)
+    // (keys of 2^31 and more: packed slabs hold one pair and take the Horner form, int32 slabs
+    // share the key's powers x^2, x^3 among their pairs)
     auto hashk = [&](const int64_t (&k)[KPT], int nv) {
-      KeyPow kp[KPT];
-      KeyX kx[KPT];
-      uint32_t hi_or = 0;
-      // keys in [0, p) are their own residue (every non-negative key below 2^61)
-      bool in_field = true;
+      // keys in [0, 2^31) are their own residue and take the small-key steps
+      uint64_t bits = 0;
 #pragma unroll
-      for (int q = 0; q < KPT; q++) in_field &= uint64_t(k[q]) < kP61;
-      in_field = __all_sync(__activemask(), in_field);
+      for (int q = 0; q < KPT; q++) bits |= uint64_t(k[q]);
+      // (a third copy of the packed loop spilled, and its single pair feels a second vote)
+      const int kf = !PACK16 ? key_form(bits) : __all_sync(__activemask(), (bits >> 31) == 0) ? kSmall31 : kAnyKey;
+      with_form<!PACK16>(kf, [&](auto form) {
+        constexpr int F = decltype(form)::value;
+        constexpr bool SX = F != kAnyKey;
+        KeyPow kp[KPT];
+        KeyX kx[KPT];
+        // keys in [0, p) are their own residue: reducing them took the one pair of a packed slab
+        // 5% longer
+        bool in_field = true;
 #pragma unroll
-      for (int q = 0; q < KPT; q++) {
-        const uint64_t x = in_field ? uint64_t(k[q]) : key_field(k[q]);
-        if (PACK16) kx[q] = key_x(x);
-        else kp[q] = key_powers(x);
-        hi_or |= PACK16 ? kx[q].hi : kp[q].x.hi;
-      }
-      auto run = [&](auto smallx) {
-        constexpr bool SX = decltype(smallx)::value;
+        for (int q = 0; q < KPT; q++) in_field &= uint64_t(k[q]) < kP61;
+        if (!SX) in_field = __all_sync(__activemask(), in_field);
+#pragma unroll
+        for (int q = 0; q < KPT; q++) {
+          if (SX) continue;
+          const uint64_t x = in_field ? uint64_t(k[q]) : key_field(k[q]);
+          if (PACK16) kx[q] = key_x(x);
+          else kp[q] = key_powers(x);
+        }
         for (int p = 0; p < n_pairs; p++) {
           const PairParam prm_p = prm[p];
-          const uint64_t c2 = prm_p.c2_lo | (uint64_t(prm_p.c2_hi) << 31);
-          const uint64_t c1 = prm_p.c1_lo | (uint64_t(prm_p.c1_hi) << 31);
+          const PairLimb lim_p = PACK16 && !SX ? lim : pair_limbs(prm_p);
           uint32_t h[KPT];
           int sg[KPT];
 #pragma unroll
           for (int q = 0; q < KPT; q++) {
-            if (PACK16) {
-              h[q] = cw_bucket_h<POW2, SX>(prm_p, kx[q], w, A.m31, A.m4);
-              sg[q] = cw_sign_h<SX>(prm_p, kx[q], c2, c1, A.m31, A.m4);
+            if (SX) {
+              h[q] = sx_bucket<POW2, F>(prm_p, uint32_t(k[q]), w);
+              sg[q] = 1 - 2 * int(sx_odd<F>(prm_p, uint32_t(k[q])));
+            } else if (PACK16) {
+              h[q] = cw_bucket_h<POW2>(prm_p, lim_p, kx[q], w);
+              sg[q] = cw_sign_h(prm_p, lim_p, kx[q]);
             } else {
-              h[q] = cw_bucket<POW2, SX>(prm_p, kp[q], w);
-              sg[q] = cw_sign<SX>(prm_p, kp[q]);
+              h[q] = cw_bucket<POW2>(prm_p, lim_p, kp[q], w);
+              sg[q] = cw_sign(prm_p, lim_p, kp[q]);
             }
           }
           if (PACK16) {
@@ -150,9 +161,7 @@ __global__ void __launch_bounds__(kUniqThreads, 2) k_uniq_hash(const __grid_cons
               if (q < nv) red_add_shared(c + h[q], sg[q]);
           }
         }
-      };
-      if (__all_sync(__activemask(), hi_or == 0)) run(std::true_type{});
-      else run(std::false_type{});
+      });
     };
     for (int64_t r0 = it.row_begin; r0 < it.row_end; r0 += R) {
       const int rows_in_tile = int(min(int64_t(R), it.row_end - r0));
@@ -217,8 +226,6 @@ static cudaError_t launch_uniq_t(const BuildArgs& a, int32_t grid, int32_t threa
   if (e != cudaSuccess) return e;
   BuildArgs b = a;
   b.tile_rows = tile_rows;
-  b.m31 = 1u << 31;
-  b.m4 = 4;
   // programmatic dependent launch: may start while the previous kernel on the stream runs,
   // once that kernel allows it (the counting pass does, at its start)
   cudaLaunchConfig_t cfg = {};

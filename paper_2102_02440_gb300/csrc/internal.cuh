@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "compass.h"
 
 namespace cmpk {
@@ -46,25 +48,101 @@ __device__ __forceinline__ uint64_t mulmod61(Limb a, Limb b) {
   return canon61(fold61(s));
 }
 
-// Hash parameters of one (edge, row) pre-split into limbs (48 bytes, 16-aligned).
+// Hash parameters of one (edge, row), 16-aligned for shared-memory reads.
 struct __align__(16) PairParam {
-  uint32_t a_lo, a_hi, c1_lo, c1_hi, c2_lo, c2_hi, c3_lo, c3_hi;
-  uint64_t b, c0;
+  uint64_t a, b, c0, c1, c2, c3;
 };
 
-__host__ __device__ inline PairParam make_pair_param(const cmp_hash& h) {
-  PairParam q;
-  q.a_lo = uint32_t(h.a) & kM31;
-  q.a_hi = uint32_t(h.a >> 31);
-  q.c1_lo = uint32_t(h.c1) & kM31;
-  q.c1_hi = uint32_t(h.c1 >> 31);
-  q.c2_lo = uint32_t(h.c2) & kM31;
-  q.c2_hi = uint32_t(h.c2 >> 31);
-  q.c3_lo = uint32_t(h.c3) & kM31;
-  q.c3_hi = uint32_t(h.c3 >> 31);
-  q.b = h.b;
-  q.c0 = h.c0;
-  return q;
+__host__ __device__ inline PairParam make_pair_param(const cmp_hash& h) { return {h.a, h.b, h.c0, h.c1, h.c2, h.c3}; }
+
+// Their coefficients in limbs, for the any-key forms.
+struct __align__(16) PairLimb {
+  Limb a, c1, c2, c3;
+};
+__device__ __forceinline__ PairLimb pair_limbs(const PairParam& q) {
+  return {limb(q.a), limb(q.c1), limb(q.c2), limb(q.c3)};
+}
+
+// ---- Small keys: Horner steps of two multiplications, in two forms, kSmall29 for keys below
+// 2^29 and kSmall31 for keys below 2^31 (every non-negative int32 key).
+// sx_step: a value congruent to y x + c (mod p), below 2^64 - 8, for any y < 2^64 and c < 2^61.
+// With y = yh 2^32 + yl and u = yh x, u 2^32 = (u >> 29) 2^61 + (u mod 2^29) 2^32 and 2^61 = 1:
+//   y x + c = yl x + c + (u >> 29) + (u mod 2^29) 2^32,
+// at most 2^63 + 2^61 + 2^34 + 2^61; the sum of one step is the next one's y as it is.  For x <
+// 2^29, u >> 29 is the high word of yh (8 x), and u mod 2^29 the low word over 8.
+// Bound by the integer ALU (64 lanes per cycle and SM, half the issue rate), so what counts is
+// additions, shifts and masks; the carries are written out because the compiler's 64-bit sums
+// took more of them.  Bucket and sign of a key, in registers: 389 G/s with every step's result
+// folded below 2^61 + 8 (59 instructions), 430 G/s (kSmall31, 45), 550 G/s (kSmall29, 38).
+enum KeyForm { kSmall29, kSmall31, kAnyKey };
+template <int FORM>
+__device__ __forceinline__ uint64_t sx_step(uint64_t y, uint32_t x, uint64_t c) {
+  uint64_t s;
+  if (FORM == kSmall29)
+    asm("{\n\t.reg .u64 u, v;\n\t.reg .u32 yl, yh, ul, uh, vl, vh;\n\t"
+        "mov.b64 {yl, yh}, %1;\n\t"
+        "mul.wide.u32 u, yh, %4;\n\t"
+        "mad.wide.u32 v, yl, %2, %3;\n\t"
+        "mov.b64 {ul, uh}, u;\n\t"
+        "mov.b64 {vl, vh}, v;\n\t"
+        "shr.u32 ul, ul, 3;\n\t"
+        "add.cc.u32 vl, vl, uh;\n\t"
+        "addc.u32 vh, vh, ul;\n\t"
+        "mov.b64 %0, {vl, vh};\n\t}"
+        : "=l"(s)
+        : "l"(y), "r"(x), "l"(c), "r"(x << 3));
+  else
+    asm("{\n\t.reg .u64 u, v;\n\t.reg .u32 yl, yh, ul, uh, vl, vh, t, m, h;\n\t"
+        "mov.b64 {yl, yh}, %1;\n\t"
+        "mul.wide.u32 u, yh, %2;\n\t"
+        "mad.wide.u32 v, yl, %2, %3;\n\t"
+        "mov.b64 {ul, uh}, u;\n\t"
+        "mov.b64 {vl, vh}, v;\n\t"
+        "shf.r.clamp.b32 t, ul, uh, 29;\n\t"
+        "and.b32 m, ul, 0x1fffffff;\n\t"
+        "shr.u32 h, uh, 29;\n\t"
+        "add.u32 m, m, h;\n\t"
+        "add.cc.u32 vl, vl, t;\n\t"
+        "addc.u32 vh, vh, m;\n\t"
+        "mov.b64 %0, {vl, vh};\n\t}"
+        : "=l"(s)
+        : "l"(y), "r"(x), "l"(c));
+  return s;
+}
+// How often p goes into s < 2^64 - 8: s = q 2^61 + r = q p + (q + r), and q + r < 2p.  The
+// residue is then s - k p = (s + k) mod 2^61.
+__device__ __forceinline__ uint32_t sx_floor(uint64_t s) { return uint32_t((s + (s >> 61) + 1) >> 61); }
+
+// Bucket ((a x + b) mod p) mod w of a small key (w a power of two divides 2^61).
+template <bool POW2, int FORM>
+__device__ __forceinline__ uint32_t sx_bucket(const PairParam& q, uint32_t x, uint32_t w) {
+  const uint64_t s = sx_step<FORM>(q.a, x, q.b);
+  const uint32_t k = sx_floor(s);
+  if (POW2) return (uint32_t(s) + k) & (w - 1);
+  return uint32_t(((s + k) & kP61) % w);
+}
+// Parity of (((c3 x + c2) x + c1) x + c0) mod p of a small key: 1 where the sign is -1.
+template <int FORM>
+__device__ __forceinline__ uint32_t sx_odd(const PairParam& q, uint32_t x) {
+  uint64_t y = sx_step<FORM>(q.c3, x, q.c2);
+  y = sx_step<FORM>(y, x, q.c1);
+  y = sx_step<FORM>(y, x, q.c0);
+  return (uint32_t(y) ^ sx_floor(y)) & 1u;  // p is odd
+}
+// The form every lane's keys fit, given the bits set in any of this lane's (active lanes only).
+__device__ __forceinline__ int key_form(uint64_t bits) {
+  const unsigned m = __activemask();
+  if (__all_sync(m, (bits >> 29) == 0)) return kSmall29;
+  return __all_sync(m, (bits >> 31) == 0) ? kSmall31 : kAnyKey;
+}
+// f(integral constant of the form); SMALL29: it may be kSmall29.
+template <bool SMALL29 = true, typename F>
+__device__ __forceinline__ void with_form(int form, F&& f) {
+  if constexpr (SMALL29) {
+    if (form == kSmall29) return f(std::integral_constant<int, kSmall29>{});
+  }
+  if (form == kSmall31) f(std::integral_constant<int, kSmall31>{});
+  else f(std::integral_constant<int, kAnyKey>{});
 }
 
 // Powers of the key, shared by every (sketch, row) that hashes the same key.
@@ -83,19 +161,17 @@ __device__ __forceinline__ KeyPow key_powers(uint64_t x) {
 
 // Bucket: ((a x + b) mod p) mod w.  Sum bound: t0 + (t1>>30) + ((t1&M30)<<31) + 2 t2 + b
 // < 2^62 + 2^32 + 3 * 2^61 < 2^64.
-// SMALLX: the caller guarantees x < 2^31 (k.x.hi == 0), so the products with x.hi, which
-// are zero, are left out (same value, fewer multiplies).
-template <bool SMALLX = false>
-__device__ __forceinline__ uint64_t cw_bucket_residue(const PairParam& q, const KeyPow& k) {
-  const uint64_t t0 = uint64_t(q.a_lo) * k.x.lo;
-  const uint64_t t1 = SMALLX ? uint64_t(q.a_hi) * k.x.lo : uint64_t(q.a_lo) * k.x.hi + uint64_t(q.a_hi) * k.x.lo;
-  const uint64_t t2 = SMALLX ? 0 : uint64_t(q.a_hi) * k.x.hi;
+__device__ __forceinline__ uint64_t cw_bucket_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+  const Limb a = l.a;
+  const uint64_t t0 = uint64_t(a.lo) * k.x.lo;
+  const uint64_t t1 = uint64_t(a.lo) * k.x.hi + uint64_t(a.hi) * k.x.lo;
+  const uint64_t t2 = uint64_t(a.hi) * k.x.hi;
   const uint64_t s = t0 + (t1 >> 30) + ((t1 & kM30) << 31) + 2 * t2 + q.b;
   return canon61(fold61(s));
 }
-template <bool POW2, bool SMALLX = false>
-__device__ __forceinline__ uint32_t cw_bucket(const PairParam& q, const KeyPow& k, uint32_t w) {
-  const uint64_t r = cw_bucket_residue<SMALLX>(q, k);
+template <bool POW2>
+__device__ __forceinline__ uint32_t cw_bucket(const PairParam& q, const PairLimb& l, const KeyPow& k, uint32_t w) {
+  const uint64_t r = cw_bucket_residue(q, l, k);
   if (POW2) return uint32_t(r) & (w - 1);
   return uint32_t(r % w);
 }
@@ -103,20 +179,17 @@ __device__ __forceinline__ uint32_t cw_bucket(const PairParam& q, const KeyPow& 
 // Sign: parity of (c3 x^3 + c2 x^2 + c1 x + c0) mod p, as +1 / -1.  The three products
 // are summed by limb position: S0 < 3 * 2^62, S1 < 6 * 2^61, S2 < 3 * 2^60, and
 // fold(S0) + (S1>>30) + ((S1&M30)<<31) + 2 S2 + c0 < 6 * 2^61 + 2^35 < 2^64.
-template <bool SMALLX = false>
-__device__ __forceinline__ uint64_t cw_sign_residue(const PairParam& q, const KeyPow& k) {
-  const uint64_t S0 = uint64_t(q.c1_lo) * k.x.lo + uint64_t(q.c2_lo) * k.x2.lo + uint64_t(q.c3_lo) * k.x3.lo;
-  const uint64_t S1 = (SMALLX ? 0 : uint64_t(q.c1_lo) * k.x.hi) + uint64_t(q.c1_hi) * k.x.lo +
-                      uint64_t(q.c2_lo) * k.x2.hi + uint64_t(q.c2_hi) * k.x2.lo + uint64_t(q.c3_lo) * k.x3.hi +
-                      uint64_t(q.c3_hi) * k.x3.lo;
-  const uint64_t S2 = (SMALLX ? 0 : uint64_t(q.c1_hi) * k.x.hi) + uint64_t(q.c2_hi) * k.x2.hi +
-                      uint64_t(q.c3_hi) * k.x3.hi;
+__device__ __forceinline__ uint64_t cw_sign_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+  const Limb c1 = l.c1, c2 = l.c2, c3 = l.c3;
+  const uint64_t S0 = uint64_t(c1.lo) * k.x.lo + uint64_t(c2.lo) * k.x2.lo + uint64_t(c3.lo) * k.x3.lo;
+  const uint64_t S1 = uint64_t(c1.lo) * k.x.hi + uint64_t(c1.hi) * k.x.lo + uint64_t(c2.lo) * k.x2.hi +
+                      uint64_t(c2.hi) * k.x2.lo + uint64_t(c3.lo) * k.x3.hi + uint64_t(c3.hi) * k.x3.lo;
+  const uint64_t S2 = uint64_t(c1.hi) * k.x.hi + uint64_t(c2.hi) * k.x2.hi + uint64_t(c3.hi) * k.x3.hi;
   const uint64_t v = fold61(S0) + (S1 >> 30) + ((S1 & kM30) << 31) + 2 * S2 + q.c0;
   return canon61(fold61(v));
 }
-template <bool SMALLX = false>
-__device__ __forceinline__ int cw_sign(const PairParam& q, const KeyPow& k) {
-  return 1 - 2 * int(cw_sign_residue<SMALLX>(q, k) & 1);
+__device__ __forceinline__ int cw_sign(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+  return 1 - 2 * int(cw_sign_residue(q, l, k) & 1);
 }
 
 // ---- Horner form (one (sketch, row) pair per key: no powers to share).  The same two
@@ -130,32 +203,14 @@ __device__ __forceinline__ KeyX key_x(uint64_t x) {
   return {uint32_t(x) & kM31, uint32_t(x >> 31), uint32_t(x >> 30) & ~1u};
 }
 
-// y x + c folded once, for y < 2^61 + 8 given as (ylo < 2^31, yhi <= 2^30), x < p, c < 2^61.
+// y x + c folded once, for y < 2^61 + 8 (ylo < 2^31, yhi <= 2^30), x < p, c < 2^61.
 // y x = ylo xlo + (ylo xhi + yhi xlo) 2^31 + yhi xhi 2^62 and 2^62 = 2, 2^61 = 1 (mod p), so with
 // t1 = ylo xhi + yhi xlo (< 2^62 + 2^31):
 //   y x + c = ylo xlo + yhi (2 xhi) + c + (t1 >> 30) + (t1 & (2^30-1)) 2^31   (mod p),
 // a sum below 2^62 + 2^61 + 2^61 + 2^33 + 2^61 < 2^64; one fold leaves it below 2^61 + 5.
-// SMALLX: x < 2^31 (xhi = 0), the products with xhi are zero and left out.
-template <bool SMALLX>
-__device__ __forceinline__ uint64_t mul_add_fold(uint32_t ylo, uint32_t yhi, const KeyX& x, uint64_t c) {
-  const uint64_t t1 = SMALLX ? uint64_t(yhi) * x.lo : uint64_t(ylo) * x.hi + uint64_t(yhi) * x.lo;
-  const uint64_t s = uint64_t(ylo) * x.lo + (SMALLX ? 0 : uint64_t(yhi) * x.hi2) + c + (t1 >> 30) +
-                     ((t1 & kM30) << 31);
-  return fold61(s);
-}
-
-// The same step for x < 2^31 (xhi = 0) with every product, shift and add on the multiply
-// pipe: with t1 = yhi xlo (< 2^61: yhi <= 2^30) split as t1hi 2^32 + t1lo,
-//   t1 2^31 = t1hi 2^63 + t1lo 2^31 = 4 t1hi + t1lo 2^31   (mod p, 2^63 = 4 2^61),
-// so y x + c = ylo xlo + c + t1lo 2^31 + 4 t1hi (mod p), a sum below 2^62 + 2^61 + 2^63 +
-// 2^31 < 2^64, folded once.  m31 = 2^31 and m4 = 4 come in as run-time values so that the
-// compiler keeps them as multiplications.
-__device__ __forceinline__ uint64_t mul_add_fold_sx(uint32_t ylo, uint32_t yhi, uint32_t xlo, uint64_t c,
-                                                    uint32_t m31, uint32_t m4) {
-  const uint64_t t1 = uint64_t(yhi) * xlo;
-  uint64_t s = uint64_t(ylo) * xlo + c;
-  s += uint64_t(uint32_t(t1)) * m31;
-  s += uint64_t(uint32_t(t1 >> 32)) * m4;
+__device__ __forceinline__ uint64_t mul_add_fold(Limb l, const KeyX& x, uint64_t c) {
+  const uint64_t t1 = uint64_t(l.lo) * x.hi + uint64_t(l.hi) * x.lo;
+  const uint64_t s = uint64_t(l.lo) * x.lo + uint64_t(l.hi) * x.hi2 + c + (t1 >> 30) + ((t1 & kM30) << 31);
   return fold61(s);
 }
 
@@ -164,30 +219,19 @@ __device__ __forceinline__ uint32_t ge_p(uint64_t y) { return uint32_t((y + 1) >
 
 // Bucket ((a x + b) mod p) mod w; the same value as cw_bucket.  For w a power of two (w <=
 // 2^31 divides 2^61), y - p = y + 1 (mod w).
-template <bool POW2, bool SMALLX>
-__device__ __forceinline__ uint32_t cw_bucket_h(const PairParam& q, const KeyX& x, uint32_t w, uint32_t m31 = 0,
-                                                uint32_t m4 = 0) {
-  const uint64_t y = SMALLX ? mul_add_fold_sx(q.a_lo, q.a_hi, x.lo, q.b, m31, m4)
-                            : mul_add_fold<false>(q.a_lo, q.a_hi, x, q.b);
+template <bool POW2>
+__device__ __forceinline__ uint32_t cw_bucket_h(const PairParam& q, const PairLimb& l, const KeyX& x, uint32_t w) {
+  const uint64_t y = mul_add_fold(l.a, x, q.b);
   if (POW2) return (uint32_t(y) + ge_p(y)) & (w - 1);
   return uint32_t((ge_p(y) ? y - kP61 : y) % w);
 }
 
 // Sign: parity of ((c3 x + c2) x + c1) x + c0 mod p, as +1 / -1; the same value as cw_sign.
 // The residue of the last y is y - p when y >= p, whose parity is flipped (p is odd).
-template <bool SMALLX>
-__device__ __forceinline__ int cw_sign_h(const PairParam& q, const KeyX& x, uint64_t c2, uint64_t c1,
-                                         uint32_t m31 = 0, uint32_t m4 = 0) {
-  uint64_t y;
-  if (SMALLX) {
-    y = mul_add_fold_sx(q.c3_lo, q.c3_hi, x.lo, c2, m31, m4);
-    y = mul_add_fold_sx(uint32_t(y) & kM31, uint32_t(y >> 31), x.lo, c1, m31, m4);
-    y = mul_add_fold_sx(uint32_t(y) & kM31, uint32_t(y >> 31), x.lo, q.c0, m31, m4);
-  } else {
-    y = mul_add_fold<false>(q.c3_lo, q.c3_hi, x, c2);
-    y = mul_add_fold<false>(uint32_t(y) & kM31, uint32_t(y >> 31), x, c1);
-    y = mul_add_fold<false>(uint32_t(y) & kM31, uint32_t(y >> 31), x, q.c0);
-  }
+__device__ __forceinline__ int cw_sign_h(const PairParam& q, const PairLimb& l, const KeyX& x) {
+  uint64_t y = mul_add_fold(l.c3, x, q.c2);
+  y = mul_add_fold(limb(y), x, q.c1);
+  y = mul_add_fold(limb(y), x, q.c0);
   return 1 - 2 * int((uint32_t(y) ^ ge_p(y)) & 1u);
 }
 
@@ -264,15 +308,22 @@ struct AggCol {
   int64_t off;   // byte offset of the count array (presence: the bitmap) in the workspace
   int64_t base;  // key of slot 0 (declared domain) or 0
   uint64_t mask; // ~0 (declared domain) or cap - 1 (power of two)
-  int64_t hash_chunk0;  // first chunk of this column in the hashing pass (hash_chunk slots each)
-  int32_t kind, pad;    // kAggCount / kAggPresence
+  // hashing pass: the column's pairs are hashed in slabs of hash_pairs, and each slab's slots are
+  // dealt to at most hash_groups items; its items begin at hash_item0
+  int64_t hash_item0;
+  int32_t kind;  // kAggCount / kAggPresence
+  int32_t hash_pairs, hash_groups, hash_slabs;
 };
-// Slots per chunk of the hashing pass (a multiple of 512, 32 per warp): kHashChunkMax, less only
-// where that would leave resident CTAs without a chunk (1.1 M slots: 75 us with 67 chunks for
-// 304 CTAs, 47 us with one or more each).  Shorter ones than that restart each warp's
-// compaction more often: 1024 slots took the pass over the sparse counts of a 10% sample, 9 M
-// slots, from 123 to 230 us.
-constexpr int64_t kHashChunkMin = 1024, kHashChunkMax = 16384;
+// Hashing pass (k_agg_hash): threads, pairs of a slab at most, slots a warp reads at a time; the
+// shared memory of a slab's counters (192 KB and one CTA per SM instead: 50 us more on five
+// tables, 356 us instead of 295 on a batch of graphs); items per resident CTA, so that the
+// CTAs end together: few where counters have to be written out (4 / 8 / 16: 123 / 132 / 144 us
+// on the sparse counts of a 10% sample, 492 / 401 / 380 us on the dense ones of 48 joins), more
+// where not (24 / 48: 637 / 490 us).
+constexpr int kHashThreads = 512, kHashMaxPairs = 64;
+constexpr int64_t kHashStep = 128;
+constexpr int64_t kHashBudget = 76 << 10;      // two CTAs per SM
+constexpr int64_t kHashItems = 6, kHashDirectItems = 48;
 // Presence bitmaps are walked in runs of kDenseRun keys (8 words); a bitmap holds whole runs.
 constexpr int64_t kDenseRun = 256;
 __host__ __device__ inline int64_t presence_words(int64_t cap) { return (cap + kDenseRun - 1) / kDenseRun * (kDenseRun / 32); }
@@ -372,8 +423,8 @@ struct BuildArgs {
   int64_t cnt_chunk_begin, cnt_chunk_end;     // its chunks
   int32_t cnt_cache_slots, cnt_cache_cols;  // counting pass: hot-key cache slots per column, columns cached
   int64_t cnt_total_chunks;
-  int64_t hash_total_chunks, hash_chunk;  // hashing pass of the aggregated columns: chunks, slots of one
-  int32_t hash_max_pairs;     // most (sketch, row) pairs on one aggregated column
+  int64_t hash_items;   // hashing pass of the aggregated columns: its items,
+  int32_t hash_private;  // words of the CTA's own counters (0: counters in global memory)
   // unique-key kernel
   const UniqSlab* uslab;
   const UniqItem* uitem;
@@ -381,7 +432,6 @@ struct BuildArgs {
   int64_t n_uitems;
   int32_t u_pack16;  // 1: one pair per slab, counters as two 16-bit halves per word
   int32_t u_words;   // shared-memory counter words of a slab
-  uint32_t m31, m4;  // 2^31 and 4 (multipliers of the Horner steps)
   // dense (presence-bitmap) kernel: slabs, items and CTA map as for the unique-key kernel
   const UniqSlab* dslab;
   const UniqItem* ditem;
@@ -405,8 +455,9 @@ struct BuildPlanHdr {
   int32_t cnt_grid, cnt_threads;
   int64_t ws_bytes;
   int32_t cnt_cache_slots, cnt_cache_cols;
-  int64_t hash_total_chunks, hash_chunk;
-  int32_t hash_max_pairs, hash_grid;
+  int64_t hash_items;
+  int32_t hash_private;
+  int32_t hash_grid;
   int64_t n_uslab, off_uslab, n_uitems, off_uitems, off_u_cta;  // unique-key kernel
   int32_t u_grid, u_pack16, u_words, u_tile_rows;
   int64_t n_dslab, off_dslab, n_ditems, off_ditems, off_d_cta;  // dense kernel
@@ -420,7 +471,7 @@ struct BuildPlanHdr {
   // chunks from here on are of tables with predicates or a sample (k_agg_count; before: k_count_rows)
   int64_t cnt_filtered;
 };
-constexpr int32_t kBuildPlanVersion = 11;
+constexpr int32_t kBuildPlanVersion = 12;
 struct ZeroSpan {
   void* ptr;
   int64_t bytes;

@@ -15,13 +15,11 @@ namespace {
 constexpr int kMbThreads = 512;
 constexpr int kMbMaxPairs = 64;
 
-// form 0: the key's powers x, x^2, x^3 shared by every pair (aggregated and int32-slab
-// paths); form 1: the Horner form per pair (packed-slab path).  Keys are 0 .. n_keys - 1
-// (below 2^31: the small-key arithmetic, as for every key of a 32-bit domain).
+// form 0: the key's powers x, x^2, x^3 shared by every pair (keys of 2^31 and more); form 1:
+// the Horner steps of keys below 2^31.  Keys are 0 .. n_keys - 1.
 template <int FORM>
 __global__ void __launch_bounds__(kMbThreads) k_cw_microbench(const cmp_hash* hash, int32_t n_pairs, int64_t n_keys,
-                                                             uint32_t w_mask, uint32_t m31, uint32_t m4,
-                                                             unsigned long long* out) {
+                                                             uint32_t w_mask, unsigned long long* out) {
   __shared__ PairParam prm[kMbMaxPairs];
   for (int p = threadIdx.x; p < n_pairs; p += blockDim.x) prm[p] = make_pair_param(hash[p]);
   __syncthreads();
@@ -32,14 +30,17 @@ __global__ void __launch_bounds__(kMbThreads) k_cw_microbench(const cmp_hash* ha
     if (FORM == 0) {
       const KeyPow kp = key_powers(x);
       for (int p = 0; p < n_pairs; p++)
-        acc += cw_bucket<true, true>(prm[p], kp, w_mask + 1) ^ uint32_t(cw_sign<true>(prm[p], kp));
+        acc += cw_bucket<true>(prm[p], pair_limbs(prm[p]), kp, w_mask + 1) ^ uint32_t(cw_sign(prm[p], pair_limbs(prm[p]), kp));
     } else {
-      const KeyX kx = key_x(x);
-      for (int p = 0; p < n_pairs; p++) {
-        const PairParam q = prm[p];
-        const uint64_t c2 = q.c2_lo | (uint64_t(q.c2_hi) << 31), c1 = q.c1_lo | (uint64_t(q.c1_hi) << 31);
-        acc += cw_bucket_h<true, true>(q, kx, w_mask + 1, m31, m4) ^ uint32_t(cw_sign_h<true>(q, kx, c2, c1, m31, m4));
-      }
+      auto run = [&](auto f) {
+        constexpr int F = decltype(f)::value;
+        for (int p = 0; p < n_pairs; p++) {
+          const PairParam q = prm[p];
+          acc += sx_bucket<true, F>(q, uint32_t(x), w_mask + 1) ^ uint32_t(1 - 2 * int(sx_odd<F>(q, uint32_t(x))));
+        }
+      };
+      if (key_form(x) == kSmall29) run(std::integral_constant<int, kSmall29>{});
+      else run(std::integral_constant<int, kSmall31>{});
     }
   }
 #pragma unroll
@@ -61,10 +62,10 @@ extern "C" cmp_status cmp_microbench_cw(const cmp_hash* hash_dev, int32_t n_pair
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const unsigned grid = unsigned(sm_count()) * 4;
   if (form == 0)
-    k_cw_microbench<0><<<grid, kMbThreads, 0, st>>>(hash_dev, n_pairs, n_keys, uint32_t(w - 1), 1u << 31, 4u,
+    k_cw_microbench<0><<<grid, kMbThreads, 0, st>>>(hash_dev, n_pairs, n_keys, uint32_t(w - 1),
                                                    reinterpret_cast<unsigned long long*>(out_dev));
   else
-    k_cw_microbench<1><<<grid, kMbThreads, 0, st>>>(hash_dev, n_pairs, n_keys, uint32_t(w - 1), 1u << 31, 4u,
+    k_cw_microbench<1><<<grid, kMbThreads, 0, st>>>(hash_dev, n_pairs, n_keys, uint32_t(w - 1),
                                                    reinterpret_cast<unsigned long long*>(out_dev));
   return cudaGetLastError() == cudaSuccess ? CMP_OK : CMP_ECUDA;
 }

@@ -119,30 +119,36 @@ __global__ void __launch_bounds__(1024) k_part_build(const __grid_constant__ Par
       } else {
         for (int s = tid; s < n_surv; s += T) {
           const int64_t row = r0 + (filtered ? int64_t(surv[s]) : int64_t(s));
-          KeyPow kp[axes_or_1<K>()];
-          bool small = true;
+          int64_t key[axes_or_1<K>()];
+          uint64_t bits = 0;
 #pragma unroll
           for (int l = 0; l < K; l++) {
-            const uint64_t x = key_field(load1(kcol[l], kdt[l], row));
-            kp[l] = key_powers(x);
-            small = small && x < (1ull << 31);
+            key[l] = load1(kcol[l], kdt[l], row);
+            bits |= uint64_t(key[l]);
           }
-          auto update = [&](auto smallx) {
-            constexpr bool SX = decltype(smallx)::value;
+          with_form(key_form(bits), [&](auto form) {
+            constexpr int F = decltype(form)::value;
+            constexpr bool SX = F != kAnyKey;
+            KeyPow kp[axes_or_1<K>()];
+#pragma unroll
+            for (int l = 0; l < K; l++)
+              if (!SX) kp[l] = key_powers(key_field(key[l]));
             for (int i = 0; i < r_n; i++) {
-              uint32_t idx = 0;
-              int sg = 1;
+              uint32_t idx = 0, odd = 0;
 #pragma unroll
               for (int l = 0; l < K; l++) {
                 const PairParam& q = prm[i * K + l];
-                idx += cw_bucket<POW2, SX>(q, kp[l], A.width[l]) * A.stride[l];
-                sg *= cw_sign<SX>(q, kp[l]);
+                if (SX) {
+                  idx += sx_bucket<POW2, F>(q, uint32_t(key[l]), A.width[l]) * A.stride[l];
+                  odd ^= sx_odd<F>(q, uint32_t(key[l]));
+                } else {
+                  idx += cw_bucket<POW2>(q, pair_limbs(q), kp[l], A.width[l]) * A.stride[l];
+                  odd ^= uint32_t(cw_sign_residue(q, pair_limbs(q), kp[l])) & 1u;
+                }
               }
-              atomicAdd(out + int64_t(i) * A.size + idx, sg);
+              atomicAdd(out + int64_t(i) * A.size + idx, 1 - 2 * int(odd));
             }
-          };
-          if (__all_sync(__activemask(), small)) update(std::true_type{});
-          else update(std::false_type{});
+          });
         }
       }
       __syncthreads();  // surv is rewritten by the next tile
