@@ -289,7 +289,8 @@ struct BuildPlanParts {
   std::vector<CountItem> cnt_items;
   int64_t cnt_total_chunks = 0;
   int32_t cnt_grid = 0;
-  int64_t cnt_filtered = 0;  // first chunk of the tables with predicates or a sample
+  int64_t cnt_sampled = 0;   // first chunk of the tables with a row sample and no predicates
+  int64_t cnt_filtered = 0;  // first chunk of the tables with predicates
   int64_t cnt_split = 0;  // > 0: two launches, the tables with presence columns first
   int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the second counting launch
   int32_t cnt_grid_b = 0;
@@ -336,7 +337,7 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   P->surv_by.assign(n_tables, kSurvRow);
   P->col_agg.assign(n_tables, std::vector<int32_t>(CMP_MAX_COLS, -1));
   P->aggs.clear();
-  size_t ws = al256(16 * size_t(n_tables) * CMP_MAX_SKETCHES + 40);  // stats + chunk counters (upper bound)
+  size_t ws = al256(16 * size_t(n_tables) * CMP_MAX_SKETCHES + 48);  // stats + chunk counters (upper bound)
   for (int32_t t = 0; t < n_tables; t++) {
     const cmp_table& tb = tables[t];
     const bool agg_on = tb.n_sketches > 0 && tb.n_rows > 0 && s.dedupe &&
@@ -640,7 +641,7 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   // long), at most 64 tiles; a persistent grid of about one resident wave takes the chunks
   // in order
   // (tables with a presence column first, so that a split pass completes every bitmap in its
-  // first launch; then the other tables without a selection, then those with one: each kind is
+  // first launch; then the other tables without predicates, then those with: each kind is
   // counted by its own kernel)
   P->cnt_items.clear();
   P->cnt_total_chunks = 0;
@@ -670,19 +671,20 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   // make up a CTA's share of each kind, and a cache has at most one slot per 16 rows of a
   // chunk.  (Chunks of 16,384 rows with caches of 8192 slots sent 103 M of 162.5 M keys of 58
   // tables to L2.)
-  auto count_kind = [&](int32_t t) {  // 0 presence columns, 1 no selection, 2 a selection, -1 not counted
+  auto count_kind = [&](int32_t t) {  // 0 presence columns, 1 every row, 2 a sample, 3 predicates, -1 not counted
     int ncol = 0;
     for (int32_t c = 0; c < CMP_MAX_COLS; c++) ncol += P->col_agg[t][c] >= 0;
     if (!ncol) return -1;
-    const bool filtered = tables[t].n_preds > 0 || sample_keep_of(tables[t].sample_rate) != 0;
-    return has_presence(t) ? 0 : (filtered ? 2 : 1);
+    if (has_presence(t)) return 0;
+    return tables[t].n_preds > 0 ? 3 : (sample_keep_of(tables[t].sample_rate) != 0 ? 2 : 1);
   };
-  int64_t kind_rows[3] = {0, 0, 0};
+  int64_t kind_rows[4] = {0, 0, 0, 0};
   for (int32_t t = 0; t < n_tables; t++)
     if (count_kind(t) >= 0) kind_rows[count_kind(t)] += tables[t].n_rows;
   const int64_t cnt_ctas = int64_t(sm_count()) * (P->uitems.empty() ? 2 : 1);
-  for (int pass = 0; pass < 3; pass++) {
-  if (pass == 2) P->cnt_filtered = P->cnt_total_chunks;
+  for (int pass = 0; pass < 4; pass++) {
+  if (pass == 2) P->cnt_sampled = P->cnt_total_chunks;
+  if (pass == 3) P->cnt_filtered = P->cnt_total_chunks;
   for (int32_t t = 0; t < n_tables; t++) {
     if (count_kind(t) != pass) continue;
     CountItem ci;
@@ -832,6 +834,7 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.cnt_total_chunks = P.cnt_total_chunks;
   h.cnt_grid = P.cnt_grid;
   h.cnt_split = P.cnt_split;
+  h.cnt_sampled = P.cnt_sampled;
   h.cnt_filtered = P.cnt_filtered;
   h.hash_private = P.hash_private;
   h.cnt_grid_b = P.cnt_grid_b;
@@ -919,7 +922,7 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     a.cnt_cache_cols = h.cnt_cache_cols;
     // the (max, min) key ranges start from zero (decoding as an empty column), so do the
     // chunk counters of the counting and hashing passes after them
-    if (cudaMemsetAsync(ws_dev, 0, 16 * size_t(h.n_agg) + 40, cs) != cudaSuccess) return CMP_ECUDA;
+    if (cudaMemsetAsync(ws_dev, 0, 16 * size_t(h.n_agg) + 48, cs) != cudaSuccess) return CMP_ECUDA;
     if (launch_agg_zero(a, cs) != cudaSuccess) return CMP_ECUDA;
   }
   const int32_t hash_grid = h.n_agg > 0 ? h.hash_grid : 0;
@@ -928,9 +931,10 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     // the tables with presence columns, then the others with the dense kernel beside them
     // (its programmatic dependent: one CTA of each per SM, a memory-bound scan beside an
     // integer-bound walk; every bitmap is complete before the second launch starts)
-    if (launch_count_rows(a, h.cnt_grid, 0, 0, h.cnt_split, cs) != cudaSuccess ||
+    if (launch_count_rows(a, false, h.cnt_grid, 0, 0, h.cnt_split, cs) != cudaSuccess ||
         launch_presence_check(a, cs) != cudaSuccess ||
-        launch_count_rows(a, h.cnt_grid_b, 2, h.cnt_split, h.cnt_filtered, cs) != cudaSuccess ||
+        launch_count_rows(a, false, h.cnt_grid_b, 2, h.cnt_split, h.cnt_sampled, cs) != cudaSuccess ||
+        launch_count_rows(a, true, h.cnt_grid_b, 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
         launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid_b, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
             cudaSuccess)
       return CMP_ECUDA;
@@ -950,7 +954,8 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
   if (h.n_agg > 0 &&
       (launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
            cudaSuccess ||
-       launch_count_rows(a, h.cnt_grid, 0, 0, h.cnt_filtered, cs) != cudaSuccess))
+       launch_count_rows(a, true, h.cnt_grid, 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
+       launch_count_rows(a, false, h.cnt_grid, 0, 0, h.cnt_sampled, cs) != cudaSuccess))
     return CMP_ECUDA;
   // the unique-key kernel right after the counting pass, as its programmatic dependent:
   // one CTA of each per SM, the two overlap (memory-bound scan, integer-bound hashing)
@@ -976,10 +981,11 @@ extern "C" cmp_status cmp_build_plan_stats(const void* plan_host, cmp_build_plan
   info->n_unique_items = h.n_uitems;
   info->row_grid = h.shape.grid;
   info->ws_bytes = h.ws_bytes;
-  // zeroing; clearing, counting (tables without and with a selection, presence columns apart in
+  // zeroing; clearing, counting (tables counted whole, sampled and with predicates, presence columns apart in
   // a split pass; each when it has chunks) and hashing of the counted keys; the unique-key
   // kernel; the row kernel; the presence check and the dense kernel
-  const int32_t count_launches = (h.cnt_split > 0 ? 1 : 0) + (h.cnt_filtered > h.cnt_split ? 1 : 0) +
+  const int32_t count_launches = (h.cnt_split > 0 ? 1 : 0) + (h.cnt_sampled > h.cnt_split ? 1 : 0) +
+                                 (h.cnt_filtered > h.cnt_sampled ? 1 : 0) +
                                  (h.cnt_total_chunks > h.cnt_filtered ? 1 : 0);
   info->launches = 1 + (h.n_agg > 0 ? 1 + count_launches + (h.hash_grid > 0 ? 1 : 0) : 0) +
                    (h.n_uitems > 0 && h.u_grid > 0 ? 1 : 0) + (h.shape.grid > 0 ? 1 : 0) +

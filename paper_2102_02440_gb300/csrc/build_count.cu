@@ -1,8 +1,7 @@
-// Counting pass of key aggregation over tables without a selection: every row of every
+// Counting pass of key aggregation over tables without predicates: every (sampled) row of every
 // aggregated key column counts its key's slot (key - base) & mask in the CTA's shared-memory
 // hot-key cache or, on a miss, with a global reduction on the count array; a presence column
-// sets its key's bit.  Tables with predicates or a row sample are counted by k_agg_count
-// (build.cu).
+// sets its key's bit.  Tables with predicates are counted by k_agg_count (build.cu).
 //
 // Bound by the shared-memory and L2 reductions of the keys (about one 32-key group per 50
 // cycles and SM), so the kernel keeps everything else out of their way: a column's
@@ -169,9 +168,94 @@ __device__ __forceinline__ bool count_rows(const CntCol& cc, const KT* __restric
   return ok;
 }
 
+// Rows [r0, r0 + n) of a sampled table, by the whole CTA: each warp tries 64 rows at a time, keeps
+// the sampled ones' offsets in its buffer (128 entries) and counts 64 of them, two per lane, in
+// one or two columns whenever it holds 64.  The trials are the bulk of it: with the keys counted
+// by the few lanes whose row is kept, every column cost a whole warp's work per 32 rows.  The
+// columns' descriptors stay in shared memory: they are needed once in 64 kept rows, and in
+// registers they spilled.  40 M rows at 10%, two columns: 386 us as filtered tiles, 216 us now.
+// Returns the rows kept by this warp; key ranges as in count_rows.
+struct SampledCol {
+  CntCol cc;
+  const void* col;
+  int32_t dtype;
+};
+struct SampledRange {
+  int64_t mn, mx;
+  bool ok;
+};
+__device__ __forceinline__ uint32_t count_sampled(const volatile SampledCol* scv, SampledRange (&sr)[2], int ncol,
+                                                  int64_t r0, uint32_t n, uint64_t seed, uint64_t keep, uint32_t* buf) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t lt = (1u << lane) - 1u;
+  uint32_t nb = 0, kept = 0;  // warp-uniform
+  auto count = [&](uint32_t m) {  // the first m <= 64 entries
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      if (c >= ncol) break;
+      const volatile SampledCol& v = scv[c];
+      const void* col = v.col;
+      const int32_t dtype = v.dtype;
+      int64_t key[2];
+#pragma unroll
+      for (int e = 0; e < 2; e++)
+        if (lane + 32 * e < m) key[e] = load1(col, dtype, r0 + buf[lane + 32 * e]);
+      CntCol cc;
+      cc.cnt = v.cc.cnt, cc.base = v.cc.base, cc.ckey = v.cc.ckey, cc.ccnt = v.cc.ccnt;
+      cc.last = v.cc.last, cc.mask = v.cc.mask, cc.hshift = v.cc.hshift, cc.declared = v.cc.declared;
+#pragma unroll
+      for (int e = 0; e < 2; e++) {
+        if (lane + 32 * e >= m) continue;
+        const uint64_t off = uint64_t(key[e]) - cc.base;
+        sr[c].mn = min(sr[c].mn, key[e]);
+        sr[c].mx = max(sr[c].mx, key[e]);
+        if (cc.declared && off > cc.last) {
+          sr[c].ok = false;
+          continue;
+        }
+        const uint32_t x = uint32_t(off) & cc.mask;
+        if (!cache_count(cc, x)) red_add(cc.cnt + x, 1);
+      }
+    }
+    __syncwarp();
+  };
+  for (uint32_t b = 64 * warp; b < n; b += 64 * nw) {
+    bool in[2];
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const uint32_t r = b + 32 * h + lane;
+      in[h] = r < n && splitmix64_at(seed, uint64_t(r0) + r) < keep;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      const unsigned m = __ballot_sync(0xffffffffu, in[h]);
+      if (in[h]) buf[nb + __popc(m & lt)] = b + 32 * h + lane;
+      nb += __popc(m);
+    }
+    __syncwarp();
+    if (nb >= 64) {
+      count(64);
+      nb -= 64;  // fewer than 64 left: to the front
+      uint32_t v0 = 0, v1 = 0;
+      if (lane < nb) v0 = buf[64 + lane];
+      if (lane + 32 < nb) v1 = buf[96 + lane];
+      __syncwarp();
+      if (lane < nb) buf[lane] = v0;
+      if (lane + 32 < nb) buf[32 + lane] = v1;
+      kept += 64;
+      __syncwarp();
+    }
+  }
+  if (nb) count(nb);
+  return kept + nb;
+}
+
 }  // namespace
 
 // Persistent CTAs take chunks of a table's rows in order from an atomic counter, one ahead.
+// SAMPLED: the tables with a row sample (a kernel of their own: in one, the sample's registers
+// made the other loops spill).
+template <bool SAMPLED>
 __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ BuildArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   // the unique-key kernel or the dense kernel, launched next as a programmatic dependent, reads
@@ -179,6 +263,8 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ int32_t acol[CMP_MAX_SKETCHES], aidx[CMP_MAX_SKETCHES], n_ac;
   __shared__ unsigned long long amax[CMP_MAX_SKETCHES], amin[CMP_MAX_SKETCHES];  // encoded
+  __shared__ uint32_t sbuf[SAMPLED ? 512 / 32 : 1][128];  // sampled rows, per warp
+  __shared__ SampledCol scol[SAMPLED ? CMP_MAX_SKETCHES : 1];  // the current table's columns
   __shared__ uint32_t akeys;  // the current table's aggregated key columns (bit c: column c)
   __shared__ long long next_chunk;
   const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31;
@@ -221,7 +307,8 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
     const DevTable* tb = A.tables + ci.table;
     __syncthreads();  // every thread has read next_chunk
     if (tid == 0) next_chunk = A.cnt_chunk_begin + (long long)atomicAdd(work, 1ull);
-    if (it != item) {  // a new table: flush the caches, then set them up for its columns
+    const bool new_table = it != item;  // block-uniform
+    if (new_table) {  // flush the caches, then set them up for its columns
       if (item >= 0) flush();
       H = ci.cache_slots;
       ccnt = ckey + size_t(H) * n_cache;
@@ -257,9 +344,7 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
     const int nac = n_ac;
     const int64_t r_begin = (c - ci.chunk_begin) * ci.chunk_rows;
     const int64_t r_end = min(int64_t(tb->n_rows), r_begin + ci.chunk_rows);
-    if (tid == 0 && r_end > r_begin)
-      atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), (unsigned long long)(r_end - r_begin));
-    for (int a = 0; a < nac; a++) {
+    auto cnt_col = [&](int a) {
       const AggCol& ac = agg_of(a);
       CntCol cc;
       cc.cnt = reinterpret_cast<int32_t*>(A.ws + ac.off);
@@ -270,6 +355,50 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
       cc.mask = uint32_t(ac.mask);
       cc.hshift = uint32_t(32 - (31 - __clz(H)));  // H is a power of two >= 256
       cc.declared = ac.mask == ~0ull;
+      return cc;
+    };
+    // key ranges of column a, over the warp, into the table's
+    auto fold_range = [&](int a, const CntCol& cc, bool ok, int64_t mn, int64_t mx) {
+      const AggCol& ac = agg_of(a);
+      // a declared domain stands for its keys, unless one left it: out of range
+      if (cc.declared) mn = ac.base, mx = ac.base + (ac.cap - 1);
+      if (!ok) mn = INT64_MIN, mx = INT64_MAX;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        mn = min(mn, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mn, o));
+        mx = max(mx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mx, o));
+      }
+      if (lane == 0 && mx >= mn) {
+        atomicMax(&amax[a], (unsigned long long)enc_max(mx));
+        atomicMax(&amin[a], (unsigned long long)enc_min(mn));
+      }
+    };
+    if constexpr (SAMPLED) {
+      if (new_table) {
+        if (tid < nac) {
+          scol[tid].cc = cnt_col(tid);
+          scol[tid].col = tb->col[acol[tid]];
+          scol[tid].dtype = tb->dtype[acol[tid]];
+        }
+        __syncthreads();
+      }
+      unsigned long long kept = 0;
+      for (int a = 0; a < nac; a += 2) {  // (a sampled table has no presence columns)
+        const int ncol = min(2, nac - a);
+        SampledRange sr[2] = {{INT64_MAX, INT64_MIN, true}, {INT64_MAX, INT64_MIN, true}};
+        kept = count_sampled(scol + a, sr, ncol, r_begin, uint32_t(r_end - r_begin), tb->sample_seed, tb->sample_keep,
+                             sbuf[tid >> 5]);
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+          if (q < ncol) fold_range(a + q, scol[a + q].cc, sr[q].ok, sr[q].mn, sr[q].mx);
+      }
+      if (lane == 0 && kept) atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), kept);
+    } else {
+    if (tid == 0 && r_end > r_begin)
+      atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), (unsigned long long)(r_end - r_begin));
+    for (int a = 0; a < nac; a++) {
+      const AggCol& ac = agg_of(a);
+      const CntCol cc = cnt_col(a);
       const bool i32 = tb->dtype[acol[a]] == CMP_I32, presence = ac.kind == kAggPresence;
       // the slots of an int32 column are 32-bit sums when its domain lies in int32
       const bool small = !cc.declared || (ac.base >= INT32_MIN && ac.base + ac.cap <= int64_t(INT32_MAX) + 1);
@@ -294,18 +423,8 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
           else red_add(cc.cnt + off, 1);
         }
       }
-      // a declared domain stands for its keys, unless one left it: out of range
-      if (cc.declared) mn = ac.base, mx = ac.base + (ac.cap - 1);
-      if (!ok) mn = INT64_MIN, mx = INT64_MAX;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        mn = min(mn, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mn, o));
-        mx = max(mx, (int64_t)__shfl_xor_sync(0xffffffffu, (long long)mx, o));
-      }
-      if (lane == 0 && mx >= mn) {
-        atomicMax(&amax[a], (unsigned long long)enc_max(mx));
-        atomicMax(&amin[a], (unsigned long long)enc_min(mn));
-      }
+      fold_range(a, cc, ok, mn, mx);
+    }
     }
     c = c_next;
   }
@@ -316,23 +435,25 @@ size_t count_rows_smem_bytes(int32_t cache_slots, int32_t cache_cols) {
   return align16(sizeof(uint32_t) * 2 * size_t(cache_slots) * size_t(cache_cols));
 }
 
-// One launch over chunks [chunk_begin, chunk_end) of tables without a selection, taken from chunk
-// counter `work_slot` of the workspace header (zeroed before the build).
-cudaError_t launch_count_rows(const BuildArgs& a, int32_t grid, int32_t work_slot, int64_t chunk_begin,
+// One launch over chunks [chunk_begin, chunk_end) of tables without predicates, all with a row
+// sample or all without, taken from chunk counter `work_slot` of the workspace header (zeroed
+// before the build).
+cudaError_t launch_count_rows(const BuildArgs& a, bool sampled, int32_t grid, int32_t work_slot, int64_t chunk_begin,
                               int64_t chunk_end, cudaStream_t st) {
   if (a.n_agg <= 0 || grid <= 0 || chunk_end <= chunk_begin) return cudaSuccess;
+  auto k = sampled ? k_count_rows<true> : k_count_rows<false>;
   const size_t smem = count_rows_smem_bytes(a.cnt_cache_slots, a.cnt_cache_cols);
-  cudaError_t e = cudaFuncSetAttribute(k_count_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (e != cudaSuccess) return e;
   // the whole shared memory of the SM, so that a CTA of the unique-key or the dense kernel
   // (launched next, as a programmatic dependent) fits beside one of this pass
-  e = cudaFuncSetAttribute(k_count_rows, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+  e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;
   BuildArgs b = a;
   b.cnt_work_slot = work_slot;
   b.cnt_chunk_begin = chunk_begin;
   b.cnt_chunk_end = chunk_end;
-  k_count_rows<<<unsigned(std::min<int64_t>(grid, chunk_end - chunk_begin)), 512, smem, st>>>(b);
+  k<<<unsigned(std::min<int64_t>(grid, chunk_end - chunk_begin)), 512, smem, st>>>(b);
   return cudaGetLastError();
 }
 

@@ -468,10 +468,12 @@ struct BuildPlanHdr {
   // split pass: the dense kernel walks the first d_cut / 1024 of each item's runs beside the
   // second counting launch, the rest after it with 512 threads (d_cut = 1024: all beside)
   int32_t cnt_grid_b, d_cut;
-  // chunks from here on are of tables with predicates or a sample (k_agg_count; before: k_count_rows)
+  // chunks: tables with presence columns and without a selection, from cnt_sampled on tables with a
+  // row sample only (k_count_rows), from cnt_filtered on tables with predicates (k_agg_count)
+  int64_t cnt_sampled;
   int64_t cnt_filtered;
 };
-constexpr int32_t kBuildPlanVersion = 12;
+constexpr int32_t kBuildPlanVersion = 13;
 struct ZeroSpan {
   void* ptr;
   int64_t bytes;
@@ -508,7 +510,7 @@ cudaError_t launch_agg_zero(const BuildArgs& a, cudaStream_t st);
 cudaError_t launch_presence_check(const BuildArgs& a, cudaStream_t st);
 cudaError_t launch_agg_count(const BuildArgs& a, int32_t tile_rows, int32_t cnt_threads, int32_t cnt_grid,
                              int32_t work_slot, int64_t chunk_begin, int64_t chunk_end, cudaStream_t st);
-cudaError_t launch_count_rows(const BuildArgs& a, int32_t grid, int32_t work_slot, int64_t chunk_begin,
+cudaError_t launch_count_rows(const BuildArgs& a, bool sampled, int32_t grid, int32_t work_slot, int64_t chunk_begin,
                               int64_t chunk_end, cudaStream_t st);
 size_t uniq_smem_bytes(int32_t words, int32_t tile_rows);
 cudaError_t launch_uniq(const BuildArgs& a, int32_t grid, int32_t threads, int32_t tile_rows, cudaStream_t st);

@@ -76,3 +76,23 @@ def test_both_sides_of_the_smallest_aggregated_table(orc):
     for span in (1 << 16, 1 << 26):
         tabs.append(G.Table("sparse", [rng.integers(0, span, 9000).astype(np.int32)], [], [0], [len(tabs)]))
     _check(orc, tabs, None, 0)
+
+
+@pytest.mark.parametrize("rate", [1e-4, 0.1, 0.5, 0.999])
+@pytest.mark.parametrize("rows", [1, 31, 33, 2047, 70_001])
+def test_sampled_rows(orc, rows, rate):
+    """A row sample without predicates: few, some and nearly all rows kept per warp and buffer; the
+    reference is the oracle over the rows the oracle's sampler picks."""
+    from oracle import sample as S
+    rng = np.random.default_rng(rows)
+    cols, meta = _tables(rng, rows)
+    edges = list(range(len(cols)))
+    tab = G.Table("s", cols, [], edges, edges, meta)
+    wl = G.Workload("count", [tab], [0] * 6, [0] * 6, 3, 256, 99, 7)
+    dw = P.DeviceWorkload(wl, sample_rates=[rate], sample_seed=11)
+    dw.build_batched(K.cmp_build_cfg.make(aggregate=1))
+    torch.cuda.synchronize()
+    dw.check_status()
+    ref, n = orc.build_sketch(S.sampled_table(tab, 11, rate), dw.hash_u64, 3, 256)
+    assert int(dw.survivors.cpu()[0]) == n
+    assert np.array_equal(dw.tables[0].counters.cpu().numpy(), ref)
