@@ -129,8 +129,9 @@ typedef struct {
   int32_t tile_rows;      /* rows per tile (multiple of 128, <= 16384)                              */
   int32_t dedupe;         /* -1 auto, 0 off, 1 aggregate equal keys of a tile before hashing        */
   int32_t ctas_per_sm;    /* CTAs per SM the grid is sized for                                      */
-  int32_t aggregate;      /* batched build only: -1 auto (tables of >= 2^18 rows, and of >= 2^13 rows
-                             when the count array has at most 16 slots per row), 0 off, 1 every
+  int32_t aggregate;      /* batched build only: -1 auto (tables of >= 2^18 rows; where there is one, or
+                             enough work in columns of declared domains, also tables of >= 2^13
+                             rows whose count array has at most 16 slots per row), 0 off, 1 every
                              table: aggregate each key column's survivors per distinct key before
                              hashing (needs dedupe; same counters)                                  */
   int32_t unique;         /* batched build only: 0 or 1 on, -1 off: key columns declared
@@ -593,8 +594,8 @@ cmp_status cmp_mlp_train_step(float* params_dev, float* adam_m_dev, float* adam_
  * bucket and sign (cmp_hash; Sec. 3.1-3.2 ask for a per-row bucket hash and a 4-wise sign
  * family) of keys 0 .. n_keys-1 for each of the n_pairs parameter sets hash_dev[0..n_pairs)
  * (1..64), with no memory traffic and no counter updates, in the two forms the build uses:
- * form 0 shares the key's powers x^2, x^3 among the pairs (aggregated and int32-slab
- * paths), form 1 evaluates each pair by Horner's rule (packed-slab path).  w: a power of
+ * form 0 shares the key's powers x^2, x^3 among the pairs (keys of 2^31 and more), form 1
+ * evaluates each pair by Horner's rule (the keys here, all below 2^31).  w: a power of
  * two (the bucket mask).  XORs a checksum of every evaluation into *out_dev (one uint64,
  * device) so that none can be skipped.  n_keys <= 2^31.  Asynchronous on `stream`. */
 cmp_status cmp_microbench_cw(const cmp_hash* hash_dev, int32_t n_pairs, int64_t n_keys, int32_t w, int32_t form,

@@ -251,9 +251,15 @@ constexpr int64_t kAggMinRows = int64_t(1) << 18;
 constexpr int64_t kAggMaxCap = int64_t(1) << 27;
 // Smaller tables (from kAggSmallRows rows) are aggregated too when the count array has at most
 // kAggSmallFill slots per row: clearing and scanning 16 slots costs less than hashing one row
-// for a single sketch row does.
+// for a single sketch row does.  That holds where the passes run anyway, for a table of
+// kAggMinRows rows or more (96 tables of up to 300,000 rows: 895 us per row, 352 us counted).
+// Without one, the passes' own 100 us or so have to be earned: columns without a declared
+// domain, whose arrays are larger, stay per row (up to 100,000 rows: 24 tables 64 us per row and
+// 145 us counted, 96 tables 222 and 248 us), and declared ones are counted from
+// kAggSmallWork evaluations on (three stars, 31 M: 563 us per row, 430 us counted).
 constexpr int64_t kAggSmallRows = int64_t(1) << 13;
 constexpr int64_t kAggSmallFill = 16;
+constexpr int64_t kAggSmallWork = int64_t(1) << 24;
 // Without a declared domain the keys' range is unknown: at least kAggMinCap slots (4 MB, or
 // kAggSmallFill per row for smaller tables), so that keys sparser than the rows still fit.
 constexpr int64_t kAggMinCap = int64_t(1) << 20;
@@ -338,6 +344,18 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   P->col_agg.assign(n_tables, std::vector<int32_t>(CMP_MAX_COLS, -1));
   P->aggs.clear();
   size_t ws = al256(16 * size_t(n_tables) * CMP_MAX_SKETCHES + 48);  // stats + chunk counters (upper bound)
+  auto hashed_elsewhere = [&](const cmp_col& col) { return uniq_mode >= 0 && uniq_fits && (col.flags & CMP_COL_UNIQUE); };
+  bool large = false;      // a table of kAggMinRows rows or more is aggregated
+  int64_t small_work = 0;  // (row, sketch row) evaluations of smaller columns with declared domains
+  for (int32_t t = 0; t < n_tables; t++)
+    for (int k = 0; k < tables[t].n_sketches; k++) {
+      const cmp_col& col = tables[t].cols[tables[t].key_col[k]];
+      if (hashed_elsewhere(col)) continue;
+      const uint64_t dom = (col.flags & CMP_COL_DOMAIN) ? uint64_t(col.dom_hi) - uint64_t(col.dom_lo) : 0;
+      if (tables[t].n_rows >= kAggMinRows) large = true;
+      else if (tables[t].n_rows >= kAggSmallRows && dom > 0 && dom <= uint64_t(kAggSmallFill * tables[t].n_rows))
+        small_work += int64_t(tables[t].n_rows) * d;
+    }
   for (int32_t t = 0; t < n_tables; t++) {
     const cmp_table& tb = tables[t];
     const bool agg_on = tb.n_sketches > 0 && tb.n_rows > 0 && s.dedupe &&
@@ -346,7 +364,7 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
     for (int k = 0; k < tb.n_sketches; k++) {
       const int c = tb.key_col[k];
       const cmp_col& col = tb.cols[c];
-      if (uniq_mode >= 0 && uniq_fits && (col.flags & CMP_COL_UNIQUE)) {
+      if (hashed_elsewhere(col)) {
         const uint64_t span = (col.flags & CMP_COL_DOMAIN) ? uint64_t(col.dom_hi) - uint64_t(col.dom_lo) : 0;
         if (unfiltered && span > 0 && span <= uint64_t(kDenseMaxSpan) &&
             span <= uint64_t(kDenseMaxFill) * uint64_t(tb.n_rows)) {
@@ -382,7 +400,10 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
         a.base = 0;
         a.mask = uint64_t(a.cap) - 1;
       }
-      if (agg_mode == -1 && tb.n_rows < kAggMinRows && a.cap > kAggSmallFill * tb.n_rows) continue;  // per row
+      if (agg_mode == -1 && tb.n_rows < kAggMinRows) {
+        const bool pays = large || (a.mask == ~0ull && small_work >= kAggSmallWork);
+        if (!pays || a.cap > kAggSmallFill * tb.n_rows) continue;  // per row
+      }
       P->col_agg[t][c] = int32_t(P->aggs.size());
       P->aggs.push_back(a);
     }

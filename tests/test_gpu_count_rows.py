@@ -96,3 +96,16 @@ def test_sampled_rows(orc, rows, rate):
     ref, n = orc.build_sketch(S.sampled_table(tab, 11, rate), dw.hash_u64, 3, 256)
     assert int(dw.survivors.cpu()[0]) == n
     assert np.array_equal(dw.tables[0].counters.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("domain", [True, False])
+@pytest.mark.parametrize("n_tables", [10, 13])
+@pytest.mark.parametrize("large", [False, True])
+def test_small_tables_on_both_sides_of_the_work_they_need(orc, n_tables, domain, large):
+    """10 tables of 120,000 keys for 12 sketch rows need fewer than 2^24 evaluations, 13 more."""
+    rng = np.random.default_rng(n_tables)
+    tabs = [G.Table(f"t{i}", [rng.integers(0, 9000, 120_000).astype(np.int32)], [], [0], [i],
+                    [("domain", 0, 9000)] if domain else []) for i in range(n_tables)]
+    if large:
+        tabs.append(G.Table("large", [rng.integers(0, 9000, 1 << 18).astype(np.int32)], [], [0], [n_tables]))
+    _check(orc, tabs, None, 0, d=12, w=128)
