@@ -200,7 +200,8 @@ cmp_status cmp_sketch_build(const cmp_table* table, int32_t d, int32_t w, const 
  * (sketch, row) pair walks runs of consecutive keys, advancing h's and xi's residues by
  * finite differences (additions mod p, the same integers as evaluating the polynomials);
  * a key outside the domain, or one seen twice, sends the column to the per-row path.
- * Launches: zeroing, then (when present) clearing + counting, the unique-key kernel, the
+ * Launches: zeroing, then (when present) clearing, counting (one launch for each kind of
+ * table: with presence columns, whole, sampled, with predicates), the unique-key kernel, the
  * row kernel, the hashing of the counted keys and the presence-bitmap kernel.
  * cmp_build_plan_encode returns CMP_EWORKSPACE if plan_bytes is too small;
  * cmp_sketch_build_batched returns CMP_EWORKSPACE if ws_bytes is. */
