@@ -899,7 +899,7 @@ __global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_const
       open = false;
       cur_ai = ai;
       cur_slab = -1;
-      if (!agg_active(ac, ai, A.ws, &kmin, &range)) range = 0;
+      agg_active(ac, ai, A.ws, &kmin, &range);
       np_col = 0;
       for (int s = 0; s < tb->n_sketches; s++)
         if (tb->key_col[s] == ac.col) np_col += A.d;
@@ -922,11 +922,10 @@ __global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_const
       open = false;
       cur_slab = slab;
     }
-    // key kmin + j sits in slot (kmin - base + j) & mask; a load takes four slots from a multiple
-    // of four (count arrays are whole int4 words, a masked one at least 8 slots): from j = -shift
     const uint64_t off0 = uint64_t(kmin) - uint64_t(ac.base), mask = ac.mask;
-    const int64_t shift = int64_t(off0 & 3), begin = group * len - shift, end = min(range, begin + len);
-    if (group < groups && begin < end) {
+    const HashSpan span = hash_span(ac, kmin, range, len, group, groups);
+    const int64_t begin = span.begin, end = span.end;
+    if (begin < end) {
       if (!open) {
         const int p0 = slab * ac.hash_pairs, np = one_slab ? np_col : min(np_col - p0, ac.hash_pairs);
         if (tid < np) {

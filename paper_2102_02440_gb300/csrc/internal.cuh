@@ -341,17 +341,35 @@ __host__ __device__ inline int64_t dec_max(uint64_t e) { return int64_t(e ^ (1ul
 __host__ __device__ inline int64_t dec_min(uint64_t e) { return int64_t(~e ^ (1ull << 63)); }
 
 // Whether aggregated column `a` (index ai) takes the aggregated path in this run (read
-// after the counting pass), with its smallest surviving key and key range.
-__device__ __forceinline__ bool agg_active(const AggCol& a, int ai, const unsigned char* ws, int64_t* kmin,
-                                           int64_t* range) {
+// after the counting pass), with its smallest surviving key and key range (otherwise the
+// first slot's key and an empty range: never another column's).
+__host__ __device__ __forceinline__ bool agg_active(const AggCol& a, int ai, const unsigned char* ws, int64_t* kmin,
+                                                    int64_t* range) {
   const unsigned long long* st = reinterpret_cast<const unsigned long long*>(ws) + 2 * int64_t(ai);
   const int64_t mx = dec_max(st[0]), mn = dec_min(st[1]);
+  *kmin = a.base;
+  *range = 0;
   if (mx < mn) return false;
   const uint64_t r = uint64_t(mx) - uint64_t(mn);
   if (r >= uint64_t(a.cap)) return false;
   *kmin = mn;
   *range = int64_t(r) + 1;
   return true;
+}
+
+// The keys kmin + j, begin <= j < end, of item `group` of a column's `groups` items of `len` keys
+// each in the hashing pass.  Key kmin + j sits in slot (kmin - base + j) & mask, and a load
+// takes four slots from a multiple of four (count arrays are whole int4 words, a masked one at
+// least 8 slots), so the first item begins at j = -((kmin - base) & 3).  A column without a
+// range (inactive) has no items: its kmin says nothing about its array.
+struct HashSpan {
+  int64_t begin, end;
+};
+__host__ __device__ __forceinline__ HashSpan hash_span(const AggCol& a, int64_t kmin, int64_t range, int64_t len,
+                                                       int group, int groups) {
+  if (range <= 0 || group >= groups) return {0, 0};
+  const int64_t begin = group * len - int64_t((uint64_t(kmin) - uint64_t(a.base)) & 3);
+  return {begin, begin + len < range ? begin + len : range};
 }
 
 // Unique key columns (declared distinct, e.g. primary keys) of the batched build: no key
