@@ -328,7 +328,8 @@ size_t build_smem_bytes(const BuildShape& s, int w) {
 template <bool G, bool D, bool P>
 static cudaError_t launch_one(const BuildArgs& a, const BuildShape& s, cudaStream_t st) {
   auto k = k_sketch_build<G, D, P>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(s.smem_bytes));
+  static SmemLimit limit;
+  cudaError_t e = limit.allow(k);
   if (e != cudaSuccess) return e;
   k<<<s.grid, s.threads, s.smem_bytes, st>>>(a);
   return cudaGetLastError();
@@ -987,7 +988,8 @@ cudaError_t launch_agg_hash(const BuildArgs& a, int32_t grid, cudaStream_t st) {
   const bool pow2 = (a.w & (a.w - 1)) == 0;
   const size_t smem = kHashBufBytes + sizeof(int32_t) * size_t(a.hash_private);
   auto k = pow2 ? k_agg_hash<true> : k_agg_hash<false>;
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit[2];
+  cudaError_t e = limit[pow2].allow(k);
   if (e != cudaSuccess) return e;
   k<<<unsigned(grid), kHashThreads, smem, st>>>(a);
   return cudaGetLastError();
@@ -1055,7 +1057,8 @@ cudaError_t launch_agg_count(const BuildArgs& a, int32_t tile_rows, int32_t cnt_
                              int32_t work_slot, int64_t chunk_begin, int64_t chunk_end, cudaStream_t st) {
   if (a.n_agg <= 0 || cnt_grid <= 0 || chunk_end <= chunk_begin) return cudaSuccess;
   const size_t smem = agg_count_smem_bytes(tile_rows, a.cnt_cache_slots, a.cnt_cache_cols, cnt_threads);
-  cudaError_t e = cudaFuncSetAttribute(k_agg_count, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit;
+  cudaError_t e = limit.allow(k_agg_count);
   if (e != cudaSuccess) return e;
   // the whole shared memory of the SM, so that a CTA of the unique-key or the dense kernel
   // (launched next, as a programmatic dependent) fits beside one of this pass

@@ -443,7 +443,8 @@ cudaError_t launch_count_rows(const BuildArgs& a, bool sampled, int32_t grid, in
   if (a.n_agg <= 0 || grid <= 0 || chunk_end <= chunk_begin) return cudaSuccess;
   auto k = sampled ? k_count_rows<true> : k_count_rows<false>;
   const size_t smem = count_rows_smem_bytes(a.cnt_cache_slots, a.cnt_cache_cols);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit[2];
+  cudaError_t e = limit[sampled].allow(k);
   if (e != cudaSuccess) return e;
   // the whole shared memory of the SM, so that a CTA of the unique-key or the dense kernel
   // (launched next, as a programmatic dependent) fits beside one of this pass

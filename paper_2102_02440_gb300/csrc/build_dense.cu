@@ -227,7 +227,8 @@ template <bool PK, bool P2, int TH>
 static cudaError_t launch_dense_t(const BuildArgs& a, int32_t grid, bool pdl, cudaStream_t st) {
   auto k = k_dense_hash<PK, P2, TH>;
   const size_t smem = dense_smem_bytes(a.d_words);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit;
+  cudaError_t e = limit.allow(k);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;

@@ -220,7 +220,8 @@ template <bool PK, bool P2>
 static cudaError_t launch_uniq_t(const BuildArgs& a, int32_t grid, int32_t threads, int32_t tile_rows, cudaStream_t st) {
   auto k = k_uniq_hash<PK, P2>;
   const size_t smem = uniq_smem_bytes(a.u_words, tile_rows);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit;
+  cudaError_t e = limit.allow(k);
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
   if (e != cudaSuccess) return e;

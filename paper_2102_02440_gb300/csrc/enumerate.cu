@@ -929,8 +929,8 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
   a.warps = warps;
   while (a.warps > 1 && smem_of(a.warps) > size_t(200) * 1024) a.warps--;  // those beyond search nothing
   const size_t smem = smem_of(a.warps);
-  if (cudaFuncSetAttribute(k_enumerate, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess)
-    return CMP_ECUDA;
+  static SmemLimit limit;
+  if (limit.allow(k_enumerate) != cudaSuccess) return CMP_ECUDA;
   k_enumerate<<<unsigned(H.n_graphs), 32 * warps, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
   return cudaGetLastError() == cudaSuccess ? CMP_OK : CMP_ECUDA;
 }

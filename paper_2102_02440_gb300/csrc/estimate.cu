@@ -197,7 +197,8 @@ cudaError_t launch_presort_large(const int32_t* C, int64_t n_rows, int32_t w, ui
     const int64_t nr = n_rows - r0 < rows_per_pass ? n_rows - r0 : rows_per_pass;
     const int64_t nblk = nr * (L / kChunk);
     const int smem = int(sort_smem_bytes(kChunk));
-    cudaError_t e = cudaFuncSetAttribute(k_presort_chunks, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static SmemLimit limit;
+    cudaError_t e = limit.allow(k_presort_chunks);
     if (e != cudaSuccess) return e;
     k_presort_chunks<<<unsigned(nblk < 4096 ? nblk : 4096), 1024, smem, st>>>(C + r0 * w, nr, w, L, a);
     e = cudaGetLastError();
@@ -227,7 +228,8 @@ cudaError_t launch_presort(const int32_t* C, int64_t n_rows, int32_t w, uint32_t
   auto k = n > 8192 ? k_presort<16> : k_presort<8>;
   const int threads = n > 8192 ? n / 16 : n / 8;
   const size_t smem = sort_smem_bytes(n);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit[2];
+  cudaError_t e = limit[n > 8192].allow(k);
   if (e != cudaSuccess) return e;
   const int64_t grid = n_rows < 4096 ? n_rows : 4096;
   k<<<unsigned(grid), threads, smem, st>>>(C, n_rows, w, abs_out, perm_out);

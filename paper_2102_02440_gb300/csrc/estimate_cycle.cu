@@ -545,7 +545,8 @@ __global__ void __launch_bounds__(kCycThreads, 2) k_cycle(const __grid_constant_
 cudaError_t launch_estimate_cycle(const EstArgs& a, cudaStream_t st) {
   if (a.n_cyc <= 0) return cudaSuccess;
   const size_t smem = cyc_smem_bytes(a.w);
-  cudaError_t e = cudaFuncSetAttribute(k_cycle, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  static SmemLimit limit;
+  cudaError_t e = limit.allow(k_cycle);
   if (e != cudaSuccess) return e;
   k_cycle_prep<<<unsigned(a.n_cyc * a.d), 1024, 0, st>>>(a);
   const int64_t jobs = a.n_cyc * a.d * ((a.w + kCycBlk - 1) / kCycBlk);

@@ -545,7 +545,8 @@ cudaError_t launch_estimate_star(const EstArgs& a, cudaStream_t st) {
   const int64_t lat = a.n_star_units - a.n_star_suf_units;
   if (lat > 0) {
     const size_t smem = star_smem_bytes();
-    cudaError_t e = cudaFuncSetAttribute(k_star_lattice, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    static SmemLimit limit;
+    cudaError_t e = limit.allow(k_star_lattice);
     if (e != cudaSuccess) return e;
     const int64_t grid = std::min<int64_t>(lat, int64_t(sm_count()) * 2);  // two 80 KB CTAs per SM
     k_star_lattice<<<unsigned(grid), kStarThreads, smem, st>>>(a);

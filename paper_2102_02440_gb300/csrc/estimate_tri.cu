@@ -763,16 +763,16 @@ cudaError_t launch_estimate_tri(const EstArgs& a, cudaStream_t st) {
   const int smem0 = int(sizeof(unsigned long long)) * wp2 + int(align16(sizeof(int32_t) * size_t(a.w + 1)));
   const int sep = size_t(smem0) + 2 * sizeof(uint32_t) * size_t(wp2) <= smem_optin_bytes() - 4096 ? 1 : 0;
   const int smem = smem0 + (sep ? int(2 * sizeof(uint32_t)) * wp2 : 0);
-  cudaError_t e = cudaFuncSetAttribute(k_tri_prep, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  static SmemLimit limit_prep, limit_nodes, limit_sweep;
+  cudaError_t e = limit_prep.allow(k_tri_prep);
   if (e != cudaSuccess) return e;
   if (int64_t(4) * a.w > 48 * 1024) {
-    e = cudaFuncSetAttribute(k_tri_nodes, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * a.w);
+    e = limit_nodes.allow(k_tri_nodes);
     if (e != cudaSuccess) return e;
   }
   const bool staged = tri_sweep_smem(a.w) <= kTriSweepSmemMax;
   if (staged) {
-    e = cudaFuncSetAttribute(k_tri_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(tri_sweep_smem(a.w)));
+    e = limit_sweep.allow(k_tri_sweep<true>);
     if (e != cudaSuccess) return e;
   }
   for (int64_t r0 = 0; r0 < rows; r0 += a.tri_slots) {

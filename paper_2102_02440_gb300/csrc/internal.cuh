@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 
 #include "compass.h"
@@ -540,6 +541,31 @@ constexpr int32_t kDenseThreadsAlone = 512, kDenseThreadsBeside = 256;
 
 int sm_count();
 size_t smem_optin_bytes();
+
+// Dynamic shared memory beyond 48 KB has to be allowed per kernel, and the limit is the
+// process's, not the call's: set to what one call needs, it could be lowered by another host
+// thread's smaller call before this one's launch, which then failed.  So every call allows the
+// most the kernel can be given, the same value each time (one object per kernel; a failed
+// query is not kept).
+class SmemLimit {
+ public:
+  template <typename... A>
+  cudaError_t allow(void (*kernel)(A...)) {
+    const void* const f = reinterpret_cast<const void*>(kernel);
+    int n = most_.load(std::memory_order_relaxed);
+    if (n == 0) {
+      cudaFuncAttributes a;
+      const cudaError_t e = cudaFuncGetAttributes(&a, f);
+      if (e != cudaSuccess) return e;
+      n = int(smem_optin_bytes()) - int(a.sharedSizeBytes);
+      most_.store(n, std::memory_order_relaxed);
+    }
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+  }
+
+ private:
+  std::atomic<int> most_{0};
+};
 // host checks and device descriptor of one cmp_table (api_build.cu)
 cmp_status check_table(const cmp_table* t, int32_t d, int32_t w, int32_t n_edges);
 DevTable to_dev(const cmp_table* t, int32_t* counters, int64_t* survivors);

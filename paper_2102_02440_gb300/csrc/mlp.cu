@@ -485,7 +485,8 @@ cudaError_t launch_mlp_train(float* P, float* m, float* v, int32_t nin, int32_t 
   const int32_t np = nh * nin + 2 * nh + 1;
   if (ctas > 0) {
     const size_t smem = sizeof(float) * size_t(train_smem(nin, nh).total);
-    cudaError_t e0 = cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    static SmemLimit limit;
+    cudaError_t e0 = limit.allow(k_mlp_grad);
     if (e0 != cudaSuccess) return e0;
     k_mlp_grad<<<unsigned(ctas), kTrainSamples, smem, st>>>(P, nin, nh, skip, x, t, n, huber_delta, chunks, partial,
                                                             partial_loss);

@@ -170,7 +170,8 @@ template <int K, bool SMEM, bool POW2>
 cudaError_t launch_part_build_t(const PartBuildArgs& a, int grid, int threads, size_t smem, cudaStream_t st) {
   auto kern = k_part_build<K, SMEM, POW2>;
   if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    static SmemLimit limit;
+    const cudaError_t e = limit.allow(kern);
     if (e != cudaSuccess) return e;
   }
   kern<<<grid, threads, smem, st>>>(a);
@@ -490,7 +491,8 @@ cudaError_t launch_step_t(const PartStep& S, int sms, cudaStream_t st) {
     const int64_t items = int64_t(S.d) * S.A;
     if (std::is_same<TX, int32_t>::value && std::is_same<TV, int32_t>::value && S.vec && S.w >= 1024 &&
         items >= int64_t(sms) * kBulkWarps) {  // long int32 rows, enough of them: stream them in bulk
-      cudaError_t e = cudaFuncSetAttribute(k_part_dot_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kBulkSmem));
+      static SmemLimit limit;
+      cudaError_t e = limit.allow(k_part_dot_bulk);
       if (e != cudaSuccess) return e;
       const int64_t grid = std::min<int64_t>((items + kBulkWarps - 1) / kBulkWarps, int64_t(sms));
       k_part_dot_bulk<<<unsigned(grid), kBulkWarps * 32, size_t(kBulkSmem), st>>>(S);
