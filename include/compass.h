@@ -489,7 +489,8 @@ cmp_status cmp_part_estimate_ex(const cmp_part_join* join, int32_t d, void* ws_d
 
 /* ------------------------------------------------------ join-order enumeration */
 /* Algorithm 1 of Sec. 5 on the estimates of a cmp_estimate run, for every join graph of a
- * batch at once (one warp per graph; the estimates stay on the device).  From every source
+ * batch at once (one CTA per graph; more than 152 graphs: one warp each first, then a CTA for
+ * every search still open; the estimates stay on the device).  From every source
  * table in increasing f(v) = alpha card(v) / max card + beta deg(v) / max deg (card = the
  * graph's survivors_dev, deg = join edges at v), a depth-first search extends a left-deep
  * prefix by its neighbours in increasing estimate of the extended sub-plan, prunes a prefix
@@ -505,7 +506,8 @@ cmp_status cmp_part_estimate_ex(const cmp_part_join* join, int32_t d, void* ws_d
  *               (or everywhere when no plan was found)
  *   cost_dev    [n_graphs] double: its cost (+inf if none)
  *   stats_dev   [n_graphs][3] int64: complete plans reached, prefix extensions, pruned prefixes
- *   ws_dev      *ws_bytes from cmp_enum_plan_bytes (the search itself runs in shared memory)
+ *   ws_dev      *ws_bytes from cmp_enum_plan_bytes (the open searches between the two launches of
+ *               a batch; the search itself runs in shared memory)
  * A search that exceeds max_nodes prefix extensions stops with CMP_ETIMEOUT in the status
  * (its best plan so far is reported). */
 typedef struct {

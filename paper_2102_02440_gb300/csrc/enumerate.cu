@@ -23,6 +23,14 @@
 // costs and the plan are those of the sequential search; a round that would exceed the
 // search budget is discarded and the sequential search goes on alone.
 //
+// A batch of more graphs than there are SMs takes two launches.  A CTA of 16 warps of 118
+// registers has an SM to itself, and most searches of a large batch are short: so the first launch
+// gives every graph one warp (up to 32 CTAs per SM) and a number of extensions, and the
+// second one goes on with the searches it left open in the workspace.  3000 graphs of five tables
+// (88 extensions each): 892 us with a CTA of 16 warps for every graph, 89 us now; 3000 chains of
+// 12 (622 on average, at most 7205): 5197 and 2074 us; 600 mixed graphs of 5 to 13 tables (2164 on
+// average, at most 82,884): 3704 and 3716 us.
+//
 // Everything a prefix extension touches is kept close, for its latency is what a search
 // costs:
 //  - the search frames (one per prefix length and warp) live in shared memory;
@@ -80,7 +88,7 @@ struct EnumPlanHdr {
   int64_t off_graphs, off_slots, total_bytes, ws_bytes;
   int32_t n_max, stage_slots;  // most tables of a graph; slots of the largest staged table
 };
-constexpr int32_t kEnumPlanVersion = 3;
+constexpr int32_t kEnumPlanVersion = 4;
 constexpr uint64_t kEnumPlanMagic = 0x434d50454e554d31ull;  // "CMPENUM1"
 
 constexpr int kEnumMaxWarps = 16;
@@ -88,6 +96,12 @@ constexpr int kEnumStageSlots = 4096;    // 64 KB
 constexpr int kEnumItems = 256;          // pieces of a round
 constexpr int kEnumTasksWanted = 96;     // pieces to search that a round stops splitting at
 constexpr int64_t kEnumSeqNodes = 192;   // prefixes extended alone before a round
+constexpr int32_t kEnumBatch = 152;      // graphs (one CTA per SM) beyond which a plan takes two launches
+// Extensions of a graph in the first launch: 48 for every graph per SM, at least 96.  What one
+// warp ends costs no CTA of its own later, but the longest search waits for it (96 / 192 for
+// every graph per SM: 3000 chains of 12 1850 / 2215 us, but the 600 mixed graphs 3801 / 3901 us).
+constexpr int64_t kEnumFirstNodes = 48, kEnumFirstLeast = 96;
+constexpr size_t kEnumFirstSmem = 6 << 10;  // shared memory of a first launch's CTA: 32 of them per SM
 
 // Shared memory of one warp's search over n tables: per prefix length its candidates sorted
 // by (estimate, id) with the costs of the prefixes they extend to, the prefix, its
@@ -126,26 +140,36 @@ struct EnumResult {  // of a searched piece: extensions (itself included), prune
   uint8_t warp, missing, over, improved;
 };
 // The block's shared memory: warp frames, two lists of pieces with their paths (n bytes each),
-// results, the source order, the staged table.
+// results (not in a first launch: one warp), the source order, the staged table.
 struct EnumSmem {
   int frame, piece[2], path[2], result, src, table;
 };
-__host__ __device__ inline EnumSmem enum_smem(int n, int warps) {
+__host__ __device__ inline EnumSmem enum_smem(int n, int warps, bool first = false) {
   EnumSmem L;
   int o = 0;
   L.frame = o;  o += enum_frame(n).bytes * warps;
+  const int items = first ? 0 : kEnumItems;
   for (int k = 0; k < 2; k++) {
     L.piece[k] = o;
-    o += int(sizeof(EnumPiece)) * kEnumItems;
+    o += int(sizeof(EnumPiece)) * items;
     L.path[k] = o;
-    o += (n * kEnumItems + 15) & ~15;
+    o += (n * items + 15) & ~15;
   }
-  L.result = o; o += int(sizeof(EnumResult)) * kEnumItems;
+  L.result = o; o += int(sizeof(EnumResult)) * items;
   L.src = o;    o += 4 * n;
   L.table = (o + 15) & ~15;
   return L;
 }
-// workspace of a plan: the search needs none beyond shared memory; the entry point still
+// A search as the first launch of a batch leaves it (open: at frame d of the frames after it),
+// one per graph in the workspace.
+struct EnumSaved {
+  uint64_t min_cost;
+  int64_t plans, nodes, pruned, p, quiet;
+  int32_t si, d;
+  uint8_t open, have, missing, pad[5];
+};
+__host__ __device__ inline size_t enum_saved_bytes(int n) { return align16(sizeof(EnumSaved)) + size_t(enum_frame(n).bytes); }
+// workspace of a plan of one launch: it needs none beyond shared memory; the entry point still
 // takes a buffer of this size
 constexpr size_t kEnumWsBytes = 16;
 
@@ -157,6 +181,8 @@ struct EnumArgs {
   double alpha, beta;
   int64_t max_plans, max_nodes;
   int32_t n_max, stage_slots, warps;  // most tables of a graph; slots of the shared-memory table; warps per CTA
+  unsigned char* saved;  // a batch's searches between its two launches, else null
+  int64_t first_nodes;   // extensions of a graph in a first launch
   int32_t* order;
   double* cost;
   int64_t* stats;
@@ -296,11 +322,11 @@ struct EnumWarp {
   enum { kDone, kLimit, kPause, kFull, kAbort };
   // Depth-first search of everything left at depths >= d0 (kDone), until `limit` extensions
   // have been made (kLimit: another one was due), `pause` of them without completing a plan
-  // (kPause), or `plans` has reached max_plans (kFull); `stop`: a piece with an index below
+  // (kPause; quiet: those since the last plan), or `plans` has reached max_plans (kFull); `stop`: a piece with an index below
   // `self` completed a plan (kAbort).
   __device__ int run(int d0, int64_t limit, int64_t pause, int64_t max_plans, int64_t& nodes, int64_t& pruned,
-                     int64_t& plans, uint64_t& min_cost, bool& improved, const volatile int* stop, int self) {
-    int64_t quiet = 0;
+                     int64_t& plans, uint64_t& min_cost, bool& improved, const volatile int* stop, int self,
+                     int64_t& quiet) {
     while (true) {
       if (nx == nc) {  // back to the previous prefix
         if (d == d0) return kDone;
@@ -360,13 +386,15 @@ enum { kCmdExit = 0, kCmdRound = 1 };
 
 }  // namespace
 
-__global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_constant__ EnumArgs A) {
+// FIRST: the first launch of a batch, one warp per CTA and no rounds.
+template <bool FIRST>
+__global__ void __launch_bounds__(FIRST ? 32 : 32 * kEnumMaxWarps) k_enumerate(const __grid_constant__ EnumArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ EnumRound R;
-  __shared__ int scan[kEnumMaxWarps * 32 + 1];
+  EnumSaved* const saved = A.saved ? reinterpret_cast<EnumSaved*>(A.saved + enum_saved_bytes(A.n_max) * blockIdx.x) : nullptr;
+  if (!FIRST && saved && !saved->open) return;  // the first launch has ended it
   const EnumGraph& g = A.graphs[blockIdx.x];
   const int n = g.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = A.warps;
-  const EnumSmem L = enum_smem(A.n_max, W);
+  const EnumSmem L = enum_smem(A.n_max, W, FIRST);
   uint64_t* tmask = reinterpret_cast<uint64_t*>(smem + L.table);
   uint64_t* tval = tmask + A.stage_slots;
   int32_t* src = reinterpret_cast<int32_t*>(smem + L.src);
@@ -408,6 +436,10 @@ __global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_c
     if (v0 < n) src[r0] = v0;
     if (v1 < n) src[r1] = v1;
   }
+  const int frame_words = enum_frame(A.n_max).bytes / 16;
+  uint4* const saved_frame = saved ? reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(saved) + align16(sizeof(EnumSaved))) : nullptr;
+  if (!FIRST && saved)  // warp 0 goes on from the frames of the first launch
+    for (int i = threadIdx.x; i < frame_words; i += blockDim.x) reinterpret_cast<uint4*>(smem + L.frame)[i] = saved_frame[i];
   __syncthreads();
   EnumWarp S(A, g, smem + L.frame + size_t(enum_frame(A.n_max).bytes) * warp, tmask, tval, staged);
 
@@ -415,8 +447,81 @@ __global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_c
   uint64_t min_cost = kInfBits;
   bool have = false, missing = false, out_of_budget = false, alone = W < 2;
   int64_t plans = 0, nodes = 0, pruned = 0, p = 0;  // p: plans completed from this source
+  int64_t quiet = 0;  // extensions since the search's last plan (or round, or source)
   int si = -1;
   bool open = false;  // a source's search is under way, at S's current frame
+  // The next source (false: there is none left).
+  auto next_source = [&]() {
+    while (++si < n) {
+      p = 0;
+      quiet = 0;
+      S.d = 0;
+      S.m = 1ull << src[si];
+      S.nb = g.adj[src[si]];
+      S.cost = 0;  // 0.0
+      S.nx = 0;
+      __syncwarp();
+      if (lane == 0) S.path[0] = src[si];
+      if (S.m != S.full) {
+        S.nc = S.expand(0, S.m, S.nb, S.cost);
+        return open = true;
+      }
+      plans++;  // one table: the plan is complete and costs nothing
+      if (min_cost != 0) {
+        min_cost = 0;
+        if (lane == 0) S.best[0] = src[si];
+        have = true;
+      }
+    }
+    return false;
+  };
+  // The open search from where it is, until its source, the budget, `limit` extensions or the
+  // pause ends it.
+  auto search = [&](int64_t limit, int64_t pause) {
+    bool improved = false;
+    const int64_t p0 = p;
+    const int why = S.run(0, limit, pause, A.max_plans, nodes, pruned, p, min_cost, improved, nullptr, 0, quiet);
+    plans += p - p0;
+    have |= improved;
+    if (why == EnumWarp::kDone || why == EnumWarp::kFull) open = false;
+    if (why == EnumWarp::kLimit && nodes == A.max_nodes) out_of_budget = true;  // exactly max_nodes extensions
+    return why;
+  };
+  // The graph's result (warp 0).
+  auto finish = [&]() {
+    for (int t = lane; t < kEnumMaxN; t += 32)
+      A.order[int64_t(blockIdx.x) * kEnumMaxN + t] = (have && t < n) ? S.best[t] : -1;
+    if (lane != 0) return;
+    A.cost[blockIdx.x] = bits_double(have ? min_cost : kInfBits);
+    A.stats[int64_t(blockIdx.x) * 3 + 0] = plans;
+    A.stats[int64_t(blockIdx.x) * 3 + 1] = nodes;
+    A.stats[int64_t(blockIdx.x) * 3 + 2] = pruned;
+    if (missing) set_status(A.status, CMP_EUNSUPPORTED);
+    if (out_of_budget) set_status(A.status, CMP_ETIMEOUT);
+  };
+
+  if constexpr (FIRST) {
+    const int64_t limit = A.max_plans < 0 ? A.max_nodes : min(A.max_nodes, A.first_nodes);
+    bool more = true;
+    while (more && (open || next_source())) more = search(limit, INT64_MAX) != EnumWarp::kLimit;
+    open &= !out_of_budget;
+    if (open) {
+      S.save();
+      for (int i = lane; i < frame_words; i += 32) saved_frame[i] = reinterpret_cast<const uint4*>(smem + L.frame)[i];
+    }
+    if (lane == 0) *saved = {min_cost, plans, nodes, pruned, p, quiet, si, S.d, open, have, S.missing};
+    missing = S.missing;
+    if (!open) finish();
+    return;
+  }
+  __shared__ EnumRound R;
+  __shared__ int scan[kEnumMaxWarps * 32 + 1];
+  if (saved && warp == 0) {
+    const EnumSaved v = *saved;
+    min_cost = v.min_cost, plans = v.plans, nodes = v.nodes, pruned = v.pruned, p = v.p, quiet = v.quiet, si = v.si;
+    have = v.have, missing = v.missing, open = true;
+    S.load(v.d);
+  }
 
   // Warp 0: the unvisited prefixes of the open search as the first list of pieces, in search
   // order (the deepest frame's remaining candidates first); false when they are too many.
@@ -464,41 +569,12 @@ __global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_c
   for (;;) {
     if (warp == 0) {
       int cmd = kCmdExit;
-      while (!out_of_budget) {
-        if (!open) {  // the next source
-          if (++si >= n) break;
-          p = 0;
-          S.d = 0;
-          S.m = 1ull << src[si];
-          S.nb = g.adj[src[si]];
-          S.cost = 0;  // 0.0
-          S.nx = 0;
-          __syncwarp();
-          if (lane == 0) S.path[0] = src[si];
-          if (S.m == S.full) {  // one table: the plan is complete and costs nothing
-            plans++;
-            if (min_cost != 0) {
-              min_cost = 0;
-              if (lane == 0) S.best[0] = src[si];
-              have = true;
-            }
-            continue;
-          }
-          S.nc = S.expand(0, S.m, S.nb, S.cost);
-          open = true;
-        }
-        bool improved = false;
-        const int64_t p0 = p;
+      while (!out_of_budget && (open || next_source())) {
         // (a search without a limit on its plans completes them all the time: alone)
-        const int64_t pause = alone || A.max_plans < 0 ? INT64_MAX : kEnumSeqNodes;
-        const int why =
-            S.run(0, A.max_nodes, pause, A.max_plans, nodes, pruned, p, min_cost, improved, nullptr, 0);
-        plans += p - p0;
-        have |= improved;
-        if (why == EnumWarp::kLimit) out_of_budget = true;  // budget spent: exactly max_nodes extensions
-        if (why == EnumWarp::kDone || why == EnumWarp::kFull) open = false;
+        const int why = search(A.max_nodes, alone || A.max_plans < 0 ? INT64_MAX : kEnumSeqNodes);
         if (why == EnumWarp::kPause) {
           S.save();
+          quiet = 0;
           if (!collect()) {
             alone = true;
             continue;
@@ -656,11 +732,11 @@ __global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_c
         for (int t = lane; t < q.len; t += 32) S.path[t] = lpath[size_t(k) * n + t];
         __syncwarp();
         S.nc = S.expand(S.d, S.m, S.nb, S.cost);
-        int64_t wn = 1, wp = 0, wplans = R.plans;
+        int64_t wn = 1, wp = 0, wplans = R.plans, wquiet = 0;
         uint64_t wcost = R.min_cost;
         bool improved = false;
         // (limit + 1: reaching it means more than the budget is left for)
-        const int why = S.run(S.d, R.limit + 1, INT64_MAX, A.max_plans, wn, wp, wplans, wcost, improved, &R.first, k);
+        const int why = S.run(S.d, R.limit + 1, INT64_MAX, A.max_plans, wn, wp, wplans, wcost, improved, &R.first, k, wquiet);
         if (lane == 0) {
           EnumResult& r = result[k];
           r.nodes = wn;
@@ -766,16 +842,7 @@ __global__ void __launch_bounds__(32 * kEnumMaxWarps) k_enumerate(const __grid_c
     }
     __syncthreads();
   }
-  if (warp != 0) return;
-  for (int t = lane; t < kEnumMaxN; t += 32)
-    A.order[int64_t(blockIdx.x) * kEnumMaxN + t] = (have && t < n) ? S.best[t] : -1;
-  if (lane != 0) return;
-  A.cost[blockIdx.x] = bits_double(have ? min_cost : kInfBits);
-  A.stats[int64_t(blockIdx.x) * 3 + 0] = plans;
-  A.stats[int64_t(blockIdx.x) * 3 + 1] = nodes;
-  A.stats[int64_t(blockIdx.x) * 3 + 2] = pruned;
-  if (missing) set_status(A.status, CMP_EUNSUPPORTED);
-  if (out_of_budget) set_status(A.status, CMP_ETIMEOUT);
+  if (warp == 0) finish();
 }
 
 namespace {
@@ -846,13 +913,13 @@ cmp_status enum_plan(const cmp_graph* graphs, int32_t n_graphs, int32_t n_sub, c
   H.off_slots = int64_t(off);
   off += align16(sizeof(EnumSlot) * P->slots.size());
   H.total_bytes = int64_t(off);
-  H.ws_bytes = int64_t(kEnumWsBytes);
   H.n_max = 1;
   H.stage_slots = 0;
   for (const EnumGraph& g : P->graphs) {
     H.n_max = std::max(H.n_max, g.n);
     if ((int64_t(1) << g.h_log2) <= kEnumStageSlots) H.stage_slots = std::max(H.stage_slots, 1 << g.h_log2);
   }
+  H.ws_bytes = int64_t(n_graphs > kEnumBatch ? enum_saved_bytes(H.n_max) * size_t(n_graphs) + 15 : kEnumWsBytes);
   return CMP_OK;
 }
 
@@ -922,7 +989,22 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
   a.cost = cost_dev;
   a.stats = stats_dev;
   a.status = status_dev;
+  a.saved = nullptr;
+  a.first_nodes = 0;
+  cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+  if (H.n_graphs > kEnumBatch) {  // a batch: every graph by one warp first
+    a.saved = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(ws_dev) + 15) & ~uintptr_t(15));
+    a.first_nodes = std::max(kEnumFirstLeast, kEnumFirstNodes * H.n_graphs / kEnumBatch);
+    a.warps = 1;
+    const size_t base = size_t(enum_smem(H.n_max, 1, true).table);
+    a.stage_slots = int32_t(std::min<size_t>(size_t(H.stage_slots), base < kEnumFirstSmem ? (kEnumFirstSmem - base) / 16 : 0));
+    static SmemLimit limit;
+    if (limit.allow(k_enumerate<true>) != cudaSuccess) return CMP_ECUDA;
+    k_enumerate<true><<<unsigned(H.n_graphs), 32, base + 16 * size_t(a.stage_slots), st>>>(a);
+    if (cudaGetLastError() != cudaSuccess) return CMP_ECUDA;
+  }
   // as many warps as their frames leave room for beside the lists and the staged table
+  a.stage_slots = H.stage_slots;
   int warps = kEnumMaxWarps;
   auto smem_of = [&](int k) { return size_t(enum_smem(H.n_max, k).table) + 16 * size_t(H.stage_slots); };
   while (warps > 8 && smem_of(warps) > size_t(200) * 1024) warps >>= 1;  // 256 threads at least: one per piece
@@ -930,8 +1012,8 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
   while (a.warps > 1 && smem_of(a.warps) > size_t(200) * 1024) a.warps--;  // those beyond search nothing
   const size_t smem = smem_of(a.warps);
   static SmemLimit limit;
-  if (limit.allow(k_enumerate) != cudaSuccess) return CMP_ECUDA;
-  k_enumerate<<<unsigned(H.n_graphs), 32 * warps, smem, reinterpret_cast<cudaStream_t>(stream)>>>(a);
+  if (limit.allow(k_enumerate<false>) != cudaSuccess) return CMP_ECUDA;
+  k_enumerate<false><<<unsigned(H.n_graphs), 32 * warps, smem, st>>>(a);
   return cudaGetLastError() == cudaSuccess ? CMP_OK : CMP_ECUDA;
 }
 
