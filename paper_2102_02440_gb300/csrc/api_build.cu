@@ -294,12 +294,11 @@ struct BuildPlanParts {
   std::vector<AggCol> aggs;
   std::vector<CountItem> cnt_items;
   int64_t cnt_total_chunks = 0;
-  int32_t cnt_grid = 0;
+  int32_t cnt_grid[4] = {0, 0, 0, 0};
   int64_t cnt_sampled = 0;   // first chunk of the tables with a row sample and no predicates
   int64_t cnt_filtered = 0;  // first chunk of the tables with predicates
-  int64_t cnt_split = 0;  // > 0: two launches, the tables with presence columns first
-  int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the second counting launch
-  int32_t cnt_grid_b = 0;
+  int64_t cnt_split = 0;  // > 0: the tables with presence columns in a launch before the others
+  int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the last counting launch
   int64_t hash_items = 0;
   int32_t hash_private = 0;
   int32_t hash_grid = 0;
@@ -692,60 +691,72 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
   // make up a CTA's share of each kind, and a cache has at most one slot per 16 rows of a
   // chunk.  (Chunks of 16,384 rows with caches of 8192 slots sent 103 M of 162.5 M keys of 58
   // tables to L2.)
-  auto count_kind = [&](int32_t t) {  // 0 presence columns, 1 every row, 2 a sample, 3 predicates, -1 not counted
+  auto count_kind = [&](int32_t t) {  // kCnt*, -1: not counted
     int ncol = 0;
     for (int32_t c = 0; c < CMP_MAX_COLS; c++) ncol += P->col_agg[t][c] >= 0;
     if (!ncol) return -1;
-    if (has_presence(t)) return 0;
-    return tables[t].n_preds > 0 ? 3 : (sample_keep_of(tables[t].sample_rate) != 0 ? 2 : 1);
+    if (has_presence(t)) return int(kCntPresence);
+    if (tables[t].n_preds > 0) return int(kCntFiltered);
+    return sample_keep_of(tables[t].sample_rate) != 0 ? int(kCntSampled) : int(kCntWhole);
   };
   int64_t kind_rows[4] = {0, 0, 0, 0};
   for (int32_t t = 0; t < n_tables; t++)
     if (count_kind(t) >= 0) kind_rows[count_kind(t)] += tables[t].n_rows;
   const int64_t cnt_ctas = int64_t(sm_count()) * (P->uitems.empty() ? 2 : 1);
   for (int pass = 0; pass < 4; pass++) {
-  if (pass == 2) P->cnt_sampled = P->cnt_total_chunks;
-  if (pass == 3) P->cnt_filtered = P->cnt_total_chunks;
-  for (int32_t t = 0; t < n_tables; t++) {
-    if (count_kind(t) != pass) continue;
-    CountItem ci;
-    ci.table = t;
-    const int64_t unit = 4 * int64_t(R);
-    const int64_t want = std::max(tables[t].n_rows / (int64_t(sm_count()) * 2 * 16),
-                                  kind_rows[pass] / (cnt_ctas * kCountChunksPerCta));
-    ci.chunk_rows = unit * std::max<int64_t>(1, std::min<int64_t>(16, want / unit));
-    ci.cache_slots = P->cache_slots;
-    while (ci.cache_slots > 256 && 16 * int64_t(ci.cache_slots) > std::min(ci.chunk_rows, tables[t].n_rows))
-      ci.cache_slots >>= 1;
-    ci.chunk_begin = P->cnt_total_chunks;
-    ci.n_chunks = (tables[t].n_rows + ci.chunk_rows - 1) / ci.chunk_rows;
-    P->cnt_total_chunks += ci.n_chunks;
-    if (pass == 0) presence_chunks += ci.n_chunks;
-    P->cnt_items.push_back(ci);
+    if (pass == kCntSampled) P->cnt_sampled = P->cnt_total_chunks;
+    if (pass == kCntFiltered) P->cnt_filtered = P->cnt_total_chunks;
+    for (int32_t t = 0; t < n_tables; t++) {
+      if (count_kind(t) != pass) continue;
+      CountItem ci;
+      ci.table = t;
+      const int64_t unit = 4 * int64_t(R);
+      const int64_t want = std::max(tables[t].n_rows / (int64_t(sm_count()) * 2 * 16),
+                                    kind_rows[pass] / (cnt_ctas * kCountChunksPerCta));
+      ci.chunk_rows = unit * std::max<int64_t>(1, std::min<int64_t>(16, want / unit));
+      ci.cache_slots = P->cache_slots;
+      while (ci.cache_slots > 256 && 16 * int64_t(ci.cache_slots) > std::min(ci.chunk_rows, tables[t].n_rows))
+        ci.cache_slots >>= 1;
+      ci.chunk_begin = P->cnt_total_chunks;
+      ci.n_chunks = (tables[t].n_rows + ci.chunk_rows - 1) / ci.chunk_rows;
+      P->cnt_total_chunks += ci.n_chunks;
+      if (pass == kCntPresence) presence_chunks += ci.n_chunks;
+      P->cnt_items.push_back(ci);
+    }
   }
-  }
-  P->cnt_grid = 0;  // set below, once the unique-key items are known
-  // counting pass: 512-thread CTAs, two per SM; one per SM when the unique-key kernel runs
-  // beside it
-  P->cnt_grid = int32_t(std::min<int64_t>(P->cnt_total_chunks, int64_t(sm_count()) * (P->uitems.empty() ? 2 : 1)));
   // split pass: when presence bitmaps and other counted tables are both present (and no
   // unique-key kernel wants the place beside the counting pass), the bitmaps are counted
-  // first, then the rest with one CTA per SM and the dense kernel beside it
+  // first, then the rest with the dense kernel beside its last launch
   P->cnt_split = 0;
-  P->cnt_grid_b = 0;
   P->d_cut = 1024;
-  if (!P->ditems.empty() && P->uitems.empty() && presence_chunks > 0 && presence_chunks < P->cnt_total_chunks) {
+  if (!P->ditems.empty() && P->uitems.empty() && presence_chunks > 0 && presence_chunks < P->cnt_total_chunks)
     P->cnt_split = presence_chunks;
-    P->cnt_grid = int32_t(std::min<int64_t>(presence_chunks, int64_t(sm_count()) * 2));
-    P->cnt_grid_b = int32_t(std::min<int64_t>(P->cnt_total_chunks - presence_chunks, int64_t(sm_count())));
-    // The dense kernel's share beside the second counting launch: the part it walks while
-    // that launch scans (the rest runs after it, two warps per scheduler instead of one).  The
+  // Counting pass: 512-thread CTAs, two per SM; one per SM in the launch that the unique-key or
+  // the dense kernel runs beside: the last one (in the order of cmp_sketch_build_batched: split,
+  // predicates come last; else the whole tables do).  The launches before it scan alone: two
+  // CTAs per SM where rows are selected (two tables of 40 M rows: 324 us with one, 203 with two;
+  // sampled 298 and 208), still one for whole tables (286 and 285 us; of 10 M rows 83 and 100:
+  // each CTA writes its own hot-key caches out).
+  const int64_t kind_begin[5] = {0, P->cnt_split, P->cnt_sampled, P->cnt_filtered, P->cnt_total_chunks};
+  int last = -1;
+  for (int k = kCntWhole; k <= kCntFiltered; k++)
+    if (kind_begin[k + 1] > kind_begin[k] && (P->cnt_split > 0 || last < 0)) last = k;
+  for (int k = kCntPresence; k <= kCntFiltered; k++) {
+    const bool shared = P->cnt_split > 0 || !P->uitems.empty();  // a kernel runs beside the last one
+    const int per_sm = shared && (k == last || k == kCntWhole) ? 1 : 2;
+    P->cnt_grid[k] = int32_t(std::min<int64_t>(kind_begin[k + 1] - kind_begin[k], int64_t(sm_count()) * per_sm));
+  }
+  if (P->cnt_split > 0) {
+    // The dense kernel's share beside the last counting launch: the part it walks while that
+    // launch scans (the rest runs after it, two warps per scheduler instead of one).  The
     // scan's time is its columns' bytes at ~4.7 TB/s; the walk beside it advances at ~0.7 of
     // its ~320 G key x row steps/s alone (GB300 measurements of the 1e9-row workload, whose
-    // best share, 0.75, this gives).
+    // best share, 0.75, this gives).  Counted are the columns of all launches after the
+    // bitmaps': with those of the last one only, whose smaller tables scan slower than that
+    // rate, whole tables and predicates beside presence columns took 2% longer.
     double bytes_b = 0, steps = 0;
     for (const CountItem& ci : P->cnt_items) {
-      if (ci.chunk_begin < presence_chunks) continue;
+      if (ci.chunk_begin < P->cnt_split) continue;
       const cmp_table& tb = tables[ci.table];
       uint32_t used = 0;  // referenced columns: aggregated keys and predicates
       for (int32_t c = 0; c < CMP_MAX_COLS; c++)
@@ -853,12 +864,11 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.u_words = P.u_words;
   h.u_tile_rows = kUniqTileRows;
   h.cnt_total_chunks = P.cnt_total_chunks;
-  h.cnt_grid = P.cnt_grid;
+  std::copy(P.cnt_grid, P.cnt_grid + 4, h.cnt_grid);
   h.cnt_split = P.cnt_split;
   h.cnt_sampled = P.cnt_sampled;
   h.cnt_filtered = P.cnt_filtered;
   h.hash_private = P.hash_private;
-  h.cnt_grid_b = P.cnt_grid_b;
   h.d_cut = P.d_cut;
   h.cnt_threads = 512;
   h.cnt_cache_slots = P.cache_slots;
@@ -949,15 +959,15 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
   const int32_t hash_grid = h.n_agg > 0 ? h.hash_grid : 0;
   const int32_t d_grid = h.n_ditems > 0 ? h.d_grid : 0;
   if (h.cnt_split > 0) {
-    // the tables with presence columns, then the others with the dense kernel beside them
-    // (its programmatic dependent: one CTA of each per SM, a memory-bound scan beside an
+    // the tables with presence columns, then the others with the dense kernel beside the last
+    // of them (its programmatic dependent: one CTA of each per SM, a memory-bound scan beside an
     // integer-bound walk; every bitmap is complete before the second launch starts)
-    if (launch_count_rows(a, false, h.cnt_grid, 0, 0, h.cnt_split, cs) != cudaSuccess ||
+    if (launch_count_rows(a, false, h.cnt_grid[kCntPresence], 0, 0, h.cnt_split, cs) != cudaSuccess ||
         launch_presence_check(a, cs) != cudaSuccess ||
-        launch_count_rows(a, false, h.cnt_grid_b, 2, h.cnt_split, h.cnt_sampled, cs) != cudaSuccess ||
-        launch_count_rows(a, true, h.cnt_grid_b, 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
-        launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid_b, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
-            cudaSuccess)
+        launch_count_rows(a, false, h.cnt_grid[kCntWhole], 2, h.cnt_split, h.cnt_sampled, cs) != cudaSuccess ||
+        launch_count_rows(a, true, h.cnt_grid[kCntSampled], 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
+        launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid[kCntFiltered], 3, h.cnt_filtered,
+                         h.cnt_total_chunks, cs) != cudaSuccess)
       return CMP_ECUDA;
     // the dense kernel: its share beside the counting launch, then the rest with 512 threads
     // (programmatic dependents both: the second takes each SM the first two leave)
@@ -973,10 +983,10 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     return launch_agg_hash(a, hash_grid, cs) == cudaSuccess ? CMP_OK : CMP_ECUDA;
   }
   if (h.n_agg > 0 &&
-      (launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid, 3, h.cnt_filtered, h.cnt_total_chunks, cs) !=
-           cudaSuccess ||
-       launch_count_rows(a, true, h.cnt_grid, 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
-       launch_count_rows(a, false, h.cnt_grid, 0, 0, h.cnt_sampled, cs) != cudaSuccess))
+      (launch_agg_count(a, h.shape.tile_rows, h.cnt_threads, h.cnt_grid[kCntFiltered], 3, h.cnt_filtered,
+                        h.cnt_total_chunks, cs) != cudaSuccess ||
+       launch_count_rows(a, true, h.cnt_grid[kCntSampled], 4, h.cnt_sampled, h.cnt_filtered, cs) != cudaSuccess ||
+       launch_count_rows(a, false, h.cnt_grid[kCntWhole], 0, 0, h.cnt_sampled, cs) != cudaSuccess))
     return CMP_ECUDA;
   // the unique-key kernel right after the counting pass, as its programmatic dependent:
   // one CTA of each per SM, the two overlap (memory-bound scan, integer-bound hashing)

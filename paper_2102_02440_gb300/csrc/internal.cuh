@@ -471,7 +471,7 @@ struct BuildPlanHdr {
   int64_t total_bytes;
   int64_t n_agg, off_agg;                            // aggregated key columns
   int64_t n_cnt_items, off_cnt_items, cnt_total_chunks;  // counting pass
-  int32_t cnt_grid, cnt_threads;
+  int32_t cnt_grid[4], cnt_threads;  // CTAs of each launch of the counting pass (kCnt*)
   int64_t ws_bytes;
   int32_t cnt_cache_slots, cnt_cache_cols;
   int64_t hash_items;
@@ -481,18 +481,21 @@ struct BuildPlanHdr {
   int32_t u_grid, u_pack16, u_words, u_tile_rows;
   int64_t n_dslab, off_dslab, n_ditems, off_ditems, off_d_cta;  // dense kernel
   int32_t d_grid, d_pack16, d_words, n_presence;
-  // counting pass in two launches (cnt_split > 0): chunks [0, cnt_split) of the tables with
-  // presence columns first, then [cnt_split, total) with the dense kernel beside it
+  // split counting pass (cnt_split > 0): chunks [0, cnt_split) of the tables with presence
+  // columns first, then [cnt_split, total) with the dense kernel beside their last launch
   int64_t cnt_split;
   // split pass: the dense kernel walks the first d_cut / 1024 of each item's runs beside the
-  // second counting launch, the rest after it with 512 threads (d_cut = 1024: all beside)
-  int32_t cnt_grid_b, d_cut;
+  // last counting launch, the rest after it with 512 threads (d_cut = 1024: all beside)
+  int32_t d_cut, pad;
   // chunks: tables with presence columns and without a selection, from cnt_sampled on tables with a
   // row sample only (k_count_rows), from cnt_filtered on tables with predicates (k_agg_count)
   int64_t cnt_sampled;
   int64_t cnt_filtered;
 };
-constexpr int32_t kBuildPlanVersion = 13;
+constexpr int32_t kBuildPlanVersion = 14;
+// Launches of the counting pass: tables with presence columns (of a split pass; else they are
+// counted with the whole ones), every row, a row sample, predicates.
+enum { kCntPresence = 0, kCntWhole = 1, kCntSampled = 2, kCntFiltered = 3 };
 struct ZeroSpan {
   void* ptr;
   int64_t bytes;
