@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kStarThreads) k_star_suf(const __grid_constant
 // (reduced at the end), J = E / Ep entries per thread.  Shared memory per chunk of kStarR
 // positions: B[r][v2], A[r][v1] (int128 with byte flags), the factors f[j][r] and w[r].
 // Bound by integer issue: 52 instructions per multiply-add.
-__device__ __noinline__ void star_unit_int128(const EstArgs& A, const StarUnit& u, unsigned char* smem) {
+__device__ __forceinline__ void star_unit_int128(const EstArgs& A, const StarUnit& u, unsigned char* smem) {
   constexpr int R = kStarR, NB = 1 << kStarMaxK2;
   i128* Bs = reinterpret_cast<i128*>(smem);                      // [R][256]
   i128* As = Bs + R * NB;                                          // [R][16]
@@ -335,7 +335,7 @@ __device__ __forceinline__ void group_sync(int g) {
 __host__ __device__ constexpr int rns_group_words(int nx, int ny) { return 256 + 512 + 16 * (nx + ny); }
 
 template <int G>
-__device__ __noinline__ void star_unit_rns(const EstArgs& A, const StarUnit& u, const StarFam& F, const RnsUnit& U,
+__device__ __forceinline__ void star_unit_rns(const EstArgs& A, const StarUnit& u, const StarFam& F, const RnsUnit& U,
                                            int n_primes, unsigned char* smem) {
   constexpr int NG = kStarThreads / G, NQ = 256 / G;  // NQ: factor values per thread and chunk
   const int tid = threadIdx.x, g = tid / G, l = tid % G, w = A.w;
@@ -480,8 +480,10 @@ __device__ __noinline__ void star_unit_rns(const EstArgs& A, const StarUnit& u, 
 // T_a(V) for the 2^m1 A-side subsets of block blk (bits m1..k1-1 of V1 = blk) and all 2^k2
 // B-side subsets.  Its sums are bounded by w max_r |w_a(r)| prod_b max(1, |f_ab(r)|): below
 // 2^138 it runs on residues, on as many primes as the bound asks for, else in int128.
-// Stars of 10, 14 and 15 tables (2.0 G multiply-adds at w = 1024, d = 11): 6.13 ms all in int128,
-// 2.68 ms on residues.
+// Stars of 10, 14 and 15 tables (2.0 G multiply-adds at w = 1024, d = 11): 6.16 ms all in int128,
+// 2.53 to 2.82 ms on four and five residues.  The units are inlined: as functions of their own
+// they spilled, and stars beyond 2^138 (three of 10 to 13 tables, up to 8 M rows) took 9.03 ms,
+// 8.30 now (8.68 with an int128 kernel alone).
 __global__ void __launch_bounds__(kStarThreads, 2) k_star_lattice(const __grid_constant__ EstArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ RnsUnit U;
@@ -548,7 +550,7 @@ cudaError_t launch_estimate_star(const EstArgs& a, cudaStream_t st) {
     static SmemLimit limit;
     cudaError_t e = limit.allow(k_star_lattice);
     if (e != cudaSuccess) return e;
-    const int64_t grid = std::min<int64_t>(lat, int64_t(sm_count()) * 2);  // two 80 KB CTAs per SM
+    const int64_t grid = std::min<int64_t>(lat, int64_t(sm_count()) * 2);  // two 102 KB CTAs per SM
     k_star_lattice<<<unsigned(grid), kStarThreads, smem, st>>>(a);
   }
   return cudaGetLastError();
