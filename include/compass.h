@@ -364,7 +364,9 @@ typedef struct {
 typedef struct {
   int32_t threads;     /* threads per CTA (multiple of 32, <= 1024)                */
   int32_t ctas_per_sm; /* resident CTAs per SM the persistent grid is sized for    */
-  int32_t cond_chunk;  /* conditioning values per work item of a cyclic sub-plan   */
+  int32_t cond_chunk;  /* conditioning values per work item of a cyclic sub-plan (0: 64).
+                          Simple cycles of 4 and more tables are evaluated over distinct
+                          sketch values instead when 7 cond_chunk < w <= 4096              */
   int32_t flags;       /* CMP_EST_GENERIC_ONLY | CMP_EST_CACHE_MESSAGES | CMP_EST_STAR_LATTICE |
                           CMP_EST_NO_WIDE; other bits: CMP_EINVAL */
 } cmp_estimate_cfg;

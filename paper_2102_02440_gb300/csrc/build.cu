@@ -364,17 +364,17 @@ __host__ __device__ inline size_t agg_count_surv_entries(int32_t tile_rows, int3
   return tile_rows > 16 * threads ? size_t(tile_rows) : size_t(16) * threads;
 }
 
-// Counting pass of key aggregation over tables with predicates or a row sample (the others:
-// k_count_rows, build_count.cu).  Persistent CTAs take chunks of whole tiles of a table's rows (CountItem.chunk_rows) in order from an atomic counter.  For every surviving
-// row and every aggregated key column of the table, the key's slot (key - base) & mask gets
-// one count (a presence column: its bit is set; a bit found set already makes the column
-// inactive): in the CTA's two-way set-associative shared-memory cache when a way of its set
-// holds that slot index or is free (the frequent keys of a skewed column settle there),
-// else with one global atomic on the count array.  Caches are added to the count arrays
-// when the CTA moves to another table or ends.  The pass also records each column's
-// smallest and largest surviving key (thread-local, then warp and CTA reductions, then one
-// global atomic pair per column and table visit; a declared domain stands for them), and
-// counts the table's survivors.
+// Counting pass of key aggregation over tables with predicates, and perhaps a row sample (the
+// others, and every presence column: k_count_rows, build_count.cu).  Persistent CTAs take
+// chunks of whole tiles of a table's rows (CountItem.chunk_rows) in order from an atomic
+// counter.  For every surviving row and every aggregated key column of the table, the key's
+// slot (key - base) & mask gets one count: in the CTA's two-way set-associative shared-memory
+// cache when a way of its set holds that slot index or is free (the frequent keys of a
+// skewed column settle there), else with one global atomic on the count array.  Caches are
+// added to the count arrays when the CTA moves to another table or ends.  The pass also
+// records each column's smallest and largest surviving key (thread-local, then warp and CTA
+// reductions, then one global atomic pair per column and table visit; a declared domain
+// stands for them), and counts the table's survivors.
 __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ BuildArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   // The unique-key kernel, launched next as a programmatic dependent, reads nothing this
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
   __shared__ int32_t* acnt[CMP_MAX_SKETCHES];  // the current table's aggregated columns
   __shared__ int64_t abase[CMP_MAX_SKETCHES], acap[CMP_MAX_SKETCHES];
   __shared__ uint64_t amask[CMP_MAX_SKETCHES];
-  __shared__ int32_t acol[CMP_MAX_SKETCHES], aidx[CMP_MAX_SKETCHES], akind[CMP_MAX_SKETCHES];
+  __shared__ int32_t acol[CMP_MAX_SKETCHES], aidx[CMP_MAX_SKETCHES];
   __shared__ unsigned long long amax[CMP_MAX_SKETCHES], amin[CMP_MAX_SKETCHES];  // encoded
   __shared__ int32_t n_ac;
   __shared__ uint32_t akeys;  // the current table's aggregated key columns (bit c: column c)
@@ -399,7 +399,7 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
   sp += align16(sizeof(uint16_t) * agg_count_surv_entries(R, T));
   int32_t* sint = reinterpret_cast<int32_t*>(sp);
   constexpr uint32_t kEmpty = 0xFFFFFFFFu;  // never a slot index: cap <= 2^31 - 1
-  // this launch's chunk counter: slot 0 (the only launch, or the first of two), 2 (the second)
+  // this launch's chunk counter
   unsigned long long* work = reinterpret_cast<unsigned long long*>(A.ws) + 2 * int64_t(A.n_agg) + A.cnt_work_slot;
 
   // One surviving key of column a.  Returns false when the key lies outside the column's
@@ -428,10 +428,6 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
   auto count_key = [&](int a, int64_t key) {
     const uint64_t off = uint64_t(key) - uint64_t(abase[a]);
     if (amask[a] == ~0ull && off >= uint64_t(acap[a])) return false;
-    if (akind[a] == kAggPresence) {  // off < cap <= 2^32; repeated keys are found by k_presence_check
-      red_or(reinterpret_cast<uint32_t*>(acnt[a]) + (off >> 5), 1u << (off & 31));
-      return true;
-    }
     const uint32_t x = uint32_t(off & amask[a]);  // < cap
     if (a < n_cache && cache_count(ckey + size_t(a) * H, ccnt + size_t(a) * H, x)) return true;
     red_add(acnt[a] + x, 1);
@@ -510,26 +506,22 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
       if (tid == 0) {
         int n = 0;
         uint32_t keys = 0;
-        for (int col = 0; col < tb->n_cols; col++)
-          if (tb->agg[col] >= 0) keys |= 1u << col;
+        for (int col = 0; col < tb->n_cols && n < CMP_MAX_SKETCHES; col++) {
+          const int ai = tb->agg[col];
+          if (ai < 0) continue;
+          keys |= 1u << col;
+          const AggCol& ac = A.agg[ai];
+          acnt[n] = reinterpret_cast<int32_t*>(A.ws + ac.off);
+          abase[n] = ac.base;
+          acap[n] = ac.cap;
+          amask[n] = ac.mask;
+          acol[n] = col;
+          aidx[n] = ai;
+          amax[n] = 0;
+          amin[n] = 0;
+          n++;
+        }
         akeys = keys;
-        // count arrays first (they take the hot-key caches), then presence bitmaps
-        for (int kind = kAggCount; kind <= kAggPresence; kind++)
-          for (int col = 0; col < tb->n_cols && n < CMP_MAX_SKETCHES; col++) {
-            const int ai = tb->agg[col];
-            if (ai < 0 || A.agg[ai].kind != kind) continue;
-            const AggCol& ac = A.agg[ai];
-            acnt[n] = reinterpret_cast<int32_t*>(A.ws + ac.off);
-            abase[n] = ac.base;
-            acap[n] = ac.cap;
-            amask[n] = ac.mask;
-            acol[n] = col;
-            aidx[n] = ai;
-            akind[n] = kind;
-            amax[n] = 0;
-            amin[n] = 0;
-            n++;
-          }
         n_ac = n;
       }
       for (int s = tid; s < H * n_cache; s += T) {
@@ -544,8 +536,7 @@ __global__ void __launch_bounds__(512, 2) k_agg_count(const __grid_constant__ Bu
     const int64_t r_begin = (c - ci.chunk_begin) * ci.chunk_rows, r_end = min(n_rows, r_begin + ci.chunk_rows);
     const bool vec = tb->vec_ok != 0;
     if (vec && !tb->sample_keep && tb->n_preds >= 1 && tb->n_preds <= 2 && nac <= 2 &&
-               tb->dtype[tb->pred[0].col] == CMP_I32 && tb->dtype[tb->pred[tb->n_preds - 1].col] == CMP_I32 &&
-               akind[0] == kAggCount && akind[nac - 1] == kAggCount) {
+        tb->dtype[tb->pred[0].col] == CMP_I32 && tb->dtype[tb->pred[tb->n_preds - 1].col] == CMP_I32) {
       // Warp-autonomous scan in three stages (no block barrier inside the chunk).  Warp w
       // takes the 256-row steps w, w + nwarps, ...; lane l the 16-byte groups at 4 l and 128 +
       // 4 l of a step.  While it counts the survivors of step s (lane e holds the keys of

@@ -394,37 +394,37 @@ __global__ void __launch_bounds__(512, 2) k_count_rows(const __grid_constant__ B
       }
       if (lane == 0 && kept) atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), kept);
     } else {
-    if (tid == 0 && r_end > r_begin)
-      atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), (unsigned long long)(r_end - r_begin));
-    for (int a = 0; a < nac; a++) {
-      const AggCol& ac = agg_of(a);
-      const CntCol cc = cnt_col(a);
-      const bool i32 = tb->dtype[acol[a]] == CMP_I32, presence = ac.kind == kAggPresence;
-      // the slots of an int32 column are 32-bit sums when its domain lies in int32
-      const bool small = !cc.declared || (ac.base >= INT32_MIN && ac.base + ac.cap <= int64_t(INT32_MAX) + 1);
-      const int32_t* k32 = reinterpret_cast<const int32_t*>(tb->col[acol[a]]) + r_begin;
-      const int64_t* k64 = reinterpret_cast<const int64_t*>(tb->col[acol[a]]) + r_begin;
-      const uint32_t n = uint32_t(r_end - r_begin);  // a chunk is at most 64 tiles
-      int64_t mn = INT64_MAX, mx = INT64_MIN;
-      bool ok = true;
-      if (i32 && small) {
-        int32_t mn32 = INT32_MAX, mx32 = INT32_MIN;
-        ok = presence ? count_rows<int32_t, true, true>(cc, k32, n, &mn32, &mx32)
-                      : count_rows<int32_t, true, false>(cc, k32, n, &mn32, &mx32);
-        if (mx32 >= mn32) mn = mn32, mx = mx32;  // (else: no key seen)
-      } else if (!i32) {
-        ok = presence ? count_rows<int64_t, false, true>(cc, k64, n, &mn, &mx)
-                      : count_rows<int64_t, false, false>(cc, k64, n, &mn, &mx);
-      } else {  // int32 keys with a domain beyond int32: one by one (declared)
-        for (uint32_t r = tid; r < n; r += T) {
-          const uint64_t off = uint64_t(int64_t(__ldg(k32 + r))) - cc.base;
-          if (off > cc.last) ok = false;
-          else if (presence) red_or(reinterpret_cast<uint32_t*>(cc.cnt) + (off >> 5), 1u << (off & 31));
-          else red_add(cc.cnt + off, 1);
+      if (tid == 0 && r_end > r_begin)
+        atomicAdd(reinterpret_cast<unsigned long long*>(tb->survivors), (unsigned long long)(r_end - r_begin));
+      for (int a = 0; a < nac; a++) {
+        const AggCol& ac = agg_of(a);
+        const CntCol cc = cnt_col(a);
+        const bool i32 = tb->dtype[acol[a]] == CMP_I32, presence = ac.kind == kAggPresence;
+        // the slots of an int32 column are 32-bit sums when its domain lies in int32
+        const bool small = !cc.declared || (ac.base >= INT32_MIN && ac.base + ac.cap <= int64_t(INT32_MAX) + 1);
+        const int32_t* k32 = reinterpret_cast<const int32_t*>(tb->col[acol[a]]) + r_begin;
+        const int64_t* k64 = reinterpret_cast<const int64_t*>(tb->col[acol[a]]) + r_begin;
+        const uint32_t n = uint32_t(r_end - r_begin);  // a chunk is at most 64 tiles
+        int64_t mn = INT64_MAX, mx = INT64_MIN;
+        bool ok = true;
+        if (i32 && small) {
+          int32_t mn32 = INT32_MAX, mx32 = INT32_MIN;
+          ok = presence ? count_rows<int32_t, true, true>(cc, k32, n, &mn32, &mx32)
+                        : count_rows<int32_t, true, false>(cc, k32, n, &mn32, &mx32);
+          if (mx32 >= mn32) mn = mn32, mx = mx32;  // (else: no key seen)
+        } else if (!i32) {
+          ok = presence ? count_rows<int64_t, false, true>(cc, k64, n, &mn, &mx)
+                        : count_rows<int64_t, false, false>(cc, k64, n, &mn, &mx);
+        } else {  // int32 keys with a domain beyond int32: one by one (declared)
+          for (uint32_t r = tid; r < n; r += T) {
+            const uint64_t off = uint64_t(int64_t(__ldg(k32 + r))) - cc.base;
+            if (off > cc.last) ok = false;
+            else if (presence) red_or(reinterpret_cast<uint32_t*>(cc.cnt) + (off >> 5), 1u << (off & 31));
+            else red_add(cc.cnt + off, 1);
+          }
         }
+        fold_range(a, cc, ok, mn, mx);
       }
-      fold_range(a, cc, ok, mn, mx);
-    }
     }
     c = c_next;
   }

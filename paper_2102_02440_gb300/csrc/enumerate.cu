@@ -21,7 +21,8 @@
 // completed a plan (all of it: its warp lowered the best cost for itself).  What came after
 // that piece is discarded and searched again under the new best cost.  The counters, the
 // costs and the plan are those of the sequential search; a round that would exceed the
-// search budget is discarded and the sequential search goes on alone.
+// search budget is discarded and the sequential search goes on alone, to the end, as it does
+// when a paused search has more than kEnumItems unvisited prefixes.
 //
 // A batch of more graphs than there are SMs takes two launches.  A CTA of 16 warps of 118
 // registers has an SM to itself, and most searches of a large batch are short: so the first launch
@@ -390,7 +391,8 @@ enum { kCmdExit = 0, kCmdRound = 1 };
 template <bool FIRST>
 __global__ void __launch_bounds__(FIRST ? 32 : 32 * kEnumMaxWarps) k_enumerate(const __grid_constant__ EnumArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
-  EnumSaved* const saved = A.saved ? reinterpret_cast<EnumSaved*>(A.saved + enum_saved_bytes(A.n_max) * blockIdx.x) : nullptr;
+  EnumSaved* const saved =
+      A.saved ? reinterpret_cast<EnumSaved*>(A.saved + enum_saved_bytes(A.n_max) * blockIdx.x) : nullptr;
   if (!FIRST && saved && !saved->open) return;  // the first launch has ended it
   const EnumGraph& g = A.graphs[blockIdx.x];
   const int n = g.n, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = A.warps;
@@ -437,9 +439,10 @@ __global__ void __launch_bounds__(FIRST ? 32 : 32 * kEnumMaxWarps) k_enumerate(c
     if (v1 < n) src[r1] = v1;
   }
   const int frame_words = enum_frame(A.n_max).bytes / 16;
-  uint4* const saved_frame = saved ? reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(saved) + align16(sizeof(EnumSaved))) : nullptr;
+  uint4* const frame0 = reinterpret_cast<uint4*>(smem + L.frame);
+  uint4* const saved_frame = saved ? reinterpret_cast<uint4*>(saved) + align16(sizeof(EnumSaved)) / 16 : nullptr;
   if (!FIRST && saved)  // warp 0 goes on from the frames of the first launch
-    for (int i = threadIdx.x; i < frame_words; i += blockDim.x) reinterpret_cast<uint4*>(smem + L.frame)[i] = saved_frame[i];
+    for (int i = threadIdx.x; i < frame_words; i += blockDim.x) frame0[i] = saved_frame[i];
   __syncthreads();
   EnumWarp S(A, g, smem + L.frame + size_t(enum_frame(A.n_max).bytes) * warp, tmask, tval, staged);
 
@@ -507,7 +510,7 @@ __global__ void __launch_bounds__(FIRST ? 32 : 32 * kEnumMaxWarps) k_enumerate(c
     open &= !out_of_budget;
     if (open) {
       S.save();
-      for (int i = lane; i < frame_words; i += 32) saved_frame[i] = reinterpret_cast<const uint4*>(smem + L.frame)[i];
+      for (int i = lane; i < frame_words; i += 32) saved_frame[i] = frame0[i];
     }
     if (lane == 0) *saved = {min_cost, plans, nodes, pruned, p, quiet, si, S.d, open, have, S.missing};
     missing = S.missing;
@@ -997,7 +1000,8 @@ cmp_status cmp_enumerate(const void* plan_host, const void* plan_dev, const doub
     a.first_nodes = std::max(kEnumFirstLeast, kEnumFirstNodes * H.n_graphs / kEnumBatch);
     a.warps = 1;
     const size_t base = size_t(enum_smem(H.n_max, 1, true).table);
-    a.stage_slots = int32_t(std::min<size_t>(size_t(H.stage_slots), base < kEnumFirstSmem ? (kEnumFirstSmem - base) / 16 : 0));
+    const size_t room = base < kEnumFirstSmem ? (kEnumFirstSmem - base) / 16 : 0;
+    a.stage_slots = int32_t(std::min<size_t>(size_t(H.stage_slots), room));
     static SmemLimit limit;
     if (limit.allow(k_enumerate<true>) != cudaSuccess) return CMP_ECUDA;
     k_enumerate<true><<<unsigned(H.n_graphs), 32, base + 16 * size_t(a.stage_slots), st>>>(a);

@@ -25,7 +25,10 @@
 // Before: one contraction per conditioning value, a block scan per table each, and once more
 // per prime for the rows beyond int128.  The cycles of 4, 5, 15 and 17 tables of a batch at
 // w = 1024, d = 11: 74 ms of estimate kernels before, 1.4 ms now (0.85 here).
-// A row whose L does not fit keeps the generic path (k_estimate_items), decided on the device.
+// A row whose L does not fit keeps the generic path (k_estimate_items), decided on the device;
+// so does, in the plan, a cycle with w > kCycMaxW or with fewer conditioning chunks than
+// kCycRowItems (a row's state is kept in their partial sums): w <= 7 cond_chunk, which is w <= 448
+// at the default of 64 values.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -92,143 +92,143 @@ __device__ __forceinline__ void star_unit_int128(const EstArgs& A, const StarUni
   float* Am = Bm + R * NB;                                         // [R][16]
   const int tid = threadIdx.x;
   const int w = A.w, d = A.d;
-      const StarFam F = A.star[u.fam];
-      const int K = F.K, k = K - 1, k1 = F.k1, k2 = F.k2, m1 = F.m1;
-      const int NV2 = 1 << k2, E = 1 << (m1 + k2);
-      const int Ep = E < kStarThreads ? E : kStarThreads;
-      const int L = kStarThreads / Ep, J = E / Ep;
-      const int es = tid % Ep, lane = tid / Ep;
-      const int64_t ro = int64_t(u.row) * w;
-      const EstIn xa = A.inputs[F.in_begin + u.a];
-      const int64_t* suf0 = A.star_suf + F.suf_off + int64_t(u.row) * K * (int64_t(w) + 1);
-      i128 acc[16];
-      uint32_t accf = 0;
+  const StarFam F = A.star[u.fam];
+  const int K = F.K, k = K - 1, k1 = F.k1, k2 = F.k2, m1 = F.m1;
+  const int NV2 = 1 << k2, E = 1 << (m1 + k2);
+  const int Ep = E < kStarThreads ? E : kStarThreads;
+  const int L = kStarThreads / Ep, J = E / Ep;
+  const int es = tid % Ep, lane = tid / Ep;
+  const int64_t ro = int64_t(u.row) * w;
+  const EstIn xa = A.inputs[F.in_begin + u.a];
+  const int64_t* suf0 = A.star_suf + F.suf_off + int64_t(u.row) * K * (int64_t(w) + 1);
+  i128 acc[16];
+  uint32_t accf = 0;
 #pragma unroll
-      for (int j = 0; j < 16; j++) acc[j] = 0;
+  for (int j = 0; j < 16; j++) acc[j] = 0;
 
-      for (int r0 = 0; r0 < w; r0 += R) {
-        // 1. the chunk's factors f[j][r] (position j of U \ {a}) and w[r]
-        for (int q = tid; q < (k + 1) * R; q += kStarThreads) {
-          const int j = q / R, rr = q % R, r = r0 + rr;
-          if (j < k) {
-            int64_t f = 0;
-            if (r < w) {
-              const int ub = j < u.a ? j : j + 1;
-              const EstIn& xb = A.inputs[F.in_begin + ub];
-              const int32_t pos = __ldg(star_rank_row(xa, xb, d, u.row, w) + r);
-              f = suf0[int64_t(ub) * (w + 1) + pos];
-            }
-            fv[j * R + rr] = f;
-          } else {
-            int64_t wr = 0;
-            if (r < w) {
-              const int32_t jj = __ldg(xa.perm + ro + r);
-              wr = int64_t(__ldg(xa.s + ro + jj)) * int64_t(__ldg(xa.msk + ro + jj));  // |int32 int32| < 2^62
-            }
-            wv[rr] = wr;
-          }
+  for (int r0 = 0; r0 < w; r0 += R) {
+    // 1. the chunk's factors f[j][r] (position j of U \ {a}) and w[r]
+    for (int q = tid; q < (k + 1) * R; q += kStarThreads) {
+      const int j = q / R, rr = q % R, r = r0 + rr;
+      if (j < k) {
+        int64_t f = 0;
+        if (r < w) {
+          const int ub = j < u.a ? j : j + 1;
+          const EstIn& xb = A.inputs[F.in_begin + ub];
+          const int32_t pos = __ldg(star_rank_row(xa, xb, d, u.row, w) + r);
+          f = suf0[int64_t(ub) * (w + 1) + pos];
         }
-        __syncthreads();
-        // 2. table roots: B[r][0] = 1, A[r][0] = w(r) times the factors of blk's bits
-        for (int rr = tid; rr < R; rr += kStarThreads) {
-          Bs[rr * NB] = 1;
-          Bf[rr * NB] = 0;
-          Bm[rr * NB] = 1.0f;
-          i128 v = i128(wv[rr]);
-          bool fl = false;
-          for (int i = 0; i < k1 - m1; i++)
-            if ((u.blk >> i) & 1) star_step(v, fl, fv[(m1 + i) * R + rr]);
-          As[rr * 16] = v;
-          Af[rr * 16] = fl;
-          Am[rr * 16] = star_mag(v, fl);
+        fv[j * R + rr] = f;
+      } else {
+        int64_t wr = 0;
+        if (r < w) {
+          const int32_t jj = __ldg(xa.perm + ro + r);
+          wr = int64_t(__ldg(xa.s + ro + jj)) * int64_t(__ldg(xa.msk + ro + jj));  // |int32 int32| < 2^62
         }
-        __syncthreads();
-        // 3. doubling: entries [h, 2h) from [0, h) times the factor of bit jj
-        const int steps = k2 > m1 ? k2 : m1;
-        for (int jj = 0; jj < steps; jj++) {
-          const int h = 1 << jj;
-          if (jj < k2)
-            for (int q = tid; q < h * R; q += kStarThreads) {
-              const int rr = q / h, idx = h + q % h;
-              i128 v = Bs[rr * NB + idx - h];
-              bool fl = Bf[rr * NB + idx - h];
-              star_step(v, fl, fv[(k1 + jj) * R + rr]);
-              Bs[rr * NB + idx] = v;
-              Bf[rr * NB + idx] = fl;
-              Bm[rr * NB + idx] = star_mag(v, fl);
-            }
-          if (jj < m1)
-            for (int q = tid; q < h * R; q += kStarThreads) {
-              const int rr = q / h, idx = h + q % h;
-              i128 v = As[rr * 16 + idx - h];
-              bool fl = Af[rr * 16 + idx - h];
-              star_step(v, fl, fv[jj * R + rr]);
-              As[rr * 16 + idx] = v;
-              Af[rr * 16 + idx] = fl;
-              Am[rr * 16 + idx] = star_mag(v, fl);
-            }
-          __syncthreads();
+        wv[rr] = wr;
+      }
+    }
+    __syncthreads();
+    // 2. table roots: B[r][0] = 1, A[r][0] = w(r) times the factors of blk's bits
+    for (int rr = tid; rr < R; rr += kStarThreads) {
+      Bs[rr * NB] = 1;
+      Bf[rr * NB] = 0;
+      Bm[rr * NB] = 1.0f;
+      i128 v = i128(wv[rr]);
+      bool fl = false;
+      for (int i = 0; i < k1 - m1; i++)
+        if ((u.blk >> i) & 1) star_step(v, fl, fv[(m1 + i) * R + rr]);
+      As[rr * 16] = v;
+      Af[rr * 16] = fl;
+      Am[rr * 16] = star_mag(v, fl);
+    }
+    __syncthreads();
+    // 3. doubling: entries [h, 2h) from [0, h) times the factor of bit jj
+    const int steps = k2 > m1 ? k2 : m1;
+    for (int jj = 0; jj < steps; jj++) {
+      const int h = 1 << jj;
+      if (jj < k2)
+        for (int q = tid; q < h * R; q += kStarThreads) {
+          const int rr = q / h, idx = h + q % h;
+          i128 v = Bs[rr * NB + idx - h];
+          bool fl = Bf[rr * NB + idx - h];
+          star_step(v, fl, fv[(k1 + jj) * R + rr]);
+          Bs[rr * NB + idx] = v;
+          Bf[rr * NB + idx] = fl;
+          Bm[rr * NB + idx] = star_mag(v, fl);
         }
-        // 4. multiply-add over the chunk's positions.  When the magnitude bounds keep the product
-        //    below 2^126 (float rounding stays far from 2^127), the product modulo 2^128 is exact.
+      if (jj < m1)
+        for (int q = tid; q < h * R; q += kStarThreads) {
+          const int rr = q / h, idx = h + q % h;
+          i128 v = As[rr * 16 + idx - h];
+          bool fl = Af[rr * 16 + idx - h];
+          star_step(v, fl, fv[jj * R + rr]);
+          As[rr * 16 + idx] = v;
+          Af[rr * 16 + idx] = fl;
+          Am[rr * 16 + idx] = star_mag(v, fl);
+        }
+      __syncthreads();
+    }
+    // 4. multiply-add over the chunk's positions.  When the magnitude bounds keep the product
+    //    below 2^126 (float rounding stays far from 2^127), the product modulo 2^128 is exact.
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-          if (j >= J) break;
-          const int e = es + Ep * j;
-          const int v1 = e >> k2, v2 = e & (NV2 - 1);
-          i128 s = acc[j];
-          bool sf = (accf >> j) & 1u;
-          for (int rr = lane; rr < R; rr += L) {
-            const i128 a = As[rr * 16 + v1], b = Bs[rr * NB + v2];
-            if (Am[rr * 16 + v1] * Bm[rr * NB + v2] < 0x1p126f) {
-              sf |= add_ovf(s, i128(u128(a) * u128(b)), &s);
-              continue;
-            }
-            const bool fa = Af[rr * 16 + v1], fb = Bf[rr * NB + v2];
-            if ((!fa && a == 0) || (!fb && b == 0)) continue;  // an exact zero factor
-            if (fa || fb) {
-              sf = true;
-              continue;
-            }
-            i128 p;
-            sf |= mul_ovf(a, b, &p);
-            sf |= add_ovf(s, p, &s);
-          }
-          acc[j] = s;
-          accf = (accf & ~(1u << j)) | (uint32_t(sf) << j);
+    for (int j = 0; j < 16; j++) {
+      if (j >= J) break;
+      const int e = es + Ep * j;
+      const int v1 = e >> k2, v2 = e & (NV2 - 1);
+      i128 s = acc[j];
+      bool sf = (accf >> j) & 1u;
+      for (int rr = lane; rr < R; rr += L) {
+        const i128 a = As[rr * 16 + v1], b = Bs[rr * NB + v2];
+        if (Am[rr * 16 + v1] * Bm[rr * NB + v2] < 0x1p126f) {
+          sf |= add_ovf(s, i128(u128(a) * u128(b)), &s);
+          continue;
         }
-        __syncthreads();
-      }
-      // 5. lanes of one slot (L > 1 means J = 1): exact sum of their partial sums
-      if (L > 1) {
-        red[tid] = acc[0];
-        redf[tid] = uint8_t(accf & 1u);
-        __syncthreads();
-        if (lane == 0) {
-          i128 s = 0;
-          bool sf = false;
-          for (int l = 0; l < L; l++) {
-            const int t = es + Ep * l;
-            if (redf[t]) sf = true;
-            else sf |= add_ovf(s, red[t], &s);
-          }
-          acc[0] = s;
-          accf = sf ? 1u : 0u;
+        const bool fa = Af[rr * 16 + v1], fb = Bf[rr * NB + v2];
+        if ((!fa && a == 0) || (!fb && b == 0)) continue;  // an exact zero factor
+        if (fa || fb) {
+          sf = true;
+          continue;
         }
-        __syncthreads();
+        i128 p;
+        sf |= mul_ovf(a, b, &p);
+        sf |= add_ovf(s, p, &s);
       }
-      if (lane == 0) {
-        const int64_t base = F.t_off + ((int64_t(u.row) * K + u.a) << k);
+      acc[j] = s;
+      accf = (accf & ~(1u << j)) | (uint32_t(sf) << j);
+    }
+    __syncthreads();
+  }
+  // 5. lanes of one slot (L > 1 means J = 1): exact sum of their partial sums
+  if (L > 1) {
+    red[tid] = acc[0];
+    redf[tid] = uint8_t(accf & 1u);
+    __syncthreads();
+    if (lane == 0) {
+      i128 s = 0;
+      bool sf = false;
+      for (int l = 0; l < L; l++) {
+        const int t = es + Ep * l;
+        if (redf[t]) sf = true;
+        else sf |= add_ovf(s, red[t], &s);
+      }
+      acc[0] = s;
+      accf = sf ? 1u : 0u;
+    }
+    __syncthreads();
+  }
+  if (lane == 0) {
+    const int64_t base = F.t_off + ((int64_t(u.row) * K + u.a) << k);
 #pragma unroll
-        for (int j = 0; j < 16; j++) {
-          if (j >= J) break;
-          const int e = es + Ep * j;
-          const int v1 = e >> k2, v2 = e & (NV2 - 1);
-          const int64_t V = int64_t((u.blk << m1) | v1) | (int64_t(v2) << k1);
-          A.star_t[base + V] = acc[j];
-          A.star_tf[base + V] = uint8_t((accf >> j) & 1u);
-        }
-      }
+    for (int j = 0; j < 16; j++) {
+      if (j >= J) break;
+      const int e = es + Ep * j;
+      const int v1 = e >> k2, v2 = e & (NV2 - 1);
+      const int64_t V = int64_t((u.blk << m1) | v1) | (int64_t(v2) << k1);
+      A.star_t[base + V] = acc[j];
+      A.star_tf[base + V] = uint8_t((accf >> j) & 1u);
+    }
+  }
 }
 
 // ---------------------------------------------------------------- residues
@@ -353,8 +353,6 @@ __device__ __forceinline__ void star_unit_rns(const EstArgs& A, const StarUnit& 
   uint32_t* Y = X + 16 * nx;
   // position among the k factors of free bit i, of side bits and of the fixed bits
   auto free_pos = [&](int i) { return i < m1 ? i : k1 + i - m1; };
-  const int64_t ro = 0;
-  (void)ro;
   for (int q = tid; q < n_primes * E; q += kStarThreads) stash[q] = 0;
   __syncthreads();
   const int chunks = (w + kRnsR - 1) / kRnsR;
