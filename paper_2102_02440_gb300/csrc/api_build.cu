@@ -300,7 +300,7 @@ struct BuildPlanParts {
   int64_t cnt_split = 0;  // > 0: the tables with presence columns in a launch before the others
   int32_t d_cut = 1024;   // split pass: the dense kernel's share beside the last counting launch
   int64_t hash_items = 0;
-  int32_t hash_private = 0;
+  int32_t hash_private = 0, hash_few = 0;
   int32_t hash_grid = 0;
   std::vector<std::vector<int32_t>> col_agg;  // [table][col] AggCol index or -1
   size_t bytes = 0, ws_bytes = 0;
@@ -555,9 +555,11 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
       if (ac.kind != kAggPresence) total += double(ac.cap) * pairs_of(ac);
     const int64_t ctas = int64_t(sm_count()) * 2;
     const double per_item = std::max(1.0, total / double(ctas * items));
+    int64_t counters = 0;
     for (AggCol& ac : P->aggs) {
       ac.hash_item0 = P->hash_items;
       if (ac.kind == kAggPresence) continue;  // hashed by the dense kernel
+      counters += int64_t(pairs_of(ac)) * w;
       const int32_t np = pairs_of(ac), most = std::min(kHashMaxPairs, fit > 0 ? fit : kHashMaxPairs);
       ac.hash_slabs = (np + most - 1) / most;
       ac.hash_pairs = (np + ac.hash_slabs - 1) / ac.hash_slabs;
@@ -568,6 +570,7 @@ static cmp_status plan_layout(const cmp_table* tables, int32_t n_tables, int32_t
       if (fit > 0) P->hash_private = std::max(P->hash_private, ac.hash_pairs * w);
     }
     P->hash_grid = int32_t(std::min<int64_t>(P->hash_items, ctas));
+    P->hash_few = fit > 0 && counters <= kHashFewCounters ? 1 : 0;
   }
   // dense kernel: slabs of each presence column's pairs (as for the unique-key kernel);
   // each slab's domain split into items of whole runs, about equal work (keys x pairs) per
@@ -869,6 +872,7 @@ extern "C" cmp_status cmp_build_plan_encode(const cmp_table* tables, int32_t n_t
   h.cnt_sampled = P.cnt_sampled;
   h.cnt_filtered = P.cnt_filtered;
   h.hash_private = P.hash_private;
+  h.hash_few = P.hash_few;
   h.d_cut = P.d_cut;
   h.cnt_threads = 512;
   h.cnt_cache_slots = P.cache_slots;
@@ -949,6 +953,7 @@ extern "C" cmp_status cmp_sketch_build_batched(const void* plan_host, const void
     a.cnt_total_chunks = h.cnt_total_chunks;
     a.hash_items = h.hash_items;
     a.hash_private = h.hash_private;
+    a.hash_few = h.hash_few;
     a.cnt_cache_slots = h.cnt_cache_slots;
     a.cnt_cache_cols = h.cnt_cache_cols;
     // the (max, min) key ranges start from zero (decoding as an empty column), so do the

@@ -757,7 +757,7 @@ constexpr size_t kHashBufBytes = size_t(kHashThreads / 32) * kHashBuf * sizeof(u
 // The first n <= 32 E entries (offset j, count) of a warp's buffer, lane l taking l, l + 32, ...:
 // E independent chains per lane.  Keys are kmin + j, all of form F.  cs: the slab's counters in
 // shared memory (a shared address; PRIV), else rows grow[p] in global memory.  Lanes past n add 0.
-template <bool POW2, bool PRIV, int F, int E>
+template <bool POW2, bool PRIV, bool FEW, int F, int E>
 __device__ __forceinline__ void hash_batch(const PairParam* prm, int32_t* const* grow, uint32_t cs, int np, uint32_t w,
                                            int64_t kmin, const uint2* buf, int n) {
   constexpr bool SMALL = F != kAnyKey;
@@ -774,7 +774,13 @@ __device__ __forceinline__ void hash_batch(const PairParam* prm, int32_t* const*
     if (SMALL) x[e] = uint32_t(kmin) + off;
     else k[SMALL ? 0 : e] = key_powers(key_field(kmin + int64_t(off)));
   }
-  for (int p = 0; p < np; p++, cs += 4 * w) {
+  // Few rows, in global memory: each warp begins at another pair, so that the reductions of a
+  // moment do not all fall on one row (1 M keys, w = 1024, 5 pairs: 108 us in order, 91 like this).
+  constexpr bool ROT = FEW && !PRIV;
+  int next = ROT ? int((threadIdx.x >> 5) + blockIdx.x) % np : 0;
+  for (int t = 0; t < np; t++, cs += 4 * w) {
+    const int p = ROT ? next : t;
+    if (ROT) next = p + 1 < np ? p + 1 : 0;
     const PairParam q = prm[p];
     int32_t* row = PRIV ? nullptr : grow[p];
 #pragma unroll
@@ -788,7 +794,8 @@ __device__ __forceinline__ void hash_batch(const PairParam* prm, int32_t* const*
   }
 }
 
-template <bool POW2>
+// FEW: a plan of few counters (kHashFewCounters).
+template <bool POW2, bool FEW>
 __global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_constant__ BuildArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
   // the presence-bitmap kernel, launched next as a programmatic dependent, reads nothing
@@ -818,14 +825,14 @@ __global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_const
     auto run = [&](auto pv) {
       constexpr bool PRIV = decltype(pv)::value;
       if (kend <= (1ll << 29)) {
-        if (n > 64) hash_batch<POW2, PRIV, kSmall29, 4>(prm, grow, cs32, np, w, k0, buf, n);
-        else hash_batch<POW2, PRIV, kSmall29, 2>(prm, grow, cs32, np, w, k0, buf, n);
+        if (n > 64) hash_batch<POW2, PRIV, FEW, kSmall29, 4>(prm, grow, cs32, np, w, k0, buf, n);
+        else hash_batch<POW2, PRIV, FEW, kSmall29, 2>(prm, grow, cs32, np, w, k0, buf, n);
       } else {  // (the powers of two keys fit the registers)
         for (int i = 0; i < n; i += 64) {
           if (kend <= (1ll << 31))
-            hash_batch<POW2, PRIV, kSmall31, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
+            hash_batch<POW2, PRIV, FEW, kSmall31, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
           else
-            hash_batch<POW2, PRIV, kAnyKey, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
+            hash_batch<POW2, PRIV, FEW, kAnyKey, 2>(prm, grow, cs32, np, w, k0, buf + i, min(64, n - i));
         }
       }
     };
@@ -898,7 +905,16 @@ __global__ void __launch_bounds__(kHashThreads, 2) k_agg_hash(const __grid_const
       // Writing a slab's counters out costs about two updates for each, so private ones want
       // twice as many entries as buckets in an item (at most as many as survivors).
       groups = int(max(int64_t(1), min(int64_t(ac.hash_groups), range * ac.hash_pairs / item_work)));
-      priv = A.hash_private > 0 && min(range, int64_t(*tb->survivors)) / groups >= 2 * int64_t(w);
+      const int64_t survivors = int64_t(*tb->survivors), entries = min(range, survivors);
+      if constexpr (FEW) {
+        if (range >= kHashFewRange && entries < 2 * int64_t(w) * groups &&
+            (ac.hash_slabs == 1 || (ac.hash_slabs <= 3 && survivors >= 2 * range))) {
+          // fewer items, down to one a CTA, if a quarter of the CTAs get enough for theirs
+          const int64_t ctas = max(int64_t(1), range * ac.hash_pairs / item_work / kHashItems);
+          if (entries >= int64_t(w) * ctas) groups = int(max(int64_t(1), min(entries / (2 * int64_t(w)), ctas)));
+        }
+      }
+      priv = A.hash_private > 0 && entries / groups >= 2 * int64_t(w);
       if (!priv) {  // all pairs at once (as far as they fit), shorter items
         const bool one = np_col <= kHashMaxPairs;
         const int64_t most = one ? int64_t(ac.hash_groups) * ac.hash_slabs : ac.hash_groups;
@@ -978,9 +994,11 @@ cudaError_t launch_agg_hash(const BuildArgs& a, int32_t grid, cudaStream_t st) {
   if (a.n_agg <= 0 || grid <= 0) return cudaSuccess;
   const bool pow2 = (a.w & (a.w - 1)) == 0;
   const size_t smem = kHashBufBytes + sizeof(int32_t) * size_t(a.hash_private);
-  auto k = pow2 ? k_agg_hash<true> : k_agg_hash<false>;
-  static SmemLimit limit[2];
-  cudaError_t e = limit[pow2].allow(k);
+  const bool few = a.hash_few != 0;
+  auto k = few ? (pow2 ? k_agg_hash<true, true> : k_agg_hash<false, true>)
+               : (pow2 ? k_agg_hash<true, false> : k_agg_hash<false, false>);
+  static SmemLimit limit[4];
+  cudaError_t e = limit[2 * few + pow2].allow(k);
   if (e != cudaSuccess) return e;
   k<<<unsigned(grid), kHashThreads, smem, st>>>(a);
   return cudaGetLastError();

@@ -325,6 +325,15 @@ constexpr int kHashThreads = 512, kHashMaxPairs = 64;
 constexpr int64_t kHashStep = 128;
 constexpr int64_t kHashBudget = 76 << 10;      // two CTAs per SM
 constexpr int64_t kHashItems = 6, kHashDirectItems = 48;
+// Where that many items are too short for private counters, updates of few counters in global
+// memory get in each other's way (3 M keys of a domain of 1 M, w = 1024, 5 pairs: 185 us), and
+// fewer items with private ones pay (34 us): in plans of at most kHashFewCounters counters of
+// counted columns (12 columns of 300,000 skewed keys, 61,000 counters: 55 us shared, 66 private)
+// and for a key range of at least kHashFewRange (100,000 keys are too few for the CTAs: 10 us
+// shared, 21 private).  Several slabs read the slots as often, so they also want two
+// survivors for each (3 M keys, w = 4096, 5 pairs: 70 and 38 us; 1 M skewed ones 16 and 21).  The
+// kernel of such plans is one of its own: the rule's registers cost the others 0.5%.
+constexpr int64_t kHashFewCounters = 48 << 10, kHashFewRange = 1 << 18;
 // Presence bitmaps are walked in runs of kDenseRun keys (8 words); a bitmap holds whole runs.
 constexpr int64_t kDenseRun = 256;
 __host__ __device__ inline int64_t presence_words(int64_t cap) { return (cap + kDenseRun - 1) / kDenseRun * (kDenseRun / 32); }
@@ -444,6 +453,7 @@ struct BuildArgs {
   int64_t cnt_total_chunks;
   int64_t hash_items;   // hashing pass of the aggregated columns: its items,
   int32_t hash_private;  // words of the CTA's own counters (0: counters in global memory)
+  int32_t hash_few;      // 1: at most kHashFewCounters counters
   // unique-key kernel
   const UniqSlab* uslab;
   const UniqItem* uitem;
@@ -486,7 +496,7 @@ struct BuildPlanHdr {
   int64_t cnt_split;
   // split pass: the dense kernel walks the first d_cut / 1024 of each item's runs beside the
   // last counting launch, the rest after it with 512 threads (d_cut = 1024: all beside)
-  int32_t d_cut, pad;
+  int32_t d_cut, hash_few;  // (hash_few: of the hashing pass)
   // chunks: tables with presence columns and without a selection, from cnt_sampled on tables with a
   // row sample only (k_count_rows), from cnt_filtered on tables with predicates (k_agg_count)
   int64_t cnt_sampled;
