@@ -167,8 +167,8 @@ __global__ void __launch_bounds__(1024) k_sketch_build(const __grid_constant__ B
         const PairLimb l = pair_limbs(q);
         h0 = cw_bucket<POW2>(q, l, k0, uint32_t(w));
         h1 = cw_bucket<POW2>(q, l, k1, uint32_t(w));
-        v0 = cw_sign(q, l, k0) * m0;
-        v1 = cw_sign(q, l, k1) * m1;
+        v0 = cw_odd(q, l, k0) ? -m0 : m0;
+        v1 = cw_odd(q, l, k1) ? -m1 : m1;
       }
       int32_t* row = (GLOBAL ? gcnt : cnt) + size_t(pp) * w;  // L2 counters, or the CTA's shared ones
       if (GLOBAL) {
@@ -786,7 +786,7 @@ __device__ __forceinline__ void hash_batch(const PairParam* prm, int32_t* const*
 #pragma unroll
     for (int e = 0; e < E; e++) {
       const uint32_t h = SMALL ? sx_bucket<POW2, F>(q, x[e], w) : cw_bucket<POW2>(q, pair_limbs(q), k[SMALL ? 0 : e], w);
-      const uint32_t odd = SMALL ? sx_odd<F>(q, x[e]) : uint32_t(cw_sign_residue(q, pair_limbs(q), k[SMALL ? 0 : e])) & 1u;
+      const uint32_t odd = SMALL ? sx_odd<F>(q, x[e]) : cw_odd(q, pair_limbs(q), k[SMALL ? 0 : e]);
       const uint32_t v = odd * (0u - 2u * uint32_t(m[e])) + uint32_t(m[e]);  // one multiply-add
       if (PRIV) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(cs + 4 * h), "r"(v) : "memory");
       else if (m[e]) red_add(row + h, int32_t(v));

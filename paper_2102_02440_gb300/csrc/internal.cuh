@@ -162,35 +162,51 @@ __device__ __forceinline__ KeyPow key_powers(uint64_t x) {
 
 // Bucket: ((a x + b) mod p) mod w.  Sum bound: t0 + (t1>>30) + ((t1&M30)<<31) + 2 t2 + b
 // < 2^62 + 2^32 + 3 * 2^61 < 2^64.
-__device__ __forceinline__ uint64_t cw_bucket_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+// The folded sums y are below 2^61 + 8 and congruent to the residue, which is y - p where y >= p;
+// modulo a power of two that divides 2^61, and for the parity (p is odd), that is a bit
+// added to y.  (Coefficients are split into limbs at each use, for the small-key steps take them
+// whole.  2 M rows of keys near 2^45 in 64 x 64 partitions: 473 us with limbs stored, 494 split
+// at each use with the residue formed, 486 like this.)
+__device__ __forceinline__ uint32_t ge_p(uint64_t y) { return uint32_t((y + 1) >> 61); }  // 1 if y >= p, else 0
+__device__ __forceinline__ uint64_t cw_bucket_fold(const PairParam& q, const PairLimb& l, const KeyPow& k) {
   const Limb a = l.a;
   const uint64_t t0 = uint64_t(a.lo) * k.x.lo;
   const uint64_t t1 = uint64_t(a.lo) * k.x.hi + uint64_t(a.hi) * k.x.lo;
   const uint64_t t2 = uint64_t(a.hi) * k.x.hi;
   const uint64_t s = t0 + (t1 >> 30) + ((t1 & kM30) << 31) + 2 * t2 + q.b;
-  return canon61(fold61(s));
+  return fold61(s);
+}
+__device__ __forceinline__ uint64_t cw_bucket_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+  return canon61(cw_bucket_fold(q, l, k));
 }
 template <bool POW2>
 __device__ __forceinline__ uint32_t cw_bucket(const PairParam& q, const PairLimb& l, const KeyPow& k, uint32_t w) {
-  const uint64_t r = cw_bucket_residue(q, l, k);
-  if (POW2) return uint32_t(r) & (w - 1);
-  return uint32_t(r % w);
+  const uint64_t y = cw_bucket_fold(q, l, k);
+  if (POW2) return (uint32_t(y) + ge_p(y)) & (w - 1);
+  return uint32_t(canon61(y) % w);
 }
 
 // Sign: parity of (c3 x^3 + c2 x^2 + c1 x + c0) mod p, as +1 / -1.  The three products
 // are summed by limb position: S0 < 3 * 2^62, S1 < 6 * 2^61, S2 < 3 * 2^60, and
 // fold(S0) + (S1>>30) + ((S1&M30)<<31) + 2 S2 + c0 < 6 * 2^61 + 2^35 < 2^64.
-__device__ __forceinline__ uint64_t cw_sign_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+__device__ __forceinline__ uint64_t cw_sign_fold(const PairParam& q, const PairLimb& l, const KeyPow& k) {
   const Limb c1 = l.c1, c2 = l.c2, c3 = l.c3;
   const uint64_t S0 = uint64_t(c1.lo) * k.x.lo + uint64_t(c2.lo) * k.x2.lo + uint64_t(c3.lo) * k.x3.lo;
   const uint64_t S1 = uint64_t(c1.lo) * k.x.hi + uint64_t(c1.hi) * k.x.lo + uint64_t(c2.lo) * k.x2.hi +
                       uint64_t(c2.hi) * k.x2.lo + uint64_t(c3.lo) * k.x3.hi + uint64_t(c3.hi) * k.x3.lo;
   const uint64_t S2 = uint64_t(c1.hi) * k.x.hi + uint64_t(c2.hi) * k.x2.hi + uint64_t(c3.hi) * k.x3.hi;
   const uint64_t v = fold61(S0) + (S1 >> 30) + ((S1 & kM30) << 31) + 2 * S2 + q.c0;
-  return canon61(fold61(v));
+  return fold61(v);
+}
+__device__ __forceinline__ uint64_t cw_sign_residue(const PairParam& q, const PairLimb& l, const KeyPow& k) {
+  return canon61(cw_sign_fold(q, l, k));
+}
+__device__ __forceinline__ uint32_t cw_odd(const PairParam& q, const PairLimb& l, const KeyPow& k) {  // 1: the sign is -1
+  const uint64_t y = cw_sign_fold(q, l, k);
+  return (uint32_t(y) ^ ge_p(y)) & 1u;
 }
 __device__ __forceinline__ int cw_sign(const PairParam& q, const PairLimb& l, const KeyPow& k) {
-  return 1 - 2 * int(cw_sign_residue(q, l, k) & 1);
+  return 1 - 2 * int(cw_odd(q, l, k));
 }
 
 // ---- Horner form (one (sketch, row) pair per key: no powers to share).  The same two
@@ -214,9 +230,6 @@ __device__ __forceinline__ uint64_t mul_add_fold(Limb l, const KeyX& x, uint64_t
   const uint64_t s = uint64_t(l.lo) * x.lo + uint64_t(l.hi) * x.hi2 + c + (t1 >> 30) + ((t1 & kM30) << 31);
   return fold61(s);
 }
-
-// For y < 2^61 + 8: 1 if y >= p (its residue is then y - p), else 0.
-__device__ __forceinline__ uint32_t ge_p(uint64_t y) { return uint32_t((y + 1) >> 61); }
 
 // Bucket ((a x + b) mod p) mod w; the same value as cw_bucket.  For w a power of two (w <=
 // 2^31 divides 2^61), y - p = y + 1 (mod w).

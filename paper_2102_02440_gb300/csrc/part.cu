@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(1024) k_part_build(const __grid_constant__ Par
                   odd ^= sx_odd<F>(q, uint32_t(key[l]));
                 } else {
                   idx += cw_bucket<POW2>(q, pair_limbs(q), kp[l], A.width[l]) * A.stride[l];
-                  odd ^= uint32_t(cw_sign_residue(q, pair_limbs(q), kp[l])) & 1u;
+                  odd ^= cw_odd(q, pair_limbs(q), kp[l]);
                 }
               }
               atomicAdd(out + int64_t(i) * A.size + idx, 1 - 2 * int(odd));
