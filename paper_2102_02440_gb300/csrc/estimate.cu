@@ -223,13 +223,19 @@ cudaError_t launch_presort_large(const int32_t* C, int64_t n_rows, int32_t w, ui
 cudaError_t launch_presort(const int32_t* C, int64_t n_rows, int32_t w, uint32_t* abs_out, int32_t* perm_out,
                            cudaStream_t st) {
   if (n_rows <= 0) return cudaSuccess;
-  int n = 256;  // keys of a CTA: eight a thread, sixteen beyond 8192
+  // keys of a CTA: eight a thread, sixteen beyond 8192, one to four below 256 (7000 rows of 8, 32 and
+  // 64 keys: 20 us each as 256 keys; 7.7, 9.6 and 15 with every stage in shared memory; 8.0, 8.0
+  // and 8.5 now; 128 keys 29 and 12.6)
+  int n = 32;
   while (n < w) n <<= 1;
-  auto k = n > 8192 ? k_presort<16> : k_presort<8>;
-  const int threads = n > 8192 ? n / 16 : n / 8;
+  const int lg = n <= 32 ? 0 : n <= 64 ? 1 : n <= 128 ? 2 : n <= 8192 ? 3 : 4;
+  void (*const kernels[5])(const int32_t*, int64_t, int32_t, uint32_t*, int32_t*) = {
+      k_presort<1>, k_presort<2>, k_presort<4>, k_presort<8>, k_presort<16>};
+  auto k = kernels[lg];
+  const int threads = n >> lg;
   const size_t smem = sort_smem_bytes(n);
-  static SmemLimit limit[2];
-  cudaError_t e = limit[n > 8192].allow(k);
+  static SmemLimit limit[5];
+  cudaError_t e = limit[lg].allow(k);
   if (e != cudaSuccess) return e;
   const int64_t grid = n_rows < 4096 ? n_rows : 4096;
   k<<<unsigned(grid), threads, smem, st>>>(C, n_rows, w, abs_out, perm_out);
