@@ -474,10 +474,23 @@ __device__ __forceinline__ void star_unit_rns(const EstArgs& A, const StarUnit& 
   __syncthreads();
 }
 
+// The most primes with which a unit of 2^nf entries is faster on residues than in int128.  A prime
+// costs its chunks' tables and barriers whatever the entries, and a group's first chunk (w / (w +
+// 180): the width spread over the groups); int128 costs 52 instructions an entry and position.
+// 20 stars of 3, 5 and 6 leaves at w = 1024, d = 11 on 3, 5 and 5 primes: 371, 1064 and 1336 us,
+// in int128 346, 682 and 1237; of 5 leaves at w = 512 on 5 primes 612 and 347; one of 6 at w = 64
+// on 4 primes 56 and 16.
+__device__ __forceinline__ float rns_most(int nf, int w) {
+  const float wide =
+      nf <= 2 ? 3.4f : nf == 3 ? 4.2f : nf == 4 ? 4.05f : nf == 5 ? 4.8f : nf == 6 ? 5.5f : 3.0f * float(nf) - 11.5f;
+  return wide * float(w) / float(w + 180);
+}
+
 // Lattice units (family, row, a, blk), persistent over the unit list.  A unit computes
 // T_a(V) for the 2^m1 A-side subsets of block blk (bits m1..k1-1 of V1 = blk) and all 2^k2
 // B-side subsets.  Its sums are bounded by w max_r |w_a(r)| prod_b max(1, |f_ab(r)|): below
-// 2^138 it runs on residues, on as many primes as the bound asks for, else in int128.
+// 2^138 it runs on residues, on as many primes as the bound asks for, if that pays (rns_most),
+// else in int128.
 // Stars of 10, 14 and 15 tables (2.0 G multiply-adds at w = 1024, d = 11): 6.16 ms all in int128,
 // 2.53 to 2.82 ms on four and five residues.  The units are inlined: as functions of their own
 // they spilled, and stars beyond 2^138 (three of 10 to 13 tables, up to 8 M rows) took 9.03 ms,
@@ -528,8 +541,9 @@ __global__ void __launch_bounds__(kStarThreads, 2) k_star_lattice(const __grid_c
     for (int i = 0; i < kStarThreads / 32; i++) bits = fmaxf(bits, U.bits[i]);
     bits += float(32 - __clz(w - 1)) + 2.01f;  // w terms; |T| < P / 4
     const int n_primes = max(1, int(ceilf(bits / kRnsBits)));
-    const int nf = F.m1 + F.k2, tiles = max(1, (1 << ((nf + 1) / 2)) / 8) * max(1, (1 << (nf / 2)) / 4);
-    if (n_primes > kRnsMax) star_unit_int128(A, u, smem);
+    const int nf = F.m1 + F.k2;
+    const int tiles = max(1, (1 << ((nf + 1) / 2)) / 8) * max(1, (1 << (nf / 2)) / 4);
+    if (n_primes > kRnsMax || float(n_primes) > rns_most(nf, w)) star_unit_int128(A, u, smem);
     else if (tiles <= 32) star_unit_rns<32>(A, u, F, U, n_primes, smem);
     else if (tiles <= 64) star_unit_rns<64>(A, u, F, U, n_primes, smem);
     else star_unit_rns<128>(A, u, F, U, n_primes, smem);
