@@ -17,7 +17,7 @@
 //    any L with |E| < 2^(32 L - 1): values are L-limb two's complement integers, L chosen per
 //    row from the bound |E| <= prod_t sum_j min(|a_j|, max |p|) (the infinity norms).  Rows
 //    beyond int128 come out exact as well; the exact tier only turns them into residues.
-// Layout: a CTA of 256 threads holds C product vectors (columns) in shared memory, two
+// Layout: a CTA of 256 or 512 threads holds C product vectors (columns) in shared memory, two
 // buffers [w][C][L]; thread = (segment, column), the segments cutting the merged order of 2 w
 // steps evenly (merge path), so a segment's running sums start from a scan over the
 // segments.  The integers bound it (about 12 L + 20 instructions per merged pair and column),
@@ -208,7 +208,8 @@ template <> struct Limbs<10> {
   }
 };
 
-constexpr int kCycThreads = 256;
+constexpr int kCycThreads = 256;       // two CTAs per SM
+constexpr int kCycWideThreads = 512;   // one
 constexpr int kCycBlk = 16;     // sorted positions of the cut sketch per job
 constexpr int kCycMaxCols = 8;
 
@@ -218,8 +219,11 @@ __host__ __device__ inline size_t cyc_fixed_bytes(int w) { return align16(size_t
 __host__ __device__ inline size_t cyc_col_bytes(int w, int L) { return size_t(2) * size_t(w) * size_t(L) * 4; }
 // (5 KB of static shared memory beside it) Two CTAs per SM while a column of eight limbs fits
 // beside the sketches, else one.
+__host__ __device__ inline bool cyc_two_per_sm(int w) {
+  return cyc_fixed_bytes(w) + cyc_col_bytes(w, 8) <= size_t(104) * 1024;
+}
 __host__ __device__ inline size_t cyc_smem_bytes(int w) {
-  return cyc_fixed_bytes(w) + cyc_col_bytes(w, 8) <= size_t(104) * 1024 ? size_t(104) * 1024 : size_t(220) * 1024;
+  return cyc_two_per_sm(w) ? size_t(104) * 1024 : size_t(220) * 1024;
 }
 // Columns per CTA for L limbs: a power of two, 0 when not even one fits.
 __device__ __forceinline__ int cyc_cols(int w, int L) {
@@ -333,11 +337,11 @@ __device__ __forceinline__ void cyc_store(uint32_t* p, const uint32_t (&v)[L]) {
 
 // The product vectors of the values vals[0..n_val) of the cut sketch (C at a time), and the
 // trace's share of them added to the row's accumulators.
-template <int L>
+template <int L, int T>
 __device__ __noinline__ void cyc_run(const EstArgs& A, const CycSub& cs, int row, const CycRow& cr, CycRow* out,
                                      const int32_t* vals, int n_val, unsigned char* smem, uint32_t* tot) {
   const int w = A.w, C = cr.cols, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int T = kCycThreads, NW = T / 32;
+  constexpr int NW = T / 32;
   const int nseg = T / C, c = tid & (C - 1), seg = tid / C;
   const int64_t ro = int64_t(row) * w;
   uint32_t* X = reinterpret_cast<uint32_t*>(smem);
@@ -493,8 +497,14 @@ __device__ __noinline__ void cyc_run(const EstArgs& A, const CycSub& cs, int row
 
 // Persistent over jobs (cycle, row, block of kCycBlk sorted positions of the cut sketch): the
 // block's positions that are the first of their value.
-__global__ void __launch_bounds__(kCycThreads, 2) k_cycle(const __grid_constant__ EstArgs A) {
+// T threads: with one CTA per SM, twice as many keep its latencies covered (the sums' carry chains
+// and their shared-memory operands; five rows of four tables of w = 4096, all values distinct:
+// 12.5 ms with 256, 8.5 with 512, 9.7 on the generic path; eleven rows of five of w = 2048 10.2,
+// 8.0 and 7.7).
+template <int T>
+__global__ void __launch_bounds__(T, 512 / T) k_cycle(const __grid_constant__ EstArgs A) {
   extern __shared__ __align__(16) unsigned char smem[];
+  // [T / 32][columns][2][limbs] (512 threads: columns x limbs <= 19 by the shared memory there is)
   __shared__ __align__(16) uint32_t tot[(kCycThreads / 32) * kCycMaxCols * 2 * kCycMaxLimbs];
   __shared__ int32_t vals[kCycBlk];
   __shared__ int32_t n_val;
@@ -531,11 +541,11 @@ __global__ void __launch_bounds__(kCycThreads, 2) k_cycle(const __grid_constant_
     const int n = n_val;
     if (n > 0) {
       switch (cr.limbs) {
-        case 2: cyc_run<2>(A, cs, row, cr, out, vals, n, smem, tot); break;
-        case 4: cyc_run<4>(A, cs, row, cr, out, vals, n, smem, tot); break;
-        case 6: cyc_run<6>(A, cs, row, cr, out, vals, n, smem, tot); break;
-        case 8: cyc_run<8>(A, cs, row, cr, out, vals, n, smem, tot); break;
-        default: cyc_run<10>(A, cs, row, cr, out, vals, n, smem, tot); break;
+        case 2: cyc_run<2, T>(A, cs, row, cr, out, vals, n, smem, tot); break;
+        case 4: cyc_run<4, T>(A, cs, row, cr, out, vals, n, smem, tot); break;
+        case 6: cyc_run<6, T>(A, cs, row, cr, out, vals, n, smem, tot); break;
+        case 8: cyc_run<8, T>(A, cs, row, cr, out, vals, n, smem, tot); break;
+        default: cyc_run<10, T>(A, cs, row, cr, out, vals, n, smem, tot); break;
       }
     }
     __syncthreads();  // vals and the buffers are rewritten by the next job
@@ -548,12 +558,14 @@ __global__ void __launch_bounds__(kCycThreads, 2) k_cycle(const __grid_constant_
 cudaError_t launch_estimate_cycle(const EstArgs& a, cudaStream_t st) {
   if (a.n_cyc <= 0) return cudaSuccess;
   const size_t smem = cyc_smem_bytes(a.w);
-  static SmemLimit limit;
-  cudaError_t e = limit.allow(k_cycle);
+  const bool two = cyc_two_per_sm(a.w);
+  auto k = two ? k_cycle<kCycThreads> : k_cycle<kCycWideThreads>;
+  static SmemLimit limit[2];
+  cudaError_t e = limit[two].allow(k);
   if (e != cudaSuccess) return e;
   k_cycle_prep<<<unsigned(a.n_cyc * a.d), 1024, 0, st>>>(a);
   const int64_t jobs = a.n_cyc * a.d * ((a.w + kCycBlk - 1) / kCycBlk);
-  k_cycle<<<unsigned(std::min<int64_t>(jobs, int64_t(sm_count()) * 2)), kCycThreads, smem, st>>>(a);
+  k<<<unsigned(std::min<int64_t>(jobs, int64_t(sm_count()) * (two ? 2 : 1))), two ? kCycThreads : kCycWideThreads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
